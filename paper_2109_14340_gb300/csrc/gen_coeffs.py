@@ -282,7 +282,8 @@ def sos_tables(name, spec, qnorm_abs):
     TAU2 = 2 tau (1 + 4u), DC_i >= D~_i C_i, and K0 >= tau^2 (1 + 2u)
     sum_i D~_i C_i^2 + 24 2^-53 |||A|||_2 4.01 n (the double-precision
     evaluation of the printed form on the same shifted values) + 1e-30
-    (underflow)."""
+    (underflow).  KAPPA >= 1.001 sqrt(sum_i DC_i^2 / D_i) bounds the middle
+    sum by Cauchy-Schwarz: sum_i DC_i |y~_i| <= KAPPA sqrt(beta~)."""
     import numpy as np
     offs, L, D = ldl_factors(spec)
     n = len(offs)
@@ -307,6 +308,8 @@ def sos_tables(name, spec, qnorm_abs):
                ", ".join(float.hex(d) + "f" for d in DC) + "};")
     out.append("#define %s_TAU2 %sf" % (name, float.hex(f32_up(2 * tau * (1 + 4 * u)))))
     out.append("#define %s_K0 %sf" % (name, float.hex(f32_up(k0))))
+    kappa = 1.001 * sum(c * c / d for c, d in zip(DC, Df)) ** 0.5
+    out.append("#define %s_KAPPA %sf" % (name, float.hex(f32_up(kappa))))
     out.append("")
     return out
 

@@ -25,9 +25,9 @@ struct NvtxRange {
 };
 
 // Explicit instantiations live in teno_face8.cu / teno_face10.cu.
-cudaError_t launch_face8(int nd, int d, const FaceArgs &a, cudaStream_t s);
-cudaError_t launch_face10(int nd, int d, const FaceArgs &a, cudaStream_t s);
-cudaError_t launch_face12(int nd, int d, const FaceArgs &a, cudaStream_t s);
+cudaError_t launch_chunk8(int nd, const SweepArgs &a, cudaStream_t s);
+cudaError_t launch_chunk10(int nd, const SweepArgs &a, cudaStream_t s);
+cudaError_t launch_chunk12(int nd, const SweepArgs &a, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Small kernels
@@ -213,9 +213,12 @@ __global__ void dt_from_speeds_kernel(const double *amax, int ncopies, int nd, d
 // limiter's effective dt/dx per direction: dt/dx in 1D; (dt S) / A_d with
 // S = sum_d A_d/dx_d in several dimensions (each direction's one-sided
 // updates get the share A_d/dx_d / S of the update).
+// The block also zeroes the stage's counters (one per chunk of the sweeps).
 __global__ void prepare_kernel(Status *st, int nd, double dt_host, const double *dt_dev,
-                               double3 inv_dx, int limiter)
+                               double3 inv_dx, int limiter, unsigned *counters, int ncounters)
 {
+    for (int i = threadIdx.x; i < ncounters; i += blockDim.x) counters[i] = 0u;
+    if (threadIdx.x) return;
     const double dt = dt_dev ? *dt_dev : dt_host;
     st->dt = dt;
     if (!limiter) return;
@@ -232,7 +235,8 @@ __global__ void prepare_kernel(Status *st, int nd, double dt_host, const double 
 }
 
 // Scalar reconstruction of caller-provided stencils (teno_reconstruct): the
-// certified filter first when enabled, else / then the exact path.
+// certified filter first when enabled (its first test too where no decision
+// byte is asked for, as in the sweeps), else / then the exact path.
 template <int H>
 __global__ void recon_kernel(const double *v, int64_t count, double *out, uint8_t *flags, Consts K,
                              FastK FK, int fast)
@@ -240,14 +244,13 @@ __global__ void recon_kernel(const double *v, int64_t count, double *out, uint8_
     constexpr int W = 2 * H;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
          i += (int64_t)gridDim.x * blockDim.x) {
-        double vv[W], sh[W];
+        double vv[W];
 #pragma unroll
         for (int m = 0; m < W; m++) vv[m] = v[i * W + m];
-#pragma unroll
-        for (int m = 0; m < W; m++) sh[m] = vv[m] - vv[H - 1];
         uint8_t fl = 0;
         double r;
-        if (fast && fast_decide<H>(vv, sh, FK, fl, flags != nullptr)) r = decided_value<H>(vv, fl);
+        if (fast && !flags && quick_large<H>(vv, FK)) r = flux_large<H, H>(vv);
+        else if (fast && fast_decide<H>(vv, FK, fl, flags != nullptr)) r = decided_value<H>(vv, fl);
         else r = teno_recon<H>(vv, K, fl);
         out[i] = r;
         if (flags) flags[i] = fl;
@@ -271,8 +274,51 @@ static int64_t face_grid(const teno_params *p, int d)
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Tile shape of direction d, and its tiles.
+static int64_t shape_tiles(const teno_params *p, int d, int skip_last, DirArgs &D)
+{
+    // pencils of a tile lie side by side in x, in y for the x sweep
+    const int64_t fast = d == 0 ? p->n[1] : p->n[0];
+    tile_shape(D, p->n[d] + 1 - skip_last, fast, p->scheme / 2);
+    return D.line_tiles * D.groups * (ncells(p) / p->n[d] / fast);
+}
+
+// Tiles of an evaluation at most: with face n, which a sweep may leave out.
+static int64_t all_tiles(const teno_params *p)
+{
+    int64_t t = 0;
+    for (int d = 0; d < p->ndim; d++) {
+        DirArgs D;
+        const int64_t with = shape_tiles(p, d, 0, D), without = shape_tiles(p, d, 1, D);
+        t += with > without ? with : without;
+    }
+    return t;
+}
+
+// The sweeps' buffers: the evaluation's tiles in chunks of at most nt.
+struct SweepMem {
+    char *mem;
+    unsigned *counters;
+    int64_t nt, nchunks;
+    size_t bytes;
+};
+
+static SweepMem sweep_mem(const teno_params *p, char *mem, int64_t most)
+{
+    SweepMem m;
+    const int64_t all = all_tiles(p);
+    m.nt = all < most ? all : most;
+    m.nchunks = (all + m.nt - 1) / m.nt;
+    SweepBuf b;
+    const size_t c = sweep_align(sizeof(unsigned) * (size_t)m.nchunks);
+    m.counters = (unsigned *)mem;
+    m.mem = mem + c;
+    m.bytes = c + sweep_buf_layout(b, m.mem, m.nt, p->ndim, p->scheme, p->limiter != 0);
+    return m;
+}
+
 struct Layout {
-    size_t status, flux[3], stage, prims, total;
+    size_t status, flux[3], stage, prims, sweep, total;
 };
 
 static Layout layout(const teno_params *p)
@@ -290,6 +336,8 @@ static Layout layout(const teno_params *p)
     off += align256(sizeof(double) * (size_t)nc * ncells(p));
     L.prims = off;
     off += align256(sizeof(double) * (size_t)(p->ndim + 4) * ncells(p));
+    L.sweep = off;
+    off += sweep_mem(p, nullptr, kChunkTiles).bytes;
     L.total = off;
     return L;
 }
@@ -449,22 +497,24 @@ static cudaError_t profile_mark(int which, int slot, cudaStream_t s)
 // its output for the next stage, or nullptr.
 // full_ct = false: a recorded decision byte carries its C_T exponent only
 // where the exponent was needed to decide (the selection-only record).
+// sm: the sweeps' buffers, or nullptr for the workspace's own.
 static int stage(const teno_params *p, const double *Uk, const double *Un, double *out, int mode,
                  double dt_host, const double *dt_dev, uint8_t *flags, char *ws, cudaStream_t s,
-                 const uint8_t *frozen, const double *P_in, double *P_out, bool full_ct = true)
+                 const uint8_t *frozen, const double *P_in, double *P_out, bool full_ct = true,
+                 const SweepMem *sm = nullptr)
 {
     static const char *kStageName[4] = {"teno rhs", "teno rk3 stage 1", "teno rk3 stage 2",
                                         "teno rk3 stage 3"};
-    static const char *kSweepName[3] = {"teno face sweep x", "teno face sweep y",
-                                        "teno face sweep z"};
     NvtxRange range(kStageName[mode]);
     const Layout L = layout(p);
     Status *st = (Status *)(ws + L.status);
     const Consts K = consts_of(p);
     const double3 idx = inv_dx_of(p);
     const int nd = p->ndim, nc = ncons(p);
+    const SweepMem M = sm ? *sm : sweep_mem(p, ws + L.sweep, kChunkTiles);
     if (p->limiter && nd > 1) CUDA_TRY(launch_wave_max(p, Uk, st, 0, s));
-    prepare_kernel<<<1, 1, 0, s>>>(st, nd, dt_host, dt_dev, idx, p->limiter);
+    prepare_kernel<<<1, M.nchunks > 32 ? 256 : 32, 0, s>>>(st, nd, dt_host, dt_dev, idx, p->limiter,
+                                                         M.counters, (int)M.nchunks);
     CUDA_TRY(cudaGetLastError());
     uint8_t *fl = flags;
     const uint8_t *fz = frozen;
@@ -477,49 +527,82 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
     uint16_t *am = flags ? (uint16_t *)(flags + dec_bytes) : nullptr;
     const uint16_t *fam = frozen ? (const uint16_t *)(frozen + dec_bytes) : nullptr;
     uint8_t *lr = flags ? flags + dec_bytes + 2 * nfaces_all : nullptr;   // limiter bytes
+    SweepArgs a;
+    a.g.U = Uk;
+    a.g.P = P_in;
+    a.g.st = st;
+    for (int k = 0; k < 3; k++) a.g.n[k] = p->n[k];
+    a.g.ncell = ncells(p);
+    a.g.fast = filter_on(p);
+    a.g.need_ct = (fl && full_ct) ? 1 : 0;
+    a.g.count_cells = !P_in;          // the x sweep counts the stage input's cells
+                                      // unless its primitives were stored
+    a.g.limiter = p->limiter;
+    a.g.tag = 0;
+    a.exact_count = g_prof.on ? g_prof.exact : nullptr;
+    a.FK = fastk_of(p);
+    a.K = K;
+    sweep_buf_layout(a.buf, M.mem, M.nt, nd, p->scheme, p->limiter != 0);
+    int64_t tiles[3] = {0, 0, 0};
     for (int d = 0; d < nd; d++) {
-        FaceArgs a;
-        a.U = Uk;
-        a.P = P_in;
-        a.F = (double *)(ws + L.flux[d]);
-        a.flags = fl;
-        a.frozen = fz;
-        a.argmax = am;
-        a.frozen_argmax = fam;
-        a.limrec = lr;
-        a.st = st;
-        for (int k = 0; k < 3; k++) a.n[k] = p->n[k];
-        a.ncell = ncells(p);
-        a.nfaces = face_grid(p, d);
-        a.bc_lo = p->bc_lo[d];
-        a.bc_hi = p->bc_hi[d];
-        a.bcs_lo = p->bc_state_lo[d];
-        a.bcs_hi = p->bc_state_hi[d];
-        a.lam = &st->lam[d];
-        a.fast = filter_on(p);
-        a.need_ct = (fl && full_ct) ? 1 : 0;
-        a.skip_last = (p->bc_lo[d] == TENO_BC_PERIODIC && !fl && !fz) ? 1 : 0;
-        a.count_cells = (d == 0 && !P_in);        // the x sweep counts the stage input's cells
-                                                  // unless its primitives were stored
-        a.exact_count = g_prof.on ? g_prof.exact : nullptr;
-        a.FK = fastk_of(p);
-        a.K = K;
-        const int slot = (g_prof.on && g_prof.used < ProfileRecord::kMax) ? g_prof.used++ : -1;
-        if (slot >= 0) {
-            g_prof.nf[slot] = a.nfaces - (a.skip_last ? a.ncell / p->n[d] : 0);   // faces computed
-            CUDA_TRY(profile_mark(0, slot, s));
-        }
-        nvtxRangePushA(kSweepName[d]);
-        cudaError_t e = (p->scheme == 8) ? launch_face8(nd, d, a, s)
-                      : (p->scheme == 10 ? launch_face10(nd, d, a, s) : launch_face12(nd, d, a, s));
-        nvtxRangePop();
-        if (e != cudaSuccess) return TENO_ECUDA;
-        if (slot >= 0) CUDA_TRY(profile_mark(1, slot, s));
+        DirArgs &D = a.dir[d];
+        D.F = (double *)(ws + L.flux[d]);
+        D.flags = fl;
+        D.frozen = fz;
+        D.argmax = am;
+        D.frozen_argmax = fam;
+        D.limrec = lr;
+        D.nfaces = face_grid(p, d);
+        D.bc_lo = p->bc_lo[d];
+        D.bc_hi = p->bc_hi[d];
+        D.bcs_lo = p->bc_state_lo[d];
+        D.bcs_hi = p->bc_state_hi[d];
+        D.lam = &st->lam[d];
+        D.skip_last = (p->bc_lo[d] == TENO_BC_PERIODIC && !fl && !fz) ? 1 : 0;
+        tiles[d] = shape_tiles(p, d, D.skip_last, D);
         if (fl) fl += (size_t)face_grid(p, d) * nc * 2;
         if (fz) fz += (size_t)face_grid(p, d) * nc * 2;
         if (am) am += face_grid(p, d);
         if (fam) fam += face_grid(p, d);
         if (lr) lr += face_grid(p, d);
+    }
+    // all directions' tiles in order, cut into chunks that fit the buffers
+    int d = 0;
+    int64_t done = 0;                 // tiles of direction d already in a chunk
+    for (int64_t chunk = 0; d < nd; chunk++) {
+        a.nparts = 0;
+        a.tiles = 0;
+        a.nexact = M.counters + chunk;
+        int64_t faces = 0;            // computed by this chunk (for the profile)
+        while (d < nd && a.tiles < M.nt) {
+            const int64_t room = M.nt - a.tiles, left = tiles[d] - done;
+            const int64_t take = left < room ? left : room;
+            const int64_t fd = a.g.ncell / p->n[d] * (p->n[d] + 1 - a.dir[d].skip_last);
+            SweepPart &q = a.part[a.nparts++];
+            q.t0 = done;
+            q.first = a.tiles;
+            q.count = (int32_t)take;
+            q.d = d;
+            a.tiles += (int32_t)take;
+            faces += (int64_t)((double)fd * (double)(done + take) / (double)tiles[d]) -
+                     (int64_t)((double)fd * (double)done / (double)tiles[d]);
+            done += take;
+            if (done == tiles[d]) {
+                d++;
+                done = 0;
+            }
+        }
+        const int slot = (g_prof.on && g_prof.used < ProfileRecord::kMax) ? g_prof.used++ : -1;
+        if (slot >= 0) {
+            g_prof.nf[slot] = faces;
+            CUDA_TRY(profile_mark(0, slot, s));
+        }
+        nvtxRangePushA("teno face fluxes");
+        cudaError_t e = (p->scheme == 8) ? launch_chunk8(nd, a, s)
+                      : (p->scheme == 10 ? launch_chunk10(nd, a, s) : launch_chunk12(nd, a, s));
+        nvtxRangePop();
+        if (e != cudaSuccess) return TENO_ECUDA;
+        if (slot >= 0) CUDA_TRY(profile_mark(1, slot, s));
     }
     CombineArgs c;
     for (int d = 0; d < 3; d++) {
@@ -929,6 +1012,10 @@ const char *teno_strerror(int code)
 // ---------------------------------------------------------------------------
 
 static __device__ __align__(256) unsigned char g_rhs_scratch[TENO_RHS_STATIC_SCRATCH_BYTES];
+// The sweeps' buffers of that entry point: some 17000 faces of the largest kind
+// at a time, about one face per lane of the warps that run at once.
+constexpr size_t kStaticSweepBytes = 32u << 20;
+static __device__ __align__(256) unsigned char g_rhs_sweep[kStaticSweepBytes];
 
 namespace {
 constexpr int kMaxDevices = 64;
@@ -940,7 +1027,7 @@ std::mutex g_scratch_mutex;
 // which a re-created context never repeats).
 struct ScratchEntry {
     unsigned long long ctx_id;
-    void *ptr;
+    void *ptr, *sweep;
 };
 ScratchEntry g_scratch[kMaxDevices] = {};
 CUresult (*g_ctx_get_current)(CUcontext *) = nullptr;
@@ -972,7 +1059,7 @@ static int current_context_id(unsigned long long *id)
 // Device address of g_rhs_scratch in the current context, resolved once per
 // device and context (the host-side symbol is only a stand-in, never a device
 // address).
-static int rhs_scratch_address(void **out)
+static int rhs_scratch_address(void **out, void **sweep)
 {
     int dev = 0;
     CUDA_TRY(cudaGetDevice(&dev));
@@ -984,12 +1071,16 @@ static int rhs_scratch_address(void **out)
     ScratchEntry &e = g_scratch[dev];
     if (!e.ptr || id == 0 || e.ctx_id != id) {
         void *ptr = nullptr;
+        void *sptr = nullptr;
         CUDA_TRY(cudaGetSymbolAddress(&ptr, g_rhs_scratch));   // initialises the context if needed
+        CUDA_TRY(cudaGetSymbolAddress(&sptr, g_rhs_sweep));
         if ((r = current_context_id(&id))) return r;
         e.ptr = ptr;
+        e.sweep = sptr;
         e.ctx_id = id;
     }
     *out = e.ptr;
+    *sweep = e.sweep;
     return TENO_OK;
 }
 
@@ -1003,12 +1094,16 @@ extern "C" int teno_rhs_static(const teno_params *p, const double *U, double *rh
     // The right-hand side needs the status header and the face-flux buffers
     // (the part of the workspace layout before the RK stage buffer).
     if (layout(p).stage > (size_t)TENO_RHS_STATIC_SCRATCH_BYTES) return TENO_EINVAL;
-    void *scratch = nullptr;
-    if ((r = rhs_scratch_address(&scratch))) return r;
+    void *scratch = nullptr, *sweep = nullptr;
+    if ((r = rhs_scratch_address(&scratch, &sweep))) return r;
+    int64_t nt = kChunkTiles;             // as many tiles as the static buffers hold
+    while (nt > 1 && sweep_mem(p, nullptr, nt).bytes > kStaticSweepBytes) nt = nt * 7 / 8;
+    const SweepMem sm = sweep_mem(p, (char *)sweep, nt);
+    if (sm.bytes > kStaticSweepBytes) return TENO_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     // The array keeps the previous call's contents: zero the status header
     // (counters and reduction slots) before use.
     CUDA_TRY(cudaMemsetAsync(scratch, 0, sizeof(Status), s));
     return stage(p, U, U, rhs, 0, dt_limiter, nullptr, flags, (char *)scratch, s, nullptr, nullptr,
-                 nullptr);
+                 nullptr, true, &sm);
 }

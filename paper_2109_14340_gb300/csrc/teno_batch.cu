@@ -29,7 +29,10 @@ struct BatchSlot {
 };
 
 constexpr int kCellTile = 256;
-constexpr int kTiles[3] = {64, 128, 256};
+constexpr int kTiles[3] = {64, 128, 256};   // faces in flight per block (a warp: 32)
+constexpr int kBatchSlice =                 // doubles of shared memory per warp
+    FaceSmem<1, 5>::TOTAL > FaceSmem<1, 4>::TOTAL ? FaceSmem<1, 5>::TOTAL : FaceSmem<1, 4>::TOTAL;
+constexpr size_t batch_smem(int TF) { return sizeof(double) * kBatchSlice * (TF / 32); }
 
 // Item -> problem by binary search in an exclusive prefix of per-problem item
 // counts (prefix[nprob] = total).
@@ -99,53 +102,62 @@ __global__ void batch_finalize_kernel(const BatchProb *probs, int nprob, BatchSl
     slots[p].amax = 0ull;
 }
 
-// Registers bounded as for the 2D/3D sweeps: 384 threads' worth of blocks per SM.
+// Persistent face sweep of the chunk's tiles first .. first+count-1: every warp
+// pulls (problem, 32-face tile) items from the counter on its own.  TF threads
+// per block, registers bounded as for the single-problem sweep.
 template <int TF>
-__global__ void __launch_bounds__(TF, (384 / TF > 1 ? 384 / TF : 1)) batch_face_kernel(
-    const BatchProb *probs, int nprob, const int32_t *fprefix, const double *U, const double *P,
-    double *F, BatchSlot *slots, Status *st, Consts K, FastK FK, int fast, int *counter)
+__global__ void __launch_bounds__(TF, 512 / TF) batch_sweep_kernel(
+    const BatchProb *probs, int nprob, const int32_t *fprefix, int first, int count, const double *U,
+    const double *P, SweepBuf B, Status *st, Consts K, FastK FK, int fast, int *counter)
 {
     extern __shared__ double sm[];
-    __shared__ int s_item;
-    const int nitems = fprefix[nprob];
+    double *slice = sm + (size_t)(threadIdx.x >> 5) * kBatchSlice;
     for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
-        __syncthreads();
-        const int it = s_item;
-        if (it >= nitems) break;
-        const int p = find_problem(fprefix, nprob, it);
+        int it = 0;
+        if ((threadIdx.x & 31) == 0) it = atomicAdd(counter, 1);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= count) break;
+        const int p = find_problem(fprefix, nprob, first + it);
         const BatchProb d = probs[p];
-        FaceArgs a;
-        a.U = U + d.u_off;
-        a.P = P + d.p_off;                  // the stage input's stored primitives
-        a.F = F + d.f_off;
-        a.flags = nullptr;
-        a.frozen = nullptr;
-        a.argmax = nullptr;
-        a.frozen_argmax = nullptr;
-        a.limrec = nullptr;
-        a.st = st;
-        a.n[0] = d.n; a.n[1] = 1; a.n[2] = 1;
-        a.ncell = d.n;
+        GridArgs g;
+        g.U = U + d.u_off;
+        g.P = P + d.p_off;                  // the stage input's stored primitives
+        g.st = st;
+        g.n[0] = d.n; g.n[1] = 1; g.n[2] = 1;
+        g.ncell = d.n;
+        g.fast = fast;
+        g.need_ct = 0;
+        g.count_cells = 0;
+        g.limiter = d.limiter;
+        g.tag = d.scheme == 10 ? 0x80000000u : 0u;
+        DirArgs a;
         a.nfaces = d.n + 1;
         a.bc_lo = d.bc_lo;
         a.bc_hi = d.bc_hi;
         a.bcs_lo = nullptr;
         a.bcs_hi = nullptr;
-        a.lam = &slots[p].lam;
-        a.fast = fast;
-        a.need_ct = 0;
         a.skip_last = 0;
-        a.count_cells = 0;
-        a.exact_count = nullptr;
-        a.FK = FK;
-        a.K = K;
-        a.K.limiter = d.limiter;
-        const int64_t f0 = (int64_t)(it - fprefix[p]) * TF;
-        if (d.scheme == 10) face_block<1, 5, 0, 1, TF, kSweepPlain>(a, f0, 0, 0, 0, sm);
-        else face_block<1, 4, 0, 1, TF, kSweepPlain>(a, f0, 0, 0, 0, sm);
-        __syncthreads();
+        const int64_t f0 = (int64_t)(first + it - fprefix[p]) * kTileFaces;
+        if (d.scheme == 10) sweep_tile<1, 5, 0, kSweepPlain>(g, a, FK, K, B, f0, 0, 0, 0, it, slice);
+        else sweep_tile<1, 4, 0, kSweepPlain>(g, a, FK, K, B, f0, 0, 0, 0, it, slice);
     }
+}
+
+__global__ void __launch_bounds__(128) batch_finish_kernel(
+    const BatchProb *probs, int nprob, const int32_t *fprefix, int first, int count, double *F,
+    SweepBuf B, const BatchSlot *slots, Status *st, Consts K)
+{
+    const int it = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (it >= count) return;
+    const int p = find_problem(fprefix, nprob, first + it);
+    const BatchProb d = probs[p];
+    const int64_t f = (int64_t)(first + it - fprefix[p]) * kTileFaces + lane;
+    if (f > d.n) return;
+    DirArgs a;
+    a.F = F + d.f_off;
+    a.lam = &slots[p].lam;
+    a.nfaces = d.n + 1;
+    finish_face<1, 0, kSweepPlain>(a, d.limiter, K, B, (int64_t)it * kTileFaces + lane, f, st);
 }
 
 // Flux difference and SSP-RK3 stage per cell (the arithmetic of combine_kernel
@@ -199,11 +211,14 @@ struct teno_batch {
     teno_params common;
     std::vector<teno_batch_problem> probs;
     std::vector<BatchProb> desc;
-    std::vector<int32_t> fprefix[3];
+    std::vector<int32_t> fprefix;
     std::vector<int32_t> cprefix;
     size_t u_len = 0, f_len = 0, p_len = 0;
-    size_t off_slots = 0, off_counters = 0, off_desc = 0, off_fprefix[3] = {0, 0, 0},
-           off_cprefix = 0, off_F = 0, off_Us = 0, off_P = 0, off_single = 0, total = 0;
+    int64_t chunk_tiles = 0;    // tiles per pass through the sweep's buffers
+    bool has8 = false, has10 = false, has_limiter = false;
+    int nchunks() const { return (int)((fprefix.back() + chunk_tiles - 1) / chunk_tiles); }
+    size_t off_slots = 0, off_counters = 0, off_desc = 0, off_fprefix = 0,
+           off_cprefix = 0, off_F = 0, off_Us = 0, off_P = 0, off_sweep = 0, off_xlist10 = 0, off_single = 0, total = 0;
     size_t single_bytes = 0;
     int tile_idx = 1;           // index into kTiles
     int blocks_per_sm = 2;
@@ -263,8 +278,8 @@ Consts consts_common(const teno_params *p)
 template <int TF>
 cudaError_t set_face_attr()
 {
-    constexpr size_t smem = std::max(face_smem_bytes<1, 5, 1, TF>(), face_smem_bytes<1, 4, 1, TF>());
-    return cudaFuncSetAttribute(batch_face_kernel<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    constexpr size_t smem = batch_smem(TF);
+    return cudaFuncSetAttribute(batch_sweep_kernel<TF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem);
 }
 
@@ -277,9 +292,8 @@ int upload(teno_batch *b, char *ws, cudaStream_t s)
     CUDA_TRY(cudaMemsetAsync(ws, 0, b->off_desc, s));       // status, slots, counters
     CUDA_TRY(cudaMemcpyAsync(ws + b->off_desc, b->desc.data(), sizeof(BatchProb) * np,
                              cudaMemcpyHostToDevice, s));
-    for (int k = 0; k < 3; k++)
-        CUDA_TRY(cudaMemcpyAsync(ws + b->off_fprefix[k], b->fprefix[k].data(),
-                                 sizeof(int32_t) * (np + 1), cudaMemcpyHostToDevice, s));
+    CUDA_TRY(cudaMemcpyAsync(ws + b->off_fprefix, b->fprefix.data(), sizeof(int32_t) * (np + 1),
+                             cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaMemcpyAsync(ws + b->off_cprefix, b->cprefix.data(), sizeof(int32_t) * (np + 1),
                              cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaStreamSynchronize(s));     // the host vectors are pageable
@@ -304,14 +318,19 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
     BatchSlot *slots = (BatchSlot *)(ws + b->off_slots);
     int *counters = (int *)(ws + b->off_counters);
     const BatchProb *desc = (const BatchProb *)(ws + b->off_desc);
-    const int32_t *fpre = (const int32_t *)(ws + b->off_fprefix[tile_idx]);
+    const int32_t *fpre = (const int32_t *)(ws + b->off_fprefix);
     const int32_t *cpre = (const int32_t *)(ws + b->off_cprefix);
     double *F = (double *)(ws + b->off_F);
     double *Us = (double *)(ws + b->off_Us);
     double *P = (double *)(ws + b->off_P);
+    SweepBuf B;
+    sweep_buf_layout(B, ws + b->off_sweep, b->chunk_tiles, 1, 10, b->has_limiter);
+    uint32_t *xlist10 = (uint32_t *)(ws + b->off_xlist10);
     const int ncitems = b->cprefix[np];
     const int grid_c = std::max(1, std::min(ncitems, b->num_sms * 8));
-    CUDA_TRY(cudaMemsetAsync(counters, 0, 3 * sizeof(int), s));
+    // per stage and chunk: the sweep's item counter, the two schemes' exact-path lists
+    const int nchunks = b->nchunks();
+    CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(int) * 9 * nchunks, s));
     batch_wave_max_kernel<<<grid_c, kCellTile, 0, s>>>(desc, np, cpre, U, slots, P, st, K);
     CUDA_TRY(cudaGetLastError());
     batch_finalize_kernel<<<(np + 127) / 128, 128, 0, s>>>(desc, np, slots, cfl);
@@ -323,17 +342,28 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
     const int fast = g_fast_filter && fast_filter_valid(b->common.eps_beta, b->common.eps_eta);
     for (int stg = 0; stg < 3; stg++) {
         const double *Uin = stg == 0 ? U : Us;
-        if (TF == 64) {
-            constexpr size_t sm = std::max(face_smem_bytes<1, 5, 1, 64>(), face_smem_bytes<1, 4, 1, 64>());
-            batch_face_kernel<64><<<grid_f, 64, sm, s>>>(desc, np, fpre, Uin, P, F, slots, st, K, FK, fast, counters + stg);
-        } else if (TF == 128) {
-            constexpr size_t sm = std::max(face_smem_bytes<1, 5, 1, 128>(), face_smem_bytes<1, 4, 1, 128>());
-            batch_face_kernel<128><<<grid_f, 128, sm, s>>>(desc, np, fpre, Uin, P, F, slots, st, K, FK, fast, counters + stg);
-        } else {
-            constexpr size_t sm = std::max(face_smem_bytes<1, 5, 1, 256>(), face_smem_bytes<1, 4, 1, 256>());
-            batch_face_kernel<256><<<grid_f, 256, sm, s>>>(desc, np, fpre, Uin, P, F, slots, st, K, FK, fast, counters + stg);
+        for (int c = 0; c < nchunks; c++) {
+            int *cnt = counters + 3 * (stg * nchunks + c);
+            const int first = c * (int)b->chunk_tiles;
+            const int count = std::min((int)b->chunk_tiles, b->fprefix[np] - first);
+            if (TF == 64)
+                batch_sweep_kernel<64><<<grid_f, 64, batch_smem(64), s>>>(desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt);
+            else if (TF == 128)
+                batch_sweep_kernel<128><<<grid_f, 128, batch_smem(128), s>>>(desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt);
+            else
+                batch_sweep_kernel<256><<<grid_f, 256, batch_smem(256), s>>>(desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt);
+            CUDA_TRY(cudaGetLastError());
+            if (b->has8)
+                CUDA_TRY((launch_decisions<4, false>(B, count, 3, fast, 0, b->has10 ? 1 : 0,
+                                                     (unsigned *)cnt + 1, nullptr, FK, K, st, s)));
+            SweepBuf B10 = B;
+            B10.xlist = xlist10;
+            if (b->has10)
+                CUDA_TRY((launch_decisions<5, false>(B10, count, 3, fast, 0, b->has8 ? 2 : 0,
+                                                     (unsigned *)cnt + 2, nullptr, FK, K, st, s)));
+            batch_finish_kernel<<<(count + 3) / 4, 128, 0, s>>>(desc, np, fpre, first, count, F, B, slots, st, K);
+            CUDA_TRY(cudaGetLastError());
         }
-        CUDA_TRY(cudaGetLastError());
         batch_combine_kernel<<<grid_c, kCellTile, 0, s>>>(desc, np, cpre, Uin, U, stg == 2 ? U : Us, F,
                                                          slots, P, st, K, stg + 1);
         CUDA_TRY(cudaGetLastError());
@@ -373,8 +403,8 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
     b->common.ndim = 1;
     b->probs.assign(probs, probs + nprob);
     size_t f_off = 0, p_off = 0, u_end = 0, single = 0;
-    int64_t ftiles[3] = {0, 0, 0}, ctiles = 0;
-    for (int k = 0; k < 3; k++) b->fprefix[k].push_back(0);
+    int64_t ftiles = 0, ctiles = 0;
+    b->fprefix.push_back(0);
     b->cprefix.push_back(0);
     for (int p = 0; p < nprob; p++) {
         const teno_batch_problem &q = probs[p];
@@ -398,6 +428,8 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
         d.inv_dx = 1.0 / q.dx;
         d.scheme = q.scheme;
         d.limiter = q.limiter;
+        (q.scheme == 10 ? b->has10 : b->has8) = true;
+        if (q.limiter) b->has_limiter = true;
         d.bc_lo = q.bc_lo;
         d.bc_hi = q.bc_hi;
         b->desc.push_back(d);
@@ -405,13 +437,11 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
         f_off = (f_off + 1) & ~(size_t)1;                 // keep 16-byte alignment
         p_off += (size_t)PrimRows<1>::NP * (size_t)q.n;
         u_end = std::max(u_end, (size_t)(q.offset + 3 * q.n));
-        for (int k = 0; k < 3; k++) {
-            ftiles[k] += (q.n + 1 + kTiles[k] - 1) / kTiles[k];
-            b->fprefix[k].push_back((int32_t)ftiles[k]);
-        }
+        ftiles += (q.n + 1 + kTileFaces - 1) / kTileFaces;
+        b->fprefix.push_back((int32_t)ftiles);
         ctiles += (q.n + kCellTile - 1) / kCellTile;
         b->cprefix.push_back((int32_t)ctiles);
-        if (ftiles[0] > (int64_t)1 << 30 || ctiles > (int64_t)1 << 30) {
+        if (ftiles > (int64_t)1 << 30 || ctiles > (int64_t)1 << 30) {
             delete b;
             return TENO_EINVAL;
         }
@@ -429,14 +459,13 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
     size_t off = a256(sizeof(Status));
     b->off_slots = off;
     off += a256(sizeof(BatchSlot) * nprob);
+    b->chunk_tiles = std::min<int64_t>(kChunkTiles, ftiles);
     b->off_counters = off;
-    off += 256;
+    off += a256(sizeof(int) * 9 * (size_t)b->nchunks());
     b->off_desc = off;
     off += a256(sizeof(BatchProb) * nprob);
-    for (int k = 0; k < 3; k++) {
-        b->off_fprefix[k] = off;
-        off += a256(sizeof(int32_t) * (nprob + 1));
-    }
+    b->off_fprefix = off;
+    off += a256(sizeof(int32_t) * (nprob + 1));
     b->off_cprefix = off;
     off += a256(sizeof(int32_t) * (nprob + 1));
     b->off_F = off;
@@ -445,6 +474,11 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
     off += a256(sizeof(double) * b->u_len);
     b->off_P = off;
     off += a256(sizeof(double) * b->p_len);
+    SweepBuf B;
+    b->off_sweep = off;
+    off += sweep_buf_layout(B, nullptr, b->chunk_tiles, 1, 10, b->has_limiter);
+    b->off_xlist10 = off;
+    off += a256(sizeof(uint32_t) * 64 * 3 * (size_t)b->chunk_tiles);
     b->off_single = off;
     off += a256(single);
     b->total = off;
@@ -530,14 +564,14 @@ int teno_batch_autotune(teno_batch *b, double *U_scratch, void *ws, size_t ws_by
             const int TF = kTiles[ti];
             cudaError_t oe;
             if (TF == 64)
-                oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&maxb, batch_face_kernel<64>, 64,
-                         std::max(face_smem_bytes<1, 5, 1, 64>(), face_smem_bytes<1, 4, 1, 64>()));
+                oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&maxb, batch_sweep_kernel<64>, 64,
+                         batch_smem(64));
             else if (TF == 128)
-                oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&maxb, batch_face_kernel<128>, 128,
-                         std::max(face_smem_bytes<1, 5, 1, 128>(), face_smem_bytes<1, 4, 1, 128>()));
+                oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&maxb, batch_sweep_kernel<128>, 128,
+                         batch_smem(128));
             else
-                oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&maxb, batch_face_kernel<256>, 256,
-                         std::max(face_smem_bytes<1, 5, 1, 256>(), face_smem_bytes<1, 4, 1, 256>()));
+                oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&maxb, batch_sweep_kernel<256>, 256,
+                         batch_smem(256));
             if (oe != cudaSuccess) return TENO_ECUDA;
             if (bps_c[bi] > maxb) continue;
             CUDA_TRY(cudaEventRecord(e0, s));

@@ -95,6 +95,7 @@ static __constant__ float TENO_SOS6_D[5] = {0x1.2785020000000p+0f, 0x1.5a97ca000
 static __constant__ float TENO_SOS6_DC[5] = {0x1.9656ea0000000p+4f, 0x1.63784e0000000p+3f, 0x1.92de820000000p+2f, 0x1.5c811a0000000p+2f, 0x1.a182c60000000p-4f};
 #define TENO_SOS6_TAU2 0x1.8000060000000p-19f
 #define TENO_SOS6_K0 0x1.833f7e0000000p-30f
+#define TENO_SOS6_KAPPA 0x1.a067fa0000000p+4f
 
 // TENO_SOS8: sum-of-squares form of the large stencil's indicator, variables at offsets [4, 3, 2, 1, -1, -2, -3]
 static __constant__ float TENO_SOS8_L[7][7] = {
@@ -110,6 +111,7 @@ static __constant__ float TENO_SOS8_D[7] = {0x1.35c4d20000000p+0f, 0x1.5fd710000
 static __constant__ float TENO_SOS8_DC[7] = {0x1.c2220a0000000p+6f, 0x1.9783a00000000p+5f, 0x1.d2e30e0000000p+4f, 0x1.26cfb40000000p+4f, 0x1.8763da0000000p+4f, 0x1.b096ca0000000p-1f, 0x1.08fdfe0000000p-6f};
 #define TENO_SOS8_TAU2 0x1.8000060000000p-19f
 #define TENO_SOS8_K0 0x1.cea02c0000000p-26f
+#define TENO_SOS8_KAPPA 0x1.c6deec0000000p+6f
 
 // TENO_SOS10: sum-of-squares form of the large stencil's indicator, variables at offsets [5, 4, 3, 2, 1, -1, -2, -3, -4]
 static __constant__ float TENO_SOS10_L[9][9] = {
@@ -127,6 +129,7 @@ static __constant__ float TENO_SOS10_D[9] = {0x1.488eb20000000p+0f, 0x1.6914c400
 static __constant__ float TENO_SOS10_DC[9] = {0x1.ef67300000000p+8f, 0x1.c67c1e0000000p+7f, 0x1.fae0f80000000p+6f, 0x1.3ff9f60000000p+6f, 0x1.a36aae0000000p+5f, 0x1.6be1040000000p+6f, 0x1.22ac5a0000000p+2f, 0x1.58c6980000000p-3f, 0x1.4bb6960000000p-9f};
 #define TENO_SOS10_TAU2 0x1.8000060000000p-19f
 #define TENO_SOS10_K0 0x1.0b2d620000000p-21f
+#define TENO_SOS10_KAPPA 0x1.e89dba0000000p+8f
 
 // TENO_SOS12: sum-of-squares form of the large stencil's indicator, variables at offsets [6, 5, 4, 3, 2, 1, -1, -2, -3, -4, -5]
 static __constant__ float TENO_SOS12_L[11][11] = {
@@ -146,4 +149,5 @@ static __constant__ float TENO_SOS12_D[11] = {0x1.6052100000000p+0f, 0x1.76c0280
 static __constant__ float TENO_SOS12_DC[11] = {0x1.10d7920000000p+11f, 0x1.f762e60000000p+9f, 0x1.0c3f360000000p+9f, 0x1.52df260000000p+8f, 0x1.b473800000000p+7f, 0x1.218ae80000000p+7f, 0x1.30b05e0000000p+8f, 0x1.3dbe160000000p+4f, 0x1.1270660000000p+0f, 0x1.0d1dd60000000p-5f, 0x1.9303ca0000000p-12f};
 #define TENO_SOS12_TAU2 0x1.8000060000000p-19f
 #define TENO_SOS12_K0 0x1.309c9e0000000p-17f
+#define TENO_SOS12_KAPPA 0x1.04be3e0000000p+11f
 

@@ -197,18 +197,35 @@ __device__ __forceinline__ int ct_exponent(const double (&v)[2 * H], const Const
 #undef V
 }
 
+// x / 6 rounded to nearest: Markstein's correction of the product with the
+// correctly rounded reciprocal (IBM J. Res. Dev. 34, 1990; for a constant
+// divisor Brisebarre and Muller, 2008), three FP64 operations in place of
+// the general division's eight or so.  r = fma(-6, q, x) is exact and q' is
+// the rounded quotient where neither underflows; elsewhere (and for zeros,
+// infinities and NaN) the division itself.
+__device__ __forceinline__ double sixth(double x)
+{
+    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu;
+    if (e - 128u > 2046u - 128u - 1u) return x / 6.0;       // below 2^-895, infinity, NaN
+    const double y = 1.0 / 6.0;
+    const double q = x * y;
+    return fma(fma(-6.0, q, x), y, q);
+}
+
 // Small-stencil fallback value (Eq. renormalize, Eq. reconstuction): the
 // kept candidates (bits 0..2 of mask) weighted by d_k renormalised over them
 // (w_k = dd_k / den, tabulated in double), the 3-point candidates divided by
-// 6 exactly as written.
+// 6 exactly as written: ((-V(-1) + 5 V(0)) + 2 V(1)) / 6,
+// ((2 V(0) + 5 V(1)) - V(2)) / 6 and ((2 V(-2) - 7 V(-1)) + 11 V(0)) / 6.
+// Doubling is exact, so each doubled term joins its sum in one fma.
 template <int H>
 __device__ __forceinline__ double fallback_value(const double (&v)[2 * H], int mask)
 {
 #define V(m) v[(m) + H - 1]
     const double w0 = TENO_FBW[mask][0], w1 = TENO_FBW[mask][1], w2 = TENO_FBW[mask][2];
-    double f0 = ((-V(-1) + 5.0 * V(0)) + 2.0 * V(1)) / 6.0;
-    double f1 = ((2.0 * V(0) + 5.0 * V(1)) - V(2)) / 6.0;
-    double f2 = ((2.0 * V(-2) - 7.0 * V(-1)) + 11.0 * V(0)) / 6.0;
+    const double f0 = sixth(fma(2.0, V(1), 5.0 * V(0) - V(-1)));
+    const double f1 = sixth(fma(2.0, V(0), 5.0 * V(1)) - V(2));
+    const double f2 = sixth(fma(2.0, V(-2), -7.0 * V(-1)) + 11.0 * V(0));
     double fh = w0 * f0;
     fh = fma(w1, f1, fh);
     fh = fma(w2, f2, fh);
@@ -274,6 +291,50 @@ __device__ __forceinline__ double teno_recon(const double (&v)[2 * H], const Con
 #undef V
 }
 
+// Coefficient of S_L's linear scheme at value index m of a 2H stencil, and
+// whether S_L covers it.
+template <int H, int L>
+__device__ __forceinline__ constexpr bool covers(int m)
+{
+    return m >= H - L && m < H + L;
+}
+
+// Value of the selected large stencil S_sel (3 <= sel <= H), lanes with
+// different stencils in one chain of 2H fma: each step takes the lane's own
+// coefficient, a lane whose stencil has not begun starts from -0 (to which a
+// product adds itself, a zero's sign included), and one whose stencil has
+// ended keeps its sum.  Bitwise flux_large<H, sel>; a branch per stencil
+// would run the chains one after the other.
+template <int H>
+__device__ __forceinline__ double large_value(const double (&v)[2 * H], int sel)
+{
+    double acc = -0.0;
+#pragma unroll
+    for (int m = 0; m < 2 * H; m++) {
+        double c = lcoef<H>(m);
+        bool in = true;
+        if constexpr (H >= 6) {
+            if (sel == 5) {
+                in = covers<H, 5>(m);
+                if (covers<H, 5>(m)) c = lcoef<5>(m - (H - 5));
+            }
+        }
+        if constexpr (H >= 5) {
+            if (sel == 4) {
+                in = covers<H, 4>(m);
+                if (covers<H, 4>(m)) c = lcoef<4>(m - (H - 4));
+            }
+        }
+        if (sel == 3) {
+            in = covers<H, 3>(m);
+            if (covers<H, 3>(m)) c = lcoef<3>(m - (H - 3));
+        }
+        const double t = fma(c, v[m], acc);
+        acc = in ? t : acc;
+    }
+    return acc;
+}
+
 // The value of a reconstruction whose decisions are known (decision byte in
 // the encoding above): the selected large stencil's linear scheme or the
 // small-stencil fallback, with the exact path's arithmetic.
@@ -281,17 +342,9 @@ template <int H>
 __device__ __forceinline__ double decided_value(const double (&v)[2 * H], uint8_t flag)
 {
     const int sel = flag & 3;
-    if constexpr (H == 6) {
-        if ((flag & 31) == 0) return flux_large<H, 6>(v);
-        if (sel == 3) return flux_large<H, 5>(v);
-    } else {
-        if (sel == H - 2) return flux_large<H, H>(v);
-    }
-    if constexpr (H >= 5) {
-        if (sel == 2) return flux_large<H, 4>(v);
-    }
-    if (sel == 1) return flux_large<H, 3>(v);
-    return fallback_value<H>(v, (flag >> 2) & 7);
+    const bool s6 = H == 6 && (flag & 31) == 0;
+    if (sel == 0 && !s6) return fallback_value<H>(v, (flag >> 2) & 7);
+    return large_value<H>(v, s6 ? 6 : sel + 2);
 }
 
 // Frozen reconstruction coefficient of value index m (offset m - H + 1) for a
@@ -400,33 +453,17 @@ __device__ __forceinline__ void store_prims(const CellQ<ND> &q, double *P, int64
     P[R::SR * ncell + id] = q.sr;
 }
 
-// cell_quantities of a cell whose primitives were stored by store_prims: the
-// flux along D is formed from them with the same operations, so every value
-// is bitwise the one cell_quantities gives (rinv is not recovered).
-template <int ND, int D>
-__device__ __forceinline__ void cell_from_prims(const double (&Uc)[ND + 2], const double *P,
-                                                int64_t ncell, int64_t id, CellQ<ND> &q)
+// The primitives of a cell that store_prims stored (U, F and rinv are not set).
+template <int ND>
+__device__ __forceinline__ void load_prims(const double *P, int64_t ncell, int64_t id, CellQ<ND> &q)
 {
     using R = PrimRows<ND>;
-    constexpr int nc = ND + 2;
-#pragma unroll
-    for (int c = 0; c < nc; c++) q.U[c] = Uc[c];
 #pragma unroll
     for (int a = 0; a < ND; a++) q.u[a] = P[a * ncell + id];
     q.p = P[R::P * ncell + id];
     q.c = P[R::C * ncell + id];
     q.H = P[R::H * ncell + id];
     q.sr = P[R::SR * ncell + id];
-    q.rinv = 0.0;
-    const double Ep = Uc[nc - 1] + q.p;
-    const double md = Uc[1 + D];
-    q.F[0] = md;
-#pragma unroll
-    for (int a = 0; a < ND; a++) {
-        q.F[1 + a] = md * q.u[a];
-        if (a == D) q.F[1 + a] = q.F[1 + a] + q.p;
-    }
-    q.F[nc - 1] = q.u[D] * Ep;
 }
 
 // The non-physical test of a cell (rho <= 0, p <= 0, non-finite c or H).
@@ -491,6 +528,7 @@ __device__ __forceinline__ double roe_state(const double (&ul)[ND], double Hl, d
 template <int ND, int D>
 __device__ __forceinline__ int shear_axis(int k)
 {
+    if (ND == 2) return 1 - D;
     int t = 0, kk = 2;
 #pragma unroll
     for (int a = 0; a < ND; a++) {
@@ -522,7 +560,12 @@ __device__ __forceinline__ void l_row(const RoeScalars<ND> &rs, int k, double (&
         l[last] = -rs.b1;
     } else {
         const int t = shear_axis<ND, D>(k);
-        l[0] = -rs.ut[t];
+        // selected, not indexed: a run-time index would put rs in local memory
+        double ut = rs.ut[0];
+#pragma unroll
+        for (int a = 1; a < ND; a++)
+            if (a == t) ut = rs.ut[a];
+        l[0] = -ut;
 #pragma unroll
         for (int a = 0; a < ND; a++) l[1 + a] = (a == t) ? 1.0 : 0.0;
         l[last] = 0.0;

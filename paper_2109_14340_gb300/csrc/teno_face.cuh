@@ -1,15 +1,30 @@
-// Face-flux sweep along one direction: for every face i+1/2 of the face grid,
-// Roe average -> eigenvectors -> characteristic projection of the 2H-cell
-// stencil -> LLF/Rusanov split -> TENO-AA reconstruction of f+ and f- per
-// field -> back-projection -> positivity limiter (arXiv 2109.14340, Sec. 3-5).
+// Face fluxes: for every face i+1/2 of the face grids, Roe average ->
+// eigenvectors -> characteristic projection of the 2H-cell stencil ->
+// LLF/Rusanov split -> TENO-AA reconstruction of f+ and f- per field ->
+// back-projection -> positivity limiter (arXiv 2109.14340, Sec. 3-5).
 //
-// Tiling: a block owns TF consecutive faces along the sweep axis D for TP
-// pencils adjacent in x.  It stages the TF + 2H - 1 cells those faces touch
-// (ghost cells resolved by the boundary rules of App. A) in shared memory as
-// per-cell primitive quantities, then one thread computes one face.  U and F
-// are staged halved (exact: a power of two), so that the projections give
-// the halved characteristic variables and fluxes w/2, g/2 directly and the
-// split fluxes (g +- alpha w)/2 need no further scaling.
+// An FP64 instruction holds its scheduler's FP64 unit for 64 cycles, with one
+// lane active or 32 (2 lanes per SM and clock), so a face costs what the warps
+// issue, idle lanes included, and the unit idles whenever all warps of a
+// scheduler are busy with something else.  The work is therefore cut where
+// lanes would diverge, over four kernels that pass values through memory
+// (about 1 kB per face at most, of a bandwidth that FP64 work leaves idle):
+//
+//   sweep   a warp per tile of 32 faces, a lane per face: staging, Roe state, projection, split fluxes.  Reconstructions
+//           that quick_large accepts for the largest stencil get their value;
+//           the others go to the tile's queue.
+//   decide  the queues of several tiles by one block: the whole filter for
+//           each entry, then the values, the large stencils' and the
+//           fallback's each on compact lanes.  What the filter leaves open
+//           goes to one list.
+//   exact   that list through the exact path, a lane per entry.
+//   finish  a lane per face: back-projection, limiter, the flux.
+//
+// The buffers between them are sized for at most kChunkTiles tiles, so a larger
+// evaluation goes through them in chunks.  U and F are staged halved (exact: a
+// power of two), so that the projections give the halved characteristic
+// variables and fluxes w/2, g/2 directly and the split fluxes (g +- alpha w)/2
+// need no further scaling.
 #pragma once
 
 #include "teno_dev.cuh"
@@ -17,35 +32,176 @@
 
 namespace teno {
 
-struct FaceArgs {
-    const double *U;       // state, [nc][ncell]
-    const double *P;       // primitives of U ([PrimRows::NP][ncell], store_prims) or
-                           // nullptr: computed while staging
-    double *F;             // face fluxes of direction D, [nc][nfaces]
-    uint8_t *flags;        // decision record of direction D or nullptr
+constexpr int kTileFaces = 32;
+// Tiles a chunk holds at most: 2 M faces.  Each chunk ends with partly filled
+// waves of its four kernels, about 40 us; 65536 tiles of 3D ten-point faces
+// take some 2.6 ms and 2 GB.
+constexpr int64_t kChunkTiles = 65536;
+
+// One direction's faces.
+struct DirArgs {
+    double *F;             // face fluxes, [nc][nfaces]
+    uint8_t *flags;        // decision record or nullptr
     const uint8_t *frozen; // recorded decisions to apply instead of deciding, or nullptr
     uint16_t *argmax;      // per face: the maximising stencil cells of the splitting
                            // speeds (4 bits each: u-c, u, u+c, |u|+c), or nullptr
     const uint16_t *frozen_argmax;   // recorded maximising cells to apply, or nullptr
     uint8_t *limrec;       // per face: 1 where the positivity limiter bound, or nullptr
+    const double *bcs_lo, *bcs_hi;   // Dirichlet boundary-face states or halo arrays, or nullptr
+    const double *lam;     // limiter's effective dt/dx for this direction (device)
+    int64_t nfaces;
+    int bc_lo, bc_hi;      // boundary rules at the two ends of the axis
+    int skip_last;         // 1: face n of each line is not computed (periodic axis, no
+                           // decision record: its flux is face 0's, bitwise)
+    // A tile is 2^tps pencils (side by side in x, in y for the x sweep) by 32 >> tps
+    // faces; tiles per line of faces, and groups of 2^tps pencils along that axis.
+    int tps;
+    int64_t line_tiles, groups;
+};
+
+// The evaluation's input.
+struct GridArgs {
+    const double *U;       // state, [nc][ncell]
+    const double *P;       // primitives of U ([PrimRows::NP][ncell], store_prims) or
+                           // nullptr: computed while staging
     Status *st;
     int64_t n[3];
-    int64_t ncell, nfaces;
-    int bc_lo, bc_hi;      // boundary rules at the two ends of axis D
-    const double *bcs_lo, *bcs_hi;   // Dirichlet boundary-face states or halo arrays of
-                                     // axis D, or nullptr
-    const double *lam;     // limiter's effective dt/dx for this direction (device)
+    int64_t ncell;
     int fast;              // 1: certified FP32 decision filter first
     int need_ct;           // 1: recorded decision bytes carry their C_T exponent; 0: only
                            // where it decided (the selection bits are exact either way)
-    int count_cells;       // 1: count the non-physical cells this sweep owns (one
-                           // sweep per evaluation does, so each cell is counted once)
-    int skip_last;         // 1: face n of each line is not computed (periodic axis, no
-                           // decision record: its flux is face 0's, bitwise)
+    int count_cells;       // 1: count the non-physical cells the x sweep owns (each cell once)
+    int limiter;           // 1: positivity limiter
+    uint32_t tag;          // top bit of the queue lengths (a batch's scheme)
+};
+
+// The buffers between the four kernels; nt: tiles they hold.  Queue entries of
+// tile t are q = t per_tile .. + count[t], per_tile = 64 nc.
+struct SweepBuf {
+    double *qv;            // [2H][nt per_tile] values of the queued reconstructions
+    uint16_t *qslot;       // [nt per_tile] (2k+s) 32 + lane
+    uint32_t *xlist;       // [nt per_tile] entries left to the exact path
+    uint32_t *count;       // [nt] queue lengths
+    double *R;             // [2 nc][nt 32] reconstructed values
+    double *RO;            // [nd + 2][nt 32] Roe velocity, enthalpy, sound speed
+    double *RL;            // [4 nc + 1][nt 32] limiter: halved U, F of cells i, i+1, and the
+                           // Lax-Friedrichs speed; nullptr without a limiter
+    uint8_t *RD;           // [2 nc][nt 32] decision bytes; nullptr without a record
+    int64_t nt;
+};
+
+inline size_t sweep_align(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Lays the buffers for nt tiles out from p (null: only measures); W values per
+// entry.  Returns the bytes used.
+inline size_t sweep_buf_layout(SweepBuf &b, char *p, int64_t nt, int nd, int W, bool limiter)
+{
+    const int nc = nd + 2;
+    const size_t q = (size_t)nt * 64 * nc, f = (size_t)nt * kTileFaces;
+    size_t off = 0;
+    auto take = [&](size_t bytes) { char *r = p + off; off += sweep_align(bytes); return r; };
+    b.nt = nt;
+    b.qv = (double *)take(sizeof(double) * W * q);
+    b.xlist = (uint32_t *)take(sizeof(uint32_t) * q);
+    b.qslot = (uint16_t *)take(sizeof(uint16_t) * q);
+    b.count = (uint32_t *)take(sizeof(uint32_t) * nt);
+    b.R = (double *)take(sizeof(double) * 2 * nc * f);
+    b.RO = (double *)take(sizeof(double) * (nd + 2) * f);
+    b.RD = (uint8_t *)take(2 * nc * f);
+    b.RL = limiter ? (double *)take(sizeof(double) * (4 * nc + 1) * f) : nullptr;
+    return off;
+}
+
+// A run of tiles of one direction inside a chunk: tiles first .. first+count-1
+// of the chunk are tiles t0 .. of direction d (tile_face_at's order).
+struct SweepPart {
+    int64_t t0;
+    int32_t first, count, d;
+};
+
+struct SweepArgs {
+    GridArgs g;
+    DirArgs dir[3];
+    SweepPart part[3];
+    int32_t nparts, tiles;
+    unsigned *nexact;                  // length of the exact path's list (zeroed beforehand)
     unsigned long long *exact_count;   // adds the exact-path reconstructions, or nullptr
+    SweepBuf buf;
     FastK FK;
     Consts K;
 };
+
+// Shape of direction D's tiles: the 2^tps pencils (at most 4) that leave the
+// fewest lanes without a face, weighed with the cells a tile stages (12 FP64
+// instructions per 32 of them beside some 690 for the faces).  Lines of 65
+// faces: 3 tiles a line of 1 x 32, 2.25 of 4 x 8.
+inline void tile_shape(DirArgs &d, int64_t faces, int64_t pencils, int H)
+{
+    double best = 0.0;
+    for (int tps = 0; tps <= 2; tps++) {
+        const int64_t tp = 1 << tps, tf = kTileFaces >> tps;
+        const int64_t lt = (faces + tf - 1) / tf, gr = (pencils + tp - 1) / tp;
+        const int64_t rounds = (tp * (tf + 2 * H - 1) + 31) / 32;
+        const double cost = (double)lt * (double)gr * (690.0 + 12.0 * (double)rounds);
+        if (tps == 0 || cost < best) {
+            best = cost;
+            d.tps = tps;
+            d.line_tiles = lt;
+            d.groups = gr;
+        }
+        if (pencils == 1) break;
+    }
+}
+
+// Tile t of direction D: first face f0 and the position of its first pencil.  x
+// runs fastest in the y and z sweeps: neighbouring pencils share the sectors of
+// their strided loads.
+template <int ND, int D>
+__device__ __forceinline__ void tile_at(const int64_t (&n)[3], const DirArgs &da, int64_t t,
+                                        int64_t &f0, int64_t &x, int64_t &y, int64_t &z)
+{
+    x = y = z = 0;
+    int64_t ft = t;
+    if (ND > 1) {
+        const int64_t fast = D == 0 ? da.line_tiles : da.groups;
+        const int64_t r = t / fast, i = t - r * fast;
+        if (D == 0) {
+            ft = i;
+            z = ND == 2 ? 0 : r / da.groups;
+            y = (r - z * da.groups) << da.tps;
+        } else {
+            x = i << da.tps;
+            const int64_t o = ND == 2 ? 0 : r / da.line_tiles;
+            ft = r - o * da.line_tiles;
+            if (D == 1) z = o;
+            else y = o;
+        }
+    }
+    f0 = ft * (kTileFaces >> da.tps);
+}
+
+// The lane's face within its tile: pencil p and offset fo along D.
+template <int D>
+__device__ __forceinline__ void tile_lane(int tps, int lane, int &p, int &fo)
+{
+    if (D == 0) {
+        fo = lane & ((kTileFaces >> tps) - 1);
+        p = lane >> (5 - tps);
+    } else {
+        p = lane & ((1 << tps) - 1);
+        fo = lane >> tps;
+    }
+}
+
+// Index of face f of the pencil at (x, y, z) in direction D's face grid.
+template <int D>
+__device__ __forceinline__ int64_t face_index(const int64_t (&n)[3], int64_t f, int64_t x, int64_t y,
+                                              int64_t z)
+{
+    if (D == 0) return f + (n[0] + 1) * (y + n[1] * z);
+    if (D == 1) return x + n[0] * (f + (n[1] + 1) * z);
+    return x + n[0] * (y + n[1] * f);
+}
 
 // App. A ghost-cell rules along one axis.  Returns the interior cell whose
 // state defines the (possibly ghost) cell j, and the rule to apply to it:
@@ -122,54 +278,26 @@ __device__ __forceinline__ void apply_ghost_rule(double (&Uc)[ND + 2], int rule,
     }
 }
 
-template <int ND>
-struct SmemLayout {
-    static constexpr int nc = ND + 2;
-    static constexpr int QU = 0, QF = nc, QV = 2 * nc;           // U, F, velocity
-    static constexpr int QH = QV + ND, QSR = QH + 1, QC = QH + 2;  // enthalpy, sqrt(rho), c
-    static constexpr int QLM = QH + 3, QL0 = QLM + 1, QLP = QLM + 2, QLR = QLM + 3;
-    static constexpr int NQ = QLR + 1;
-};
-
-// Tile of the sweeps: TP pencils x TF faces along the sweep, the exact-path
-// queue's capacity in reconstructions per thread (QCAP) and the blocks per SM
-// the register allocation is bounded for (MINB).  A single line (1D) uses
-// 1 x 128.  Measured on GB300 with 128-thread blocks:
-//   3D 256^3: TENO10 at three blocks per SM (164 registers, about 60 KB of
-//   shared memory each) beats two by 8-9 % and four by 6 %; TENO8 at four
-//   (128 registers) beats three by 2 %; with face n of periodic
-//   lines left out (256 faces per line), 4 x 32 beats 8 x 16 and 16 x 8 by
-//   0.5 % and 3 % (TENO10) and stages fewer halo cells per face;
-//   2D 512^2 TENO8: 4 x 32 ahead of 8 x 16 by 4 %, a register bound (three
-//   or four blocks per SM) ahead of an unbounded allocation by 3 %.
-// TENO_FACE_TP/TF/QCAP/MINB, when defined, override every case (tuning).
+// A sweeping warp's slice of shared memory, in doubles: the halved (U_c, F_c)
+// pairs of the staged cells, [c][cell], then the quantities that the Roe
+// average and the splitting speeds need, [row][cell].
 template <int ND, int H>
-struct FaceTile {
-#ifdef TENO_FACE_TP
-    static constexpr int TP = ND == 1 ? 1 : TENO_FACE_TP;
-    static constexpr int TF = ND == 1 ? 128 : TENO_FACE_TF;
-    static constexpr int QCAP = TENO_FACE_QCAP;
-    static constexpr int MINB = TENO_FACE_MINB;
-#else
-    static constexpr int TP = ND == 1 ? 1 : 4;
-    static constexpr int TF = ND == 1 ? 128 : 32;
-    // 2D ten-point: four queue entries per thread still fit three blocks per
-    // SM (73 KB each); noise plateaus hold about eight decided, non-S_p
-    // reconstructions per thread, which otherwise diverge when done in place
-    static constexpr int QCAP = (ND == 2 && H == 5) ? 4 : 2;
-    static constexpr int MINB = ND >= 2 ? (H == 4 ? 4 : 3) : 1;
-#endif
+struct FaceSmem {
+    static constexpr int nc = ND + 2;
+    static constexpr int NS = 4 * (kTileFaces / 4 + 2 * H - 1);    // cells of the widest shape
+    static constexpr int QV = 0, QH = ND, QSR = ND + 1;           // rows of the second part
+    static constexpr int QLM = ND + 2, QL0 = ND + 3, QLP = ND + 4, QLR = ND + 5, NT = ND + 6;
+    static constexpr int TMP = 2 * nc * NS;
+    static constexpr int TOTAL = (TMP + NT * NS + 1) & ~1;         // 16-byte slices
 };
 
-template <int ND, int H, int TP, int TF>
-constexpr size_t face_smem_bytes()
+// x / 2 on the exponent bits (no FP64 operation): exact where x / 2 is normal,
+// and for zeros; anything else takes the multiplication.
+__device__ __forceinline__ double half_of(double x)
 {
-    // staged cells + exact-path queue (values, owners) + per-thread results
-    return sizeof(double) * (size_t)SmemLayout<ND>::NQ * (TF + 2 * H - 1) * TP +
-           sizeof(double) * (size_t)(FaceTile<ND, H>::QCAP * TP * TF) * (2 * H) +
-           sizeof(double) * (size_t)(TP * TF) * 2 * (ND + 2) +
-           sizeof(int) * (size_t)(FaceTile<ND, H>::QCAP * TP * TF) +
-           (size_t)(TP * TF) * 2 * (ND + 2);
+    const unsigned hi = (unsigned)__double2hiint(x), e = hi & 0x7ff00000u;
+    if (e - 0x00200000u > 0x7fe00000u - 0x00200000u && __double_as_longlong(x) << 1) return x * 0.5;
+    return __hiloint2double((int)(e ? hi - 0x00100000u : hi), __double2loint(x));
 }
 
 // Sweep modes, a compile-time choice so that each kernel holds only its own
@@ -177,320 +305,348 @@ constexpr size_t face_smem_bytes()
 // limrec), and one that applies recorded decisions (frozen, frozen_argmax).
 enum { kSweepPlain = 0, kSweepRecord = 1, kSweepFrozen = 2 };
 
-// One tile: faces f0 .. f0+TF-1 along D of the TP pencils starting at x0
-// (at y, z for the axes not swept); for D = 0 the pencils run along y instead,
-// starting at y (x0 unused).  Every thread of the block calls it; it
-// synchronises once after staging and returns with no barrier pending, so a
-// persistent caller must synchronise before reusing the shared tile.
-template <int ND, int H, int D, int TP, int TF, int MODE>
-__device__ __forceinline__ void face_block(const FaceArgs &a, int64_t f0, int64_t x0, int64_t y,
-                                           int64_t z, double *sm)
+// One tile by one warp: the faces from f0 along D of the pencils from (x, y, z);
+// tile: its index in the chunk's buffers; sm: the warp's slice.  Every lane of
+// the warp calls it; it returns with the warp in step, its values, queue and
+// Roe states in the buffers.
+template <int ND, int H, int D, int MODE>
+__device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da, const FastK &FK,
+                                           const Consts &K, const SweepBuf &B, int64_t f0, int64_t x,
+                                           int64_t y, int64_t z, int64_t tile, double *sm)
 {
-    using SL = SmemLayout<ND>;
-    constexpr int nc = ND + 2, last = nc - 1, W = 2 * H;
-    constexpr int NS = TF + 2 * H - 1;
-#define SQ(q, j, p) sm[((q) * NS + (j)) * TP + (p)]
+    using SL = FaceSmem<ND, H>;
+    constexpr int nc = ND + 2, last = nc - 1, W = 2 * H, NS = SL::NS;
+    const int lane = threadIdx.x & 31;
+    double2 *UF = (double2 *)sm;
+#define TMP(q, j) sm[SL::TMP + (q) * NS + (j)]
 
     const int64_t n0 = a.n[0], n1 = a.n[1], nD = a.n[D];
-    const int64_t pstart = (D == 0) ? y : x0;             // first pencil
-    const int64_t npen = (D == 0) ? n1 : n0;              // pencils along that axis
-    __shared__ int qcount[2];                  // queue lengths: exact path, decided
-    if (threadIdx.x < 2) qcount[threadIdx.x] = 0;
+    const int tps = ND == 1 ? 0 : da.tps, tp = 1 << tps;
+    const int nsf = (kTileFaces >> tps) + 2 * H - 1;   // cells of one pencil
+    const int64_t npen = D == 0 ? n1 - y : n0 - x;     // pencils from the first one on
+    const int64_t cstride = D == 0 ? 1 : (D == 1 ? n0 : n0 * n1);
 
-    // Stage cells f0-H .. f0+TF+H-2 along D.
-    for (int idx = threadIdx.x; idx < NS * TP; idx += TP * TF) {
-        const int j = idx / TP, p = idx % TP;
-        const int64_t pg = pstart + p;
-        if (pg >= npen) continue;
+    // Stage the cells from f0-H along D, pencil by pencil in the x sweep, pencils
+    // side by side in the others.
+    for (int idx = lane; idx < tp * nsf; idx += 32) {
+        int j, pp;
+        if (D == 0) {
+            pp = (idx >= nsf) + (idx >= 2 * nsf) + (idx >= 3 * nsf);
+            j = idx - pp * nsf;
+        } else {
+            pp = idx & (tp - 1);
+            j = idx >> tps;
+        }
+        if (pp >= npen) continue;
+        const int64_t px = D == 0 ? 0 : x + pp, py = D == 0 ? y + pp : y;
+        const int64_t cbase = px + n0 * ((D == 1 ? 0 : py) + n1 * (D == 2 ? 0 : z));
         int rule;
-        const int64_t gi = map_index(f0 - H + j, nD, H, a.bc_lo, a.bc_hi, rule);
+        const int64_t gi = map_index(f0 - H + j, nD, H, da.bc_lo, da.bc_hi, rule);
         double Uc[nc];
         CellQ<ND> q;
         if (rule >= 5) {
             // a neighbouring sub-domain's cell from the side's halo array,
             // [nc][H planes][cells of a plane, the other axes x fastest]
             const int64_t m = a.ncell / nD;
-            const int64_t sf = (D == 0) ? pg + n1 * z : (D == 1 ? pg + n0 * z : pg + n0 * y);
-            const double *hb = rule == 5 ? a.bcs_lo : a.bcs_hi;
+            const int64_t sf = (D == 0) ? py + n1 * z : (D == 1 ? px + n0 * z : px + n0 * y);
+            const double *hb = rule == 5 ? da.bcs_lo : da.bcs_hi;
             const int64_t ih = gi * m + sf;
             const bool ok = TENO_IN(a.st, ih, H * m);
 #pragma unroll
             for (int c = 0; c < nc; c++) Uc[c] = ok ? hb[(int64_t)c * H * m + ih] : 0.0;
-            cell_quantities<ND, D>(Uc, a.K, q);
+            cell_quantities<ND, D>(Uc, K, q);
         } else {
-            int64_t id;
-            if (D == 0) id = gi + n0 * (pg + n1 * z);
-            else if (D == 1) id = pg + n0 * (gi + n1 * z);
-            else id = pg + n0 * (y + n1 * gi);
+            const int64_t id = cbase + gi * cstride;
             const bool ok = TENO_IN(a.st, id, a.ncell);
 #pragma unroll
             for (int c = 0; c < nc; c++) Uc[c] = ok ? a.U[c * a.ncell + id] : 0.0;
             if (!rule && a.P && ok) {
-                cell_from_prims<ND, D>(Uc, a.P, a.ncell, id, q);      // stored for this input
+                load_prims<ND>(a.P, a.ncell, id, q);      // stored for this input
             } else {
                 if (rule) {
                     // boundary-face index among the faces of this side (other axes, x fastest)
                     const int64_t m = a.ncell / nD;
-                    const int64_t sf = (D == 0) ? pg + n1 * z : (D == 1 ? pg + n0 * z : pg + n0 * y);
+                    const int64_t sf = (D == 0) ? py + n1 * z : (D == 1 ? px + n0 * z : px + n0 * y);
                     if (rule < 3 || TENO_IN(a.st, sf, m))
-                        apply_ghost_rule<ND, D>(Uc, rule, a.bcs_lo, a.bcs_hi, m, sf, a.K.gm1);
+                        apply_ghost_rule<ND, D>(Uc, rule, da.bcs_lo, da.bcs_hi, m, sf, K.gm1);
                 }
-                cell_quantities<ND, D>(Uc, a.K, q);
+                cell_quantities<ND, D>(Uc, K, q);
             }
         }
-        if (a.count_cells) {
+        if (D == 0 && a.count_cells) {
             // interior cells of this tile's own face range: each cell once
             const int64_t ci = f0 - H + j;
-            if (ci >= f0 && ci < f0 + TF && ci < nD && nonphysical_cell<ND>(Uc[0], q))
+            if (ci >= f0 && ci < f0 + (kTileFaces >> tps) && ci < nD && nonphysical_cell<ND>(Uc[0], q))
                 atomicAdd(&a.st->nonphys, 1ull);
         }
+        // halves of U and of the flux along D: each product and sum of
+        // cell_quantities' flux with one factor or both terms halved
+        double hU[nc], hF[nc];
 #pragma unroll
-        for (int c = 0; c < nc; c++) {
-            SQ(SL::QU + c, j, p) = 0.5 * q.U[c];
-            SQ(SL::QF + c, j, p) = 0.5 * q.F[c];
-        }
+        for (int c = 0; c < nc; c++) hU[c] = half_of(Uc[c]);
+        const double hp = half_of(q.p), hm = hU[1 + D];
+        hF[0] = hm;
 #pragma unroll
-        for (int k = 0; k < ND; k++) SQ(SL::QV + k, j, p) = q.u[k];
-        SQ(SL::QH, j, p) = q.H;
-        SQ(SL::QSR, j, p) = q.sr;
-        SQ(SL::QC, j, p) = q.c;
+        for (int k = 0; k < ND; k++) hF[1 + k] = k == D ? hm * q.u[k] + hp : hm * q.u[k];
+        hF[last] = q.u[D] * (hU[last] + hp);
+#pragma unroll
+        for (int c = 0; c < nc; c++) UF[c * NS + idx] = make_double2(hU[c], hF[c]);
+#pragma unroll
+        for (int k = 0; k < ND; k++) TMP(SL::QV + k, idx) = q.u[k];
+        TMP(SL::QH, idx) = q.H;
+        TMP(SL::QSR, idx) = q.sr;
         const double vd = q.u[D], cj = q.c;
-        SQ(SL::QLM, j, p) = fabs(vd - cj);
-        SQ(SL::QL0, j, p) = fabs(vd);
-        SQ(SL::QLP, j, p) = fabs(vd + cj);
-        SQ(SL::QLR, j, p) = fabs(vd) + cj;
+        TMP(SL::QLM, idx) = fabs(vd - cj);
+        TMP(SL::QL0, idx) = fabs(vd);
+        TMP(SL::QLP, idx) = fabs(vd + cj);
+        TMP(SL::QLR, idx) = fabs(vd) + cj;
     }
-    __syncthreads();
+    __syncwarp();
 
-    const int p = threadIdx.x % TP, fo = threadIdx.x / TP;
+    int p, fo;
+    tile_lane<D>(tps, lane, p, fo);
     const int64_t f = f0 + fo;
-    const bool active = !(f > nD - a.skip_last || pstart + p >= npen);
-    const int jl = fo + H - 1, jr = fo + H;           // cells i and i+1
-
-    // Queue of reconstructions whose value is not computed in line (values,
-    // owner), and per-thread result slots; after the staged cells.
-    // Entries [0, QE) hold reconstructions for the exact path, [QE, CAP)
-    // decided ones whose value is not the largest stencil's scheme (its
-    // decision byte already in the owner's Qfl slot).
-    constexpr int CAP = FaceTile<ND, H>::QCAP * TP * TF, QE = CAP / 4;
-    double *Qv = sm + (size_t)SL::NQ * NS * TP;       // [CAP][W]
-    double *Qres = Qv + (size_t)CAP * W;              // [threads][2 nc]: every value of the face
-    int *Qmeta = (int *)(Qres + (size_t)TP * TF * 2 * nc);   // [CAP]
-    uint8_t *Qfl = (uint8_t *)(Qmeta + CAP);          // [threads][2 nc]
+    const bool active = f <= nD - da.skip_last && p < npen;
+    // the lane's first cell, the step to the next, and cells i and i+1
+    const int b0 = D == 0 ? p * nsf + fo : lane, bs = D == 0 ? 1 : tp;
+    const int bl = b0 + (H - 1) * bs, br = bl + bs;
 
     RoeScalars<ND> rs;                 // eigenvector rows / columns are built from these
     double am = 0.0, a0 = 0.0, ap = 0.0, ar = 0.0;
     int64_t flin = 0;
+    const int64_t nf = B.nt * kTileFaces, cf = tile * kTileFaces + lane;   // in the buffers
     if (active) {
         // Roe average and eigenvectors (Sec. 5).
         double ul[ND], ur[ND];
 #pragma unroll
-        for (int k = 0; k < ND; k++) { ul[k] = SQ(SL::QV + k, jl, p); ur[k] = SQ(SL::QV + k, jr, p); }
-        const double c2 = roe_state<ND, D>(ul, SQ(SL::QH, jl, p), SQ(SL::QSR, jl, p), ur,
-                                           SQ(SL::QH, jr, p), SQ(SL::QSR, jr, p), a.K.gm1, rs);
+        for (int k = 0; k < ND; k++) { ul[k] = TMP(SL::QV + k, bl); ur[k] = TMP(SL::QV + k, br); }
+        const double c2 = roe_state<ND, D>(ul, TMP(SL::QH, bl), TMP(SL::QSR, bl), ur,
+                                           TMP(SL::QH, br), TMP(SL::QSR, br), K.gm1, rs);
         if (!(c2 > 0.0)) atomicAdd(&a.st->nonphys, 1ull);
-        if (D == 0) flin = f + (n0 + 1) * (pstart + p + n1 * z);
-        else if (D == 1) flin = pstart + p + n0 * (f + (n1 + 1) * z);
-        else flin = pstart + p + n0 * (y + n1 * f);
-        if (!TENO_IN(a.st, flin, a.nfaces)) flin = 0;        // debug build: counted, redirected
+        flin = face_index<D>(a.n, f, D == 0 ? x : x + p, D == 0 ? y + p : y, z);
+        if (!TENO_IN(a.st, flin, da.nfaces)) flin = 0;        // debug build: counted, redirected
+        // what the finish kernel needs
+#pragma unroll
+        for (int k = 0; k < ND; k++) B.RO[k * nf + cf] = rs.ut[k];
+        B.RO[ND * nf + cf] = rs.Ht;
+        B.RO[(ND + 1) * nf + cf] = rs.ct;
+        if (a.limiter) {
+#pragma unroll
+            for (int c = 0; c < nc; c++) {
+                const double2 cl = UF[c * NS + bl], cr = UF[c * NS + br];
+                B.RL[(4 * c) * nf + cf] = cl.x;
+                B.RL[(4 * c + 1) * nf + cf] = cl.y;
+                B.RL[(4 * c + 2) * nf + cf] = cr.x;
+                B.RL[(4 * c + 3) * nf + cf] = cr.y;
+            }
+            const double al = TMP(SL::QLR, bl), arr = TMP(SL::QLR, br);
+            B.RL[4 * nc * nf + cf] = arr > al ? arr : al;
+        }
         // Splitting speeds over the stencil (first maximum), or at recorded cells.
         if constexpr (MODE == kSweepFrozen) {
-            unsigned w = a.frozen_argmax[flin];
+            unsigned w = da.frozen_argmax[flin];
             if (!TENO_IN(a.st, (int)(w & 15), W) || !TENO_IN(a.st, (int)((w >> 4) & 15), W) ||
                 !TENO_IN(a.st, (int)((w >> 8) & 15), W) || !TENO_IN(a.st, (int)(w >> 12), W))
                 w = 0;
-            am = SQ(SL::QLM, fo + (int)(w & 15), p);
-            a0 = SQ(SL::QL0, fo + (int)((w >> 4) & 15), p);
-            ap = SQ(SL::QLP, fo + (int)((w >> 8) & 15), p);
-            ar = SQ(SL::QLR, fo + (int)((w >> 12) & 15), p);
+            am = TMP(SL::QLM, b0 + (int)(w & 15) * bs);
+            a0 = TMP(SL::QL0, b0 + (int)((w >> 4) & 15) * bs);
+            ap = TMP(SL::QLP, b0 + (int)((w >> 8) & 15) * bs);
+            ar = TMP(SL::QLR, b0 + (int)((w >> 12) & 15) * bs);
         } else {
             int jm = 0, j0 = 0, jp = 0, jr_ = 0;
 #pragma unroll
             for (int j = 0; j < W; j++) {
-                const double em = SQ(SL::QLM, fo + j, p), e0 = SQ(SL::QL0, fo + j, p);
-                const double ep = SQ(SL::QLP, fo + j, p), er = SQ(SL::QLR, fo + j, p);
+                const double em = TMP(SL::QLM, b0 + j * bs), e0 = TMP(SL::QL0, b0 + j * bs);
+                const double ep = TMP(SL::QLP, b0 + j * bs), er = TMP(SL::QLR, b0 + j * bs);
                 if (j == 0 || speed_gt(em, am)) { am = em; jm = j; }
                 if (j == 0 || speed_gt(e0, a0)) { a0 = e0; j0 = j; }
                 if (j == 0 || speed_gt(ep, ap)) { ap = ep; jp = j; }
                 if (j == 0 || speed_gt(er, ar)) { ar = er; jr_ = j; }
             }
             if constexpr (MODE == kSweepRecord)
-                a.argmax[flin] = (uint16_t)(jm | (j0 << 4) | (jp << 8) | (jr_ << 12));
+                da.argmax[flin] = (uint16_t)(jm | (j0 << 4) | (jp << 8) | (jr_ << 12));
         }
+        if (K.split) am = a0 = ap = ar;               // Rusanov: one speed for every field
     }
-
-    // Split-flux reconstructions of every field and sign: those the filter
-    // decides for the largest stencil now, the rest queued (or, if the queue
-    // is full, done in place) and drained once per tile by the whole block --
-    // the undecided ones with the exact path, the decided ones (fallback or a
-    // smaller stencil) with their value formula, so that neither diverges
-    // inside a warp.  Each value lands in the owner's Qres slot (shared
-    // memory, not registers: 2 nc values held there would stay live across
-    // the whole field loop and push the kernel into spills).
-    unsigned pending = 0;              // bit 2k+s: value comes from the queue
+    // Split-flux reconstructions of every field and sign.
+    const int64_t nq = B.nt * (64 * nc), q0 = tile * (64 * nc);
+    int cnt = 0;                                      // queue length (warp-uniform)
 #pragma unroll 1
     for (int k = 0; k < nc; k++) {
-        if (!active) break;
-        const bool shear = (k >= 2 && k < last);
-        const int tax = shear ? shear_axis<ND, D>(k) : 0;
-        double lrow[nc];
-        l_row<ND, D>(rs, k, lrow);
-        const double alpha = a.K.split ? ar : (k == 0 ? am : (k == last ? ap : a0));
-        // hw = w/2 = l.(U/2), hg = g/2 = l.(F/2) from the halved staged values:
-        // every product and sum is the unhalved one scaled by 1/2, exactly
-        double hw[W], hg[W];
+        double v[W], vm[W];                       // v+ and v-, in stencil order
+        if (active) {
+            const bool shear = (k >= 2 && k < last);
+            const int tax = shear ? shear_axis<ND, D>(k) : 0;
+            double lrow[nc];
+            l_row<ND, D>(rs, k, lrow);
+            const double alpha = k == 0 ? am : (k == last ? ap : a0);
+            // hw = w/2 = l.(U/2), hg = g/2 = l.(F/2) from the halved staged values:
+            // every product and sum is the unhalved one scaled by 1/2, exactly.
+            // f+ on offsets m -> cell i+m; f- mirrored: offset m -> cell i+1-m;
+            // v = (g +- alpha w)/2 = fma(+-alpha, w/2, g/2), rounded once.
 #pragma unroll
-        for (int j = 0; j < W; j++) {
-            double wv, gv;
-            if (shear) {
-                wv = SQ(SL::QU + 1 + tax, fo + j, p) + lrow[0] * SQ(SL::QU, fo + j, p);
-                gv = SQ(SL::QF + 1 + tax, fo + j, p) + lrow[0] * SQ(SL::QF, fo + j, p);
-            } else {
-                wv = lrow[0] * SQ(SL::QU, fo + j, p);
-                gv = lrow[0] * SQ(SL::QF, fo + j, p);
+            for (int j = 0; j < W; j++) {
+                double wv, gv;
+                const double2 c0 = UF[b0 + j * bs];
+                if (shear) {
+                    const double2 ct = UF[(1 + tax) * NS + b0 + j * bs];
+                    wv = ct.x + lrow[0] * c0.x;
+                    gv = ct.y + lrow[0] * c0.y;
+                } else {
+                    wv = lrow[0] * c0.x;
+                    gv = lrow[0] * c0.y;
 #pragma unroll
-                for (int c = 1; c < nc; c++) {
-                    wv = fma(lrow[c], SQ(SL::QU + c, fo + j, p), wv);
-                    gv = fma(lrow[c], SQ(SL::QF + c, fo + j, p), gv);
+                    for (int c = 1; c < nc; c++) {
+                        const double2 cc = UF[c * NS + b0 + j * bs];
+                        wv = fma(lrow[c], cc.x, wv);
+                        gv = fma(lrow[c], cc.y, gv);
+                    }
                 }
+                v[j] = fma(alpha, wv, gv);
+                vm[W - 1 - j] = fma(-alpha, wv, gv);
             }
-            hw[j] = wv;
-            hg[j] = gv;
         }
 #pragma unroll 1
         for (int s = 0; s < 2; s++) {
-            // f+ on offsets m -> cell i+m; f- mirrored: offset m -> cell i+1-m.
-            // v = (g +- alpha w)/2 = fma(+-alpha, w/2, g/2), rounded once.
-            const double sa = s ? -alpha : alpha;
-            double v[W];
-#pragma unroll
-            for (int kk = 0; kk < W; kk++) {
-                const double wk = s ? hw[W - 1 - kk] : hw[kk];
-                const double gk = s ? hg[W - 1 - kk] : hg[kk];
-                v[kk] = fma(sa, wk, gk);
-            }
-            double val = 0.0;
-            uint8_t fl = 0;
-            bool done = true;
-            if constexpr (MODE == kSweepFrozen) {
-                fl = a.frozen[(flin * nc + k) * 2 + s];
-                val = frozen_recon<H>(v, fl);
-            } else {
-                double sh[W];
-#pragma unroll
-                for (int kk = 0; kk < W; kk++) sh[kk] = v[kk] - v[H - 1];
-                const bool dec = a.fast && fast_decide<H>(v, sh, a.FK, fl,
-                                                          MODE == kSweepRecord && a.need_ct != 0);
-                // the largest stencil accepted (S6 as bits 0-4 zero).  Kept
-                // inline: the same test through a helper function made the 8-
-                // and 10-point sweeps 4-14 % slower (same registers, other code).
-                if (dec && (H == 6 ? (fl & 31) == 0 : (fl & 3) == H - 2)) {
-                    val = flux_large<H, H>(v);
+            const int slot = (2 * k + s) * kTileFaces + lane;
+            bool open = false;
+            if (active) {
+                double *r = B.R + (2 * k + s) * nf + cf;
+                if constexpr (MODE == kSweepFrozen) {
+                    *r = frozen_recon<H>(v, da.frozen[(flin * nc + k) * 2 + s]);
                 } else {
-                    int q = atomicAdd(&qcount[dec ? 1 : 0], 1);
-                    const bool room = (dec ? (q < CAP - QE) : (q < QE)) &&
-                                      TENO_IN(a.st, q + (dec ? QE : 0), CAP);
-                    if (room) {
-                        if (dec) {
-                            q += QE;
-                            Qfl[threadIdx.x * (2 * nc) + 2 * k + s] = fl;
-                        }
-#pragma unroll
-                        for (int kk = 0; kk < W; kk++) Qv[(size_t)q * W + kk] = v[kk];
-                        Qmeta[q] = (threadIdx.x << 4) | (2 * k + s);
-                        pending |= 1u << (2 * k + s);
-                        done = false;
-                    } else {                                   // queue full: in place
-                        val = dec ? decided_value<H>(v, fl) : teno_recon<H>(v, a.K, fl);
+                    open = !(a.fast && !(MODE == kSweepRecord && a.need_ct) && quick_large<H>(v, FK));
+                    if (!open) {
+                        *r = flux_large<H, H>(v);
+                        if constexpr (MODE == kSweepRecord)
+                            B.RD[(2 * k + s) * nf + cf] = (uint8_t)large_code(H);
                     }
                 }
             }
-            if (done) {
-                Qres[threadIdx.x * (2 * nc) + 2 * k + s] = val;
-                if constexpr (MODE == kSweepRecord) a.flags[(flin * nc + k) * 2 + s] = fl;
-            }
-        }
-    }
-    if constexpr (MODE != kSweepFrozen) {
-        __syncthreads();
-        const int ne = min(qcount[0], QE), nd = min(qcount[1], CAP - QE);
-        if (a.exact_count && threadIdx.x == 0 && qcount[0] > 0)
-            atomicAdd(a.exact_count, (unsigned long long)qcount[0]);
-        for (int q = threadIdx.x; q < ne; q += TP * TF) {
-            double v[W];
+            if constexpr (MODE != kSweepFrozen) {
+                const unsigned m = __ballot_sync(0xffffffffu, open);
+                const int64_t q = q0 + cnt + __popc(m & ((1u << lane) - 1u));
+                if (open && TENO_IN(a.st, q, nq)) {
 #pragma unroll
-            for (int kk = 0; kk < W; kk++) v[kk] = Qv[(size_t)q * W + kk];
-            uint8_t fl;
-            const double r = teno_recon<H>(v, a.K, fl);
-            const int meta = Qmeta[q];
-            const int slot = (meta >> 4) * (2 * nc) + (meta & 15);
-            if (TENO_IN(a.st, slot, TP * TF * 2 * nc)) {
-                Qres[slot] = r;
-                Qfl[slot] = fl;
-            }
-        }
-        for (int q = QE + threadIdx.x; q < QE + nd; q += TP * TF) {
-            double v[W];
-#pragma unroll
-            for (int kk = 0; kk < W; kk++) v[kk] = Qv[(size_t)q * W + kk];
-            const int meta = Qmeta[q];
-            const int slot = (meta >> 4) * (2 * nc) + (meta & 15);
-            if (TENO_IN(a.st, slot, TP * TF * 2 * nc)) Qres[slot] = decided_value<H>(v, Qfl[slot]);
-        }
-        __syncthreads();
-        if constexpr (MODE == kSweepRecord) {
-            if (active && pending) {
-#pragma unroll
-                for (int q = 0; q < 2 * nc; q++) {
-                    if (pending & (1u << q))
-                        a.flags[(flin * nc + (q >> 1)) * 2 + (q & 1)] = Qfl[threadIdx.x * (2 * nc) + q];
+                    for (int kk = 0; kk < W; kk++) B.qv[kk * nq + q] = v[kk];
+                    B.qslot[q] = (uint16_t)slot;
                 }
+                cnt += __popc(m);
             }
+#pragma unroll
+            for (int kk = 0; kk < W; kk++) v[kk] = vm[kk];
         }
     }
+    if (MODE != kSweepFrozen && lane == 0) B.count[tile] = (uint32_t)cnt | a.tag;
+    __syncwarp();
+#undef TMP
+}
 
-    // Back-projection F = sum_k r_k (f+_k + f-_k), fields ascending; the zero
-    // and unit entries of the shear columns are skipped.
+// |x| in FP32, rounded up; infinity for what FP32 does not hold and for NaN.
+__device__ __forceinline__ float abs_up(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, e = hi >> 20;
+    if (e < 897u) return 1.17549435e-38f;
+    if (e > 1149u) return INFINITY;
+    return __uint_as_float((__funnelshift_l((unsigned)__double2loint(x), hi, 3) - (896u << 23)) + 1u);
+}
+
+// True only if the positivity limiter certainly leaves this flux as it is.  Both
+// one-sided updates U_i -+ 2 lam (F - F_i) with the whole flux are formed
+// (halved); the limiter's own come from the same terms by way of the
+// Lax-Friedrichs flux, so each component of theirs is within 2^-49 of S_c, the
+// sum of the sizes of all terms.  Density and rho p above 1e-13 times
+// those sizes (and the limiter's eps) therefore pass its tests too, with
+// theta = 1.  Some 34 FP64 instructions where the limiter's own test takes
+// about 215 (3D Noh, 64^3: 0.46 ms a stage for the finish kernel).
+template <int ND>
+__device__ __forceinline__ bool limiter_calm(const double (&Fo)[ND + 2], double lam, const Consts &K,
+                                             const SweepBuf &B, int64_t nf, int64_t cf)
+{
+    constexpr int nc = ND + 2, last = nc - 1;
+    const float af = abs_up(B.RL[4 * nc * nf + cf]), lf = abs_up(lam);
+    double ul[nc], ur[nc];
+    float S[nc];
+#pragma unroll
+    for (int c = 0; c < nc; c++) {
+        const double hUl = B.RL[(4 * c) * nf + cf], hFl = B.RL[(4 * c + 1) * nf + cf];
+        const double hUr = B.RL[(4 * c + 2) * nf + cf], hFr = B.RL[(4 * c + 3) * nf + cf];
+        ul[c] = fma(-lam, fma(-2.0, hFl, Fo[c]), hUl);
+        ur[c] = fma(lam, fma(-2.0, hFr, Fo[c]), hUr);
+        const float u = abs_up(hUl) + abs_up(hUr);
+        S[c] = u + lf * (abs_up(Fo[c]) + 2.0f * (abs_up(hFl) + abs_up(hFr)) + 2.0f * af * u);
+    }
+    float k = 2.0f * S[last] * S[0];
+#pragma unroll
+    for (int a = 0; a < ND; a++) k = fmaf(S[1 + a], S[1 + a], k);
+    const double rho_min = (double)(1.0e-13f * S[0]) + K.lim_eps;
+    const double q_min = K.gm1 * (double)(1.0e-13f * k), e2 = 2.0 * K.lim_eps;
+    bool calm = isfinite(k);
+#pragma unroll
+    for (int side = 0; side < 2; side++) {
+        const double(&u)[nc] = side ? ur : ul;
+        double q = -(u[1] * u[1]);                     // rho p / (2 (gamma - 1))
+#pragma unroll
+        for (int a = 1; a < ND; a++) q = fma(-u[1 + a], u[1 + a], q);
+        q = fma(2.0 * u[last], u[0], q);
+        calm = calm && u[0] > rho_min && K.gm1 * q > fma(e2, u[0], q_min);
+    }
+    return calm;
+}
+
+// Back-projection of a face, the limiter, and what it leaves: the flux, the
+// limiter's byte and the decision bytes of the record.
+template <int ND, int D, int MODE>
+__device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, const Consts &K,
+                                            const SweepBuf &B, int64_t cf, int64_t flin, Status *st)
+{
+    constexpr int nc = ND + 2, last = nc - 1;
+    const int64_t nf = B.nt * kTileFaces;
+    if (!TENO_IN(st, flin, da.nfaces)) return;
+    RoeScalars<ND> rs;                 // the entries r_entry reads, as roe_state forms them
+#pragma unroll
+    for (int k = 0; k < ND; k++) rs.ut[k] = B.RO[k * nf + cf];
+    rs.Ht = B.RO[ND * nf + cf];
+    rs.ct = B.RO[(ND + 1) * nf + cf];
+    rs.q2 = rs.ut[0] * rs.ut[0];
+#pragma unroll
+    for (int k = 1; k < ND; k++) rs.q2 = fma(rs.ut[k], rs.ut[k], rs.q2);
+    rs.unct = rs.ut[D] * rs.ct;
+    // F = sum_k r_k (f+_k + f-_k), fields ascending; the zero and unit entries
+    // of the shear columns are skipped.
     double Fo[nc];
-    if (active) {
 #pragma unroll
-        for (int k = 0; k < nc; k++) {
-            const double hsum = Qres[threadIdx.x * (2 * nc) + 2 * k] + Qres[threadIdx.x * (2 * nc) + 2 * k + 1];
-            if (k == 0) {
+    for (int k = 0; k < nc; k++) {
+        const double hsum = B.R[(2 * k) * nf + cf] + B.R[(2 * k + 1) * nf + cf];
+        if (k == 0) {
 #pragma unroll
-                for (int c = 0; c < nc; c++) Fo[c] = r_entry<ND, D>(rs, c, 0) * hsum;
-            } else if (k >= 2 && k < last) {
-                int tax = 0, kk = 2;
+            for (int c = 0; c < nc; c++) Fo[c] = r_entry<ND, D>(rs, c, 0) * hsum;
+        } else if (k >= 2 && k < last) {
+            const int tax = shear_axis<ND, D>(k);
 #pragma unroll
-                for (int aa = 0; aa < ND; aa++) {
-                    if (aa == D) continue;
-                    if (kk == k) tax = aa;
-                    kk++;
-                }
-                Fo[1 + tax] = Fo[1 + tax] + hsum;
-                Fo[last] = fma(r_entry<ND, D>(rs, last, k), hsum, Fo[last]);
-            } else {
+            for (int aa = 0; aa < ND; aa++)
+                if (aa == tax) Fo[1 + aa] = Fo[1 + aa] + hsum;
+            Fo[last] = fma(r_entry<ND, D>(rs, last, k), hsum, Fo[last]);
+        } else {
 #pragma unroll
-                for (int c = 0; c < nc; c++) Fo[c] = fma(r_entry<ND, D>(rs, c, k), hsum, Fo[c]);
-            }
+            for (int c = 0; c < nc; c++) Fo[c] = fma(r_entry<ND, D>(rs, c, k), hsum, Fo[c]);
         }
     }
-    if (!active) return;
 
-    if (a.K.limiter) {
+    if (limiter && limiter_calm<ND>(Fo, *da.lam, K, B, nf, cf)) {
+        if constexpr (MODE == kSweepRecord) da.limrec[flin] = 0;
+    } else if (limiter) {
         // Positivity-preserving flux limiter (cited in Sec. 5.3): blend toward
         // the Lax-Friedrichs flux so that the one-sided half updates of cells i
         // and i+1 keep rho >= eps and p >= eps.
-        const double eps = a.K.lim_eps, lam2 = 2.0 * (*a.lam);
-        const double al = SQ(SL::QLR, jl, p), arr = SQ(SL::QLR, jr, p);
-        const double af = arr > al ? arr : al;
+        const double eps = K.lim_eps, lam2 = 2.0 * (*da.lam), af = B.RL[4 * nc * nf + cf];
         double FL[nc], dF[nc], UL[nc], UR[nc], dUL[nc], dUR[nc];
 #pragma unroll
         for (int c = 0; c < nc; c++) {
             // staged halves: FL = (F_l + F_r)/2 - af (U_r - U_l)/2 exactly as
             // ((F_l + F_r) - af (U_r - U_l)) / 2
-            const double hUl = SQ(SL::QU + c, jl, p), hUr = SQ(SL::QU + c, jr, p);
-            const double hFl = SQ(SL::QF + c, jl, p), hFr = SQ(SL::QF + c, jr, p);
+            const double hUl = B.RL[(4 * c) * nf + cf], hFl = B.RL[(4 * c + 1) * nf + cf];
+            const double hUr = B.RL[(4 * c + 2) * nf + cf], hFr = B.RL[(4 * c + 3) * nf + cf];
             const double Ul = 2.0 * hUl, Ur = 2.0 * hUr, Fl = 2.0 * hFl, Fr = 2.0 * hFr;
             FL[c] = (hFl + hFr) - af * (hUr - hUl);
             dF[c] = Fo[c] - FL[c];
@@ -519,9 +675,9 @@ __device__ __forceinline__ void face_block(const FaceArgs &a, int64_t f0, int64_
                 Us[c] = side ? UR[c] : UL[c];
                 Ut[c] = Us[c] + th * (side ? dUR[c] : dUL[c]);
             }
-            const double pt = pressure_of<ND>(Ut, a.K.gm1);
+            const double pt = pressure_of<ND>(Ut, K.gm1);
             if (pt < eps) {
-                const double p0 = pressure_of<ND>(Us, a.K.gm1);
+                const double p0 = pressure_of<ND>(Us, K.gm1);
                 double t = th * ((p0 - eps) / (p0 - pt));
                 if (!(t > 0.0)) t = 0.0;
                 if (t < thp) thp = t;
@@ -531,63 +687,290 @@ __device__ __forceinline__ void face_block(const FaceArgs &a, int64_t f0, int64_
 #pragma unroll
             for (int c = 0; c < nc; c++) Fo[c] = FL[c] + thp * dF[c];
         }
-        if constexpr (MODE == kSweepRecord) a.limrec[flin] = thp < 1.0 ? 1 : 0;
+        if constexpr (MODE == kSweepRecord) da.limrec[flin] = thp < 1.0 ? 1 : 0;
     } else if constexpr (MODE == kSweepRecord) {
-        a.limrec[flin] = 0;
+        da.limrec[flin] = 0;
     }
 
+    if constexpr (MODE == kSweepRecord) {
 #pragma unroll
-    for (int c = 0; c < nc; c++) a.F[c * a.nfaces + flin] = Fo[c];
-#undef SQ
+        for (int q = 0; q < 2 * nc; q++) da.flags[flin * nc * 2 + q] = B.RD[q * nf + cf];
+    }
+#pragma unroll
+    for (int c = 0; c < nc; c++) da.F[c * da.nfaces + flin] = Fo[c];
 }
 
-template <int ND, int H, int D, int TP, int TF, int MODE>
-__global__ void __launch_bounds__(TP * TF, FaceTile<ND, H>::MINB) face_kernel(FaceArgs a)
+// Warps per block of the sweep (pencils side by side in the y and z sweeps) and
+// the blocks per SM that its registers are bounded for.
+constexpr int kSweepWarps = 4;
+template <int H>
+constexpr int kSweepBlocks = 4;
+
+template <int ND, int H, int MODE>
+__global__ void __launch_bounds__(32 * kSweepWarps, kSweepBlocks<H>) sweep_kernel(const SweepArgs a)
 {
     extern __shared__ double sm[];
-    int64_t x0 = 0, y = 0, z = 0, f0;
-    if (D == 0) { f0 = (int64_t)blockIdx.x * TF; y = (int64_t)blockIdx.y * TP; z = blockIdx.z; }
-    else if (D == 1) { x0 = (int64_t)blockIdx.x * TP; f0 = (int64_t)blockIdx.y * TF; z = blockIdx.z; }
-    else { f0 = (int64_t)blockIdx.x * TF; x0 = (int64_t)blockIdx.y * TP; y = blockIdx.z; }
-    face_block<ND, H, D, TP, TF, MODE>(a, f0, x0, y, z, sm);
+    const int w = threadIdx.x >> 5;
+    const int32_t tile = (int32_t)blockIdx.x * kSweepWarps + w;
+    if (tile >= a.tiles) return;
+    double *slice = sm + (size_t)w * FaceSmem<ND, H>::TOTAL;
+    int i = 0;
+    while (i + 1 < a.nparts && tile >= a.part[i + 1].first) i++;
+    const int64_t t = a.part[i].t0 + (tile - a.part[i].first);
+    const int d = a.part[i].d;
+    int64_t f0, x, y, z;
+    if (d == 0) {
+        tile_at<ND, 0>(a.g.n, a.dir[0], t, f0, x, y, z);
+        sweep_tile<ND, H, 0, MODE>(a.g, a.dir[0], a.FK, a.K, a.buf, f0, x, y, z, tile, slice);
+    }
+    if constexpr (ND >= 2) {
+        if (d == 1) {
+            tile_at<ND, 1>(a.g.n, a.dir[1], t, f0, x, y, z);
+            sweep_tile<ND, H, 1, MODE>(a.g, a.dir[1], a.FK, a.K, a.buf, f0, x, y, z, tile, slice);
+        }
+    }
+    if constexpr (ND >= 3) {
+        if (d == 2) {
+            tile_at<ND, 2>(a.g.n, a.dir[2], t, f0, x, y, z);
+            sweep_tile<ND, H, 2, MODE>(a.g, a.dir[2], a.FK, a.K, a.buf, f0, x, y, z, tile, slice);
+        }
+    }
 }
 
-template <int ND, int H, int D, int MODE>
-cudaError_t launch_face_mode(const FaceArgs &a, dim3 grid, cudaStream_t s)
+// The queued reconstructions of `group` consecutive tiles, by `split` warps that
+// take every split-th round of 32 entries.  A round takes one entry per lane
+// through the filter; its outcomes gather by kind in shared memory, and a
+// kind's values are evaluated when it has a warp's worth, the rest at the end.
+// Few tiles per warp and split > 1 shorten a small evaluation, many fill the
+// lanes of a large one.  RECORD: decision bytes are kept.  mixed: 0, or in a
+// batch of both schemes 1 for the tiles whose length has no top bit, 2 for
+// those that have it.
+constexpr int kDecideWarps = 4, kDecideMostTiles = 16;
+
+template <int H, bool RECORD>
+__device__ __forceinline__ void decided_out(const SweepBuf &B, int64_t nq, int64_t nf, uint32_t per,
+                                            bool fallback, uint32_t q, uint8_t f, int nc, Status *st)
 {
-    constexpr int TP = FaceTile<ND, H>::TP;
-    constexpr int TF = FaceTile<ND, H>::TF;
-    constexpr size_t smem = face_smem_bytes<ND, H, TP, TF>();
+    constexpr int W = 2 * H;
+    double v[W];
+#pragma unroll
+    for (int kk = 0; kk < W; kk++) v[kk] = B.qv[kk * nq + q];
+    const int slot = B.qslot[q];
+    const int64_t o = (slot >> 5) * nf + (int64_t)(q / per) * kTileFaces + (slot & 31);
+    if (!TENO_IN(st, o, 2 * nc * nf)) return;
+    if (fallback) B.R[o] = fallback_value<H>(v, (f >> 2) & 7);
+    else B.R[o] = large_value<H>(v, H == 6 && (f & 31) == 0 ? 6 : (f & 3) + 2);
+    if (RECORD) B.RD[o] = f;
+}
+
+template <int H, bool RECORD>
+__global__ void __launch_bounds__(32 * kDecideWarps, 6) decide_kernel(
+    const SweepBuf B, int32_t tiles, int group, int split, int nc, int fast, int need_ct, int mixed,
+    unsigned *nexact, const FastK FK, Status *st)
+{
+    constexpr int W = 2 * H;
+    __shared__ uint32_t list_[kDecideWarps][2][64];    // gathered entries: large stencil, fallback
+    __shared__ uint8_t code_[kDecideWarps][2][64];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t(*list)[64] = list_[warp];
+    uint8_t(*code)[64] = code_[warp];
+    const int64_t unit = (int64_t)blockIdx.x * kDecideWarps + warp;
+    const int64_t t0 = unit / split * group;
+    if (t0 >= tiles) return;
+    const uint32_t per = 64u * nc;
+    const int64_t nq = B.nt * per, nf = B.nt * kTileFaces;
+    // entries before each tile of the group: lane i holds tile i's
+    int before = 0, total;
+    {
+        uint32_t c = lane < group && t0 + lane < tiles ? B.count[t0 + lane] : 0u;
+        if (mixed && (c >> 31) != (uint32_t)(mixed == 2)) c = 0u;
+        int sum = (int)(c & 0x7fffffffu);
+        const int own = sum;
+#pragma unroll
+        for (int o = 1; o < kDecideMostTiles; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += u;
+        }
+        before = sum - own;
+        total = __shfl_sync(0xffffffffu, sum, kDecideMostTiles - 1);
+    }
+    int n0 = 0, n1 = 0;                                // gathered, per kind (warp-uniform)
+    for (int base = (int)(unit % split) * 32; base < total; base += 32 * split) {
+        const int e = base + lane;
+        int i = 0;
+#pragma unroll
+        for (int b = kDecideMostTiles / 2; b > 0; b >>= 1) {
+            const int f = __shfl_sync(0xffffffffu, before, i + b);
+            if (i + b < group && e >= f) i += b;
+        }
+        const uint32_t q = (uint32_t)((t0 + i) * per) + (uint32_t)(e - __shfl_sync(0xffffffffu, before, i));
+        int kind = -1;                                 // 0 large stencil, 1 fallback, 2 exact path
+        uint8_t fl = 0;
+        if (e < total) {
+            kind = 2;
+            if (fast && TENO_IN(st, q, nq)) {
+                double v[W];
+#pragma unroll
+                for (int kk = 0; kk < W; kk++) v[kk] = B.qv[kk * nq + q];
+                if (fast_decide<H>(v, FK, fl, need_ct != 0))
+                    kind = (fl & 3) != 0 || (H == 6 && (fl & 31) == 0) ? 0 : 1;
+            }
+        }
+        const unsigned below = (1u << lane) - 1u;
+        const unsigned m0 = __ballot_sync(0xffffffffu, kind == 0);
+        const unsigned m1 = __ballot_sync(0xffffffffu, kind == 1);
+        const unsigned m2 = __ballot_sync(0xffffffffu, kind == 2);
+        if (kind == 0 || kind == 1) {
+            const int at = kind ? n1 + __popc(m1 & below) : n0 + __popc(m0 & below);
+            list[kind][at] = q;
+            code[kind][at] = fl;
+        }
+        n0 += __popc(m0);
+        n1 += __popc(m1);
+        if (m2) {
+            int at = 0;
+            if (lane == 0) at = (int)atomicAdd(nexact, __popc(m2));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(m2 & below);
+            if (kind == 2 && TENO_IN(st, at, nq)) B.xlist[at] = q;
+        }
+        __syncwarp();
+        const bool end = base + 32 * split >= total;
+        if (n0 >= 32 || (end && n0 > 0)) {
+            const int n = min(n0, 32);
+            n0 -= n;
+            if (lane < n)
+                decided_out<H, RECORD>(B, nq, nf, per, false, list[0][n0 + lane], code[0][n0 + lane], nc, st);
+        }
+        if (n1 >= 32 || (end && n1 > 0)) {
+            const int n = min(n1, 32);
+            n1 -= n;
+            if (lane < n)
+                decided_out<H, RECORD>(B, nq, nf, per, true, list[1][n1 + lane], code[1][n1 + lane], nc, st);
+        }
+        __syncwarp();
+    }
+    // at most 31 of a kind are left after the last round's pass
+    if (lane < n0) decided_out<H, RECORD>(B, nq, nf, per, false, list[0][lane], code[0][lane], nc, st);
+    if (lane < n1) decided_out<H, RECORD>(B, nq, nf, per, true, list[1][lane], code[1][lane], nc, st);
+}
+
+// The listed reconstructions through the exact path.
+template <int H, bool RECORD>
+__global__ void __launch_bounds__(128) exact_kernel(SweepBuf B, int nc, const unsigned *nexact,
+                                                    unsigned long long *exact_count,
+                                                    const Consts K, Status *st)
+{
+    constexpr int W = 2 * H;
+    const int64_t per = 64 * nc, nq = B.nt * per, nf = B.nt * kTileFaces;
+    const unsigned n = *nexact;
+    if (exact_count && blockIdx.x == 0 && threadIdx.x == 0 && n)
+        atomicAdd(exact_count, (unsigned long long)n);
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint32_t q = B.xlist[i];
+        if (!TENO_IN(st, q, nq)) continue;
+        double v[W];
+#pragma unroll
+        for (int kk = 0; kk < W; kk++) v[kk] = B.qv[kk * nq + q];
+        const int slot = B.qslot[q];
+        const int64_t o = (slot >> 5) * nf + (int64_t)(q / (uint32_t)per) * kTileFaces + (slot & 31);
+        if (!TENO_IN(st, o, 2 * nc * nf)) continue;
+        uint8_t fl;
+        B.R[o] = teno_recon<H>(v, K, fl);
+        if (RECORD) B.RD[o] = fl;
+    }
+}
+
+template <int ND, int D, int MODE>
+__device__ __forceinline__ void finish_lane(const SweepArgs &a, int64_t t, int lane, int64_t cf)
+{
+    const DirArgs &da = a.dir[D];
+    int64_t f0, x, y, z;
+    int p, fo;
+    tile_at<ND, D>(a.g.n, da, t, f0, x, y, z);
+    tile_lane<D>(ND == 1 ? 0 : da.tps, lane, p, fo);
+    if (D == 0) y += p;
+    else x += p;
+    if (f0 + fo > a.g.n[D] - da.skip_last || x >= a.g.n[0] || y >= a.g.n[1]) return;
+    finish_face<ND, D, MODE>(da, a.g.limiter, a.K, a.buf, cf, face_index<D>(a.g.n, f0 + fo, x, y, z),
+                             a.g.st);
+}
+
+template <int ND, int MODE>
+__global__ void __launch_bounds__(128) finish_kernel(const SweepArgs a)
+{
+    const int32_t tile = (int32_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (tile >= a.tiles) return;
+    int i = 0;
+    while (i + 1 < a.nparts && tile >= a.part[i + 1].first) i++;
+    const int64_t t = a.part[i].t0 + (tile - a.part[i].first), cf = (int64_t)tile * kTileFaces + lane;
+    const int d = a.part[i].d;
+    if (d == 0) finish_lane<ND, 0, MODE>(a, t, lane, cf);
+    if constexpr (ND >= 2) {
+        if (d == 1) finish_lane<ND, 1, MODE>(a, t, lane, cf);
+    }
+    if constexpr (ND >= 3) {
+        if (d == 2) finish_lane<ND, 2, MODE>(a, t, lane, cf);
+    }
+}
+
+// The decide and exact kernels of one chunk.
+template <int H, bool RECORD>
+cudaError_t launch_decisions(const SweepBuf &B, int32_t tiles, int nc, int fast, int need_ct, int mixed,
+                             unsigned *nexact, unsigned long long *exact_count, const FastK &FK,
+                             const Consts &K, Status *st, cudaStream_t s)
+{
+    // warps enough to fill the chip (24 on each of 152 SMs) before tiles share one
+    const int64_t fill = 152 * 24;
+    int group = 1, split = 1;
+    while (group < kDecideMostTiles && tiles > fill * group) group *= 2;
+    while (group == 1 && split < 2 * nc && (int64_t)tiles * split * 2 <= fill) split *= 2;
+    const int64_t units = (int64_t)((tiles + group - 1) / group) * split;
+    decide_kernel<H, RECORD><<<(unsigned)((units + kDecideWarps - 1) / kDecideWarps), 32 * kDecideWarps, 0, s>>>(
+        B, tiles, group, split, nc, fast, need_ct, mixed, nexact, FK, st);
+    const int64_t most = (int64_t)tiles * nc / 2;         // blocks of 128 for every entry
+    exact_kernel<H, RECORD><<<(unsigned)(most < 608 ? (most ? most : 1) : 608), 128, 0, s>>>(
+        B, nc, nexact, exact_count, K, st);
+    return cudaGetLastError();
+}
+
+template <int ND, int H, int MODE>
+cudaError_t launch_chunk_mode(const SweepArgs &a, cudaStream_t s)
+{
+    constexpr size_t smem = sizeof(double) * (size_t)FaceSmem<ND, H>::TOTAL * kSweepWarps;
     static bool attr_done = false;
     if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(face_kernel<ND, H, D, TP, TF, MODE>,
+        cudaError_t e = cudaFuncSetAttribute(sweep_kernel<ND, H, MODE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
-    face_kernel<ND, H, D, TP, TF, MODE><<<grid, TP * TF, smem, s>>>(a);
+    const unsigned blocks = (unsigned)((a.tiles + kSweepWarps - 1) / kSweepWarps);
+    sweep_kernel<ND, H, MODE><<<blocks, 32 * kSweepWarps, smem, s>>>(a);
+    if (MODE != kSweepFrozen) {
+        cudaError_t e = launch_decisions<H, MODE == kSweepRecord>(
+            a.buf, a.tiles, ND + 2, a.g.fast, a.g.need_ct, 0, a.nexact, a.exact_count, a.FK, a.K,
+            a.g.st, s);
+        if (e != cudaSuccess) return e;
+    }
+    finish_kernel<ND, MODE><<<(unsigned)((a.tiles + 3) / 4), 128, 0, s>>>(a);
     return cudaGetLastError();
 }
 
-// Host-side launch of one direction's sweep, in the mode its arguments ask
-// for (a decision record to write, recorded decisions to apply, or neither).
-template <int ND, int H, int D>
-cudaError_t launch_face(const FaceArgs &a, cudaStream_t s)
+// One chunk's fluxes, in the mode its arguments ask for (a decision record to
+// write, recorded decisions to apply, or neither).
+template <int ND, int H>
+cudaError_t launch_chunk(const SweepArgs &a, cudaStream_t s)
 {
-    constexpr int TP = FaceTile<ND, H>::TP;
-    constexpr int TF = FaceTile<ND, H>::TF;
-    if ((a.flags && a.frozen) || (a.flags && (!a.argmax || !a.limrec)) ||
-        (a.frozen && !a.frozen_argmax))
-        return cudaErrorInvalidValue;
-    dim3 grid;
-    const int64_t nf = a.n[D] + 1 - a.skip_last;    // faces computed along D
-    if (D == 0) grid = dim3((unsigned)((nf + TF - 1) / TF), (unsigned)((a.n[1] + TP - 1) / TP), (unsigned)a.n[2]);
-    else if (D == 1) grid = dim3((unsigned)((a.n[0] + TP - 1) / TP), (unsigned)((nf + TF - 1) / TF), (unsigned)a.n[2]);
-    else   // z tiles fastest: consecutive blocks share their halo planes through L2
-        grid = dim3((unsigned)((nf + TF - 1) / TF), (unsigned)((a.n[0] + TP - 1) / TP), (unsigned)a.n[1]);
-    if (a.flags) return launch_face_mode<ND, H, D, kSweepRecord>(a, grid, s);
-    if (a.frozen) return launch_face_mode<ND, H, D, kSweepFrozen>(a, grid, s);
-    return launch_face_mode<ND, H, D, kSweepPlain>(a, grid, s);
+    for (int i = 0; i < a.nparts; i++) {
+        const DirArgs &d = a.dir[a.part[i].d];
+        if ((d.flags && d.frozen) || (d.flags && (!d.argmax || !d.limrec)) ||
+            (d.frozen && !d.frozen_argmax))
+            return cudaErrorInvalidValue;
+    }
+    if (a.dir[0].flags) return launch_chunk_mode<ND, H, kSweepRecord>(a, s);
+    if (a.dir[0].frozen) return launch_chunk_mode<ND, H, kSweepFrozen>(a, s);
+    return launch_chunk_mode<ND, H, kSweepPlain>(a, s);
 }
 
 }  // namespace teno

@@ -1,19 +1,13 @@
-// Instantiations of the face sweep for the 10-point TENO-AA scheme.
+// Instantiations of the face-flux kernels for the 10-point TENO-AA scheme.
 #include "teno_face.cuh"
 
 namespace teno {
 
-cudaError_t launch_face10(int nd, int d, const FaceArgs &a, cudaStream_t s)
+cudaError_t launch_chunk10(int nd, const SweepArgs &a, cudaStream_t s)
 {
-    switch (nd * 3 + d) {
-    case 3: return launch_face<1, 5, 0>(a, s);
-    case 6: return launch_face<2, 5, 0>(a, s);
-    case 7: return launch_face<2, 5, 1>(a, s);
-    case 9: return launch_face<3, 5, 0>(a, s);
-    case 10: return launch_face<3, 5, 1>(a, s);
-    case 11: return launch_face<3, 5, 2>(a, s);
-    default: return cudaErrorInvalidValue;
-    }
+    if (nd == 1) return launch_chunk<1, 5>(a, s);
+    if (nd == 2) return launch_chunk<2, 5>(a, s);
+    return launch_chunk<3, 5>(a, s);
 }
 
 }  // namespace teno

@@ -1,19 +1,13 @@
-// Instantiations of the face sweep for the 8-point TENO-AA scheme.
+// Instantiations of the face-flux kernels for the 8-point TENO-AA scheme.
 #include "teno_face.cuh"
 
 namespace teno {
 
-cudaError_t launch_face8(int nd, int d, const FaceArgs &a, cudaStream_t s)
+cudaError_t launch_chunk8(int nd, const SweepArgs &a, cudaStream_t s)
 {
-    switch (nd * 3 + d) {
-    case 3: return launch_face<1, 4, 0>(a, s);
-    case 6: return launch_face<2, 4, 0>(a, s);
-    case 7: return launch_face<2, 4, 1>(a, s);
-    case 9: return launch_face<3, 4, 0>(a, s);
-    case 10: return launch_face<3, 4, 1>(a, s);
-    case 11: return launch_face<3, 4, 2>(a, s);
-    default: return cudaErrorInvalidValue;
-    }
+    if (nd == 1) return launch_chunk<1, 4>(a, s);
+    if (nd == 2) return launch_chunk<2, 4>(a, s);
+    return launch_chunk<3, 4>(a, s);
 }
 
 }  // namespace teno

@@ -65,6 +65,8 @@ struct FastK {
     int flat_ok;                 // C_r <= 1 and C_T at m = 0 at most 0.1 (the flat cases'
                                  // answer, S_p with the smooth exponent, holds)
     int tiny_ok;                 // flat_ok, and both epsilons at least 2^-136
+    float rho;                   // 3 rho^7 <= thr[nexp_min]: x_p <= rho min_k x_k accepts S_p
+                                 // whatever the exponent (0: never)
 };
 
 // Filter switch (teno_set_decision_filter), process-wide.
@@ -123,6 +125,8 @@ inline FastK fastk_make(double cr, double alpha1, double alpha2, double eps_beta
         if ((double)tu < tr) tu = nextafterf(tu, INFINITY);
         F.thr_rej[n] = nextafterf(tu, INFINITY);
     }
+    const double t3 = (double)F.thr[F.nexp_min] / 3.0;
+    F.rho = t3 > 0.0 ? (float)(pow(t3, 1.0 / 7.0) * (1.0 - 1.0e-6)) : 0.0f;
     return F;
 }
 
@@ -315,6 +319,111 @@ __device__ __forceinline__ int select_large(const float (&f)[2 * H], float lo, f
     }
 }
 
+// Square root with the relative error of the approximate instruction (2^-23).
+__device__ __forceinline__ float sqrt_approx(float x)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+template <int H>
+__device__ __forceinline__ constexpr float sos_bound(int which)
+{
+    // TAU2 KAPPA and K0 of S_H's sum-of-squares form
+    if constexpr (H == 4) return which ? TENO_SOS8_K0 : TENO_SOS8_TAU2 * TENO_SOS8_KAPPA;
+    else if constexpr (H == 5) return which ? TENO_SOS10_K0 : TENO_SOS10_TAU2 * TENO_SOS10_KAPPA;
+    else return which ? TENO_SOS12_K0 : TENO_SOS12_TAU2 * TENO_SOS12_KAPPA;
+}
+
+// First test of a reconstruction whose C_T exponent is not recorded: true
+// only if S_p is certain to be accepted, whatever the exponent (chi_p >= C_T
+// holds if sum_k (x_p / x_k)^7 <= 3 (x_p / min_k x_k)^7 <= thr[nexp_min]).
+// Most reconstructions of a resolved flow end here, so it uses no FP64
+// operation at all and few others; whatever it leaves open goes to
+// fast_decide.
+//
+// The shifted values come from the bit patterns: every value, scaled by a
+// power of two to below 2, is cut exactly into h (24 bits) and l (the next
+// 23), and s_m = (h_m - h_0) + (l_m - l_0).  With M = max |s_m| and the error
+// of a value below 2^-46, every s_m is within 2^-23 |s_m| + 2^-44; for M >=
+// 2^-20 that is at most 3 2^-24 M, inside the 4 2^-24 that the tables'
+// bounds (scaled to |s| <= M) allow for the conversion.  The small
+// indicators carry, with m = max |s_+-1|, |s_+-2| and the exact path's own
+// rounding on the unshifted values (2^-48): |a| <= 5 m, |b| <= 3 m off by at
+// most 7.5 2^-23 m + 5.1 2^-44 and 4.5 2^-23 m + 3.1 2^-44, hence beta_k off
+// by at most 80 2^-23 m^2 + 33 2^-44 m (FP32 rounding included), rounded up
+// to 1e-5 m^2 + 2e-12 m.  Scale: 2^-30 <= max |v| < 2^50, where eps <= 1e-40
+// is below 2e-22 in scaled units and (beta + eps)^7 is a normal number with
+// a normal reciprocal for every beta at or above 2e-22 / rho there.
+template <int H>
+__device__ __forceinline__ bool quick_large(const double (&v)[2 * H], const FastK &F)
+{
+    constexpr int W = 2 * H;
+    unsigned hmax = 0u, hmin = 0x7fffffffu;
+#pragma unroll
+    for (int j = 0; j < W; j++) {
+        const unsigned a = (unsigned)__double2hiint(v[j]) & 0x7fffffffu;
+        hmax = max(hmax, a);
+        hmin = min(hmin, a);
+    }
+    const unsigned ev = hmax >> 20;                      // biased exponent of the largest value
+    // every exponent within 100 of the largest: no zero, subnormal, NaN or infinity
+    const bool range = ev >= 993u && ev <= 1072u && (hmin >> 20) + 100u >= ev;
+    const unsigned eb = (ev - 127u) << 23;
+    float h0, l0, s[W];
+    // offset 0 first, then the others against it
+#pragma unroll
+    for (int jj = 0; jj < W; jj++) {
+        const int j = jj == 0 ? H - 1 : (jj <= H - 1 ? jj - 1 : jj);
+        const unsigned hi = (unsigned)__double2hiint(v[j]), lo = (unsigned)__double2loint(v[j]);
+        const unsigned x = __funnelshift_l(lo, hi, 3) - eb;
+        const unsigned hb = (x & 0x7fffffffu) | (hi & 0x80000000u);
+        const unsigned es = (hb & 0xff800000u) - (23u << 23);
+        const float l = __uint_as_float(((lo >> 6) & 0x7fffffu) | es) - __uint_as_float(es);
+        const float h = __uint_as_float(hb);
+        if (jj == 0) {
+            h0 = h;
+            l0 = l;
+            s[j] = 0.0f;
+        } else {
+            s[j] = (h - h0) + (l - l0);
+        }
+    }
+#define SS(m) s[(m) + H - 1]
+    const float ms = fmaxf(fmaxf(fabsf(SS(-2)), fabsf(SS(-1))), fmaxf(fabsf(SS(1)), fabsf(SS(2))));
+    float M = ms;
+#pragma unroll
+    for (int j = 0; j < W; j++)
+        if (j < H - 3 || j > H + 1) M = fmaxf(M, fabsf(s[j]));
+    const float c13 = 13.0f / 12.0f;
+    const float a0 = SS(-1) - SS(1), b0 = SS(-1) + SS(1);
+    const float a1 = fmaf(-4.0f, SS(1), SS(2)), b1 = fmaf(-2.0f, SS(1), SS(2));
+    const float a2 = fmaf(-4.0f, SS(-1), SS(-2)), b2 = fmaf(-2.0f, SS(-1), SS(-2));
+    const float m0 = fmaf(c13, b0 * b0, 0.25f * (a0 * a0));
+    const float m1 = fmaf(c13, b1 * b1, 0.25f * (a1 * a1));
+    const float m2 = fmaf(c13, b2 * b2, 0.25f * (a2 * a2));
+    const float xk = fminf(m0, fminf(m1, m2)) - ms * fmaf(1.0e-5f, ms, 2.0e-12f);
+    constexpr int n = 2 * H - 1;
+    float bt = 0.0f;
+#pragma unroll
+    for (int i = 0; i < n; i++) {
+        const int oi = i < H ? H - i : H - 1 - i;
+        float y = SS(oi);
+#pragma unroll
+        for (int m = i + 1; m < n; m++) {
+            const int om = m < H ? H - m : H - 1 - m;
+            y = fmaf(sos_l<H>(m, i), SS(om), y);
+        }
+        bt = fmaf(sos_d<H>(i), y * y, bt);
+    }
+    const float E = fmaf(sos_bound<H>(0) * M, sqrt_approx(bt),
+                         fmaf(bt, (float)(n + 3) * 5.9604645e-8f, sos_bound<H>(1) * (M * M)));
+    const float xp = fmaf(bt + E, 1.0f + 4.0e-6f, 2.0e-22f);
+#undef SS
+    return range && M >= 9.5367431640625e-7f && xp <= (F.rho * (1.0f - 2.0e-6f)) * xk;
+}
+
 // A small indicator's FP64 input as the exact path forms it, converted to
 // scaled FP32 with the bound of its truncation and flush.
 __device__ __forceinline__ void small_in_exact(double x, int emax, float &v, float &err)
@@ -323,17 +432,168 @@ __device__ __forceinline__ void small_in_exact(double x, int emax, float &v, flo
     err = 1.1920929e-7f * 1.0001f * fabsf(v) + 1.6e-30f;
 }
 
-// The filter.  v: the 2H values (FP64); s: shifted values s_m = v_m - v_0
-// (s[H-1] == 0); need_ct: the caller records the decision byte, so its C_T
-// exponent must be known.  Returns true with the decision byte (the exact
-// path's encoding) when every decision is certain.
+// The filter's single-precision inputs of one reconstruction, scaled by
+// 2^-emax (so that every |f_m| < 2): the shifted values f_m, each off by at
+// most 2^-23 |f_m| + zs, and the small indicators' inputs as the exact path
+// forms them, with their absolute error bounds.
 template <int H>
-__device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const double (&s)[2 * H],
-                                            const FastK &F, uint8_t &flag, bool need_ct)
+struct FilterInput {
+    float f[2 * H];
+    float sa[3], sea[3], sb[3], seb[3];
+    float zs;
+    int emax;
+};
+
+// Inputs a_k, b_k of the small indicators on the shifted values (s_0 = 0);
+// the slack eo holds the exact path's rounding on the unshifted values.
+template <int H>
+__device__ __forceinline__ void small_in_shifted(FilterInput<H> &o, float eo)
+{
+#define FF(m) o.f[(m) + H - 1]
+    const float u23 = 1.1920929e-7f * 1.0001f, u24 = 5.9604645e-8f * 1.0001f;
+    const float sl0 = 2.0f * o.zs + 4.0f * eo, sl1 = 5.0f * o.zs + 8.0f * eo;
+    o.sa[0] = FF(-1) - FF(1);
+    o.sea[0] = u23 * (fabsf(FF(-1)) + fabsf(FF(1))) + u24 * fabsf(o.sa[0]) + sl0;
+    o.sb[0] = FF(-1) + FF(1);
+    o.seb[0] = u23 * (fabsf(FF(-1)) + fabsf(FF(1))) + u24 * fabsf(o.sb[0]) + sl0;
+    o.sa[1] = FF(2) - 4.0f * FF(1);
+    o.sea[1] = u23 * (fabsf(FF(2)) + 4.0f * fabsf(FF(1))) + u24 * fabsf(o.sa[1]) + sl1;
+    o.sb[1] = FF(2) - 2.0f * FF(1);
+    o.seb[1] = u23 * (fabsf(FF(2)) + 2.0f * fabsf(FF(1))) + u24 * fabsf(o.sb[1]) + sl1;
+    o.sa[2] = FF(-2) - 4.0f * FF(-1);
+    o.sea[2] = u23 * (fabsf(FF(-2)) + 4.0f * fabsf(FF(-1))) + u24 * fabsf(o.sa[2]) + sl1;
+    o.sb[2] = FF(-2) - 2.0f * FF(-1);
+    o.seb[2] = u23 * (fabsf(FF(-2)) + 2.0f * fabsf(FF(-1))) + u24 * fabsf(o.sb[2]) + sl1;
+#undef FF
+}
+
+// RNE(t, u) - t for a positive integer t given by its low three bits, u = 4
+// (wide) or 2: what rounding to a multiple of u adds.
+__device__ __forceinline__ int rne_change(unsigned t, bool wide)
+{
+    const int r = (int)(t & 3u);
+    if (wide) return r == 0 ? 0 : (r == 1 ? -1 : (r == 3 ? 1 : ((t & 4u) ? 2 : -2)));
+    return r == 1 ? -1 : (r == 3 ? 1 : 0);
+}
+
+enum { kFrontOpen = 0, kFrontReady = 1, kFrontFlat = 2, kFrontTiny = 3 };
+
+// The inputs from the bit patterns alone, without an FP64 operation (each
+// holds a scheduler's FP64 unit for 64 cycles).  Two forms are taken.
+//
+// Values that agree in sign and exponent and differ by less than 2^20 units
+// of their last place (a plateau that carries rounding noise): the
+// differences d_m are small integers, and so are the exact path's own inputs
+// on the unshifted values.  With m_0 the integer significand of v_0 (2^23
+// below 2^53 at least, so that sums near m_0 stay exact), every step of
+// a_0, b_0, b_1 and b_2 is exact, and 3 v_0 and V(-2) - 4 V(-1), of size
+// 3 m_0, round to multiples of 2 or 4 (below and above 2^54, 2^25 away from
+// it at least): a_1 = d_2 - 4 d_1 + r and a_2 = d_-2 - 4 d_-1 + r - r' with
+// the two roundings r, r'.  Signs drop out (both indicators and the eta
+// measure are even), so magnitudes are used throughout.
+//
+// Otherwise values of ordinary variation: h + l as in quick_large, values
+// 2^100 times smaller than the largest taken as zero; M >= 2^-20.
+template <int H>
+__device__ __forceinline__ int front_bits(const double (&v)[2 * H], FilterInput<H> &o)
 {
     constexpr int W = 2 * H;
-#define SV(m) s[(m) + H - 1]
+    unsigned hmax = 0u, hmin = 0x7fffffffu, sx = 0u;
+    const unsigned hi0 = (unsigned)__double2hiint(v[H - 1]);
+#pragma unroll
+    for (int j = 0; j < W; j++) {
+        const unsigned hi = (unsigned)__double2hiint(v[j]), a = hi & 0x7fffffffu;
+        hmax = max(hmax, a);
+        hmin = min(hmin, a);
+        sx |= hi ^ hi0;
+    }
+    const unsigned ev = hmax >> 20;
+    if (ev < 928u || ev > 1072u) return kFrontOpen;     // 2^-95 <= max |v| < 2^50
+#define FF(m) o.f[(m) + H - 1]
+    if (!(sx >> 31) && ev == hmin >> 20 && hmax - hmin <= 1u) {
+        const long long z0 = __double_as_longlong(v[H - 1]);
+        int d[W];
+        unsigned far = 0u;
+        int big = 0;
+#pragma unroll
+        for (int j = 0; j < W; j++) {
+            const long long dj = __double_as_longlong(v[j]) - z0;
+            const long long up = dj + (1ll << 20);
+            far |= (unsigned)(up >> 32) | ((unsigned)up >> 21);
+            d[j] = (int)dj;
+            big = max(big, abs(d[j]));
+        }
+        if (far) return kFrontOpen;
+        if (big == 0) return kFrontFlat;
+        const long long m0 = (z0 & 0xFFFFFFFFFFFFFll) | (1ll << 52);
+        const long long t3 = 3 * m0, away = t3 - (1ll << 54);
+        if (m0 > (1ll << 53) - (1ll << 23) || (away > -(1ll << 25) && away < (1ll << 25)))
+            return kFrontOpen;
+        const int kb = 31 - __clz(big);
+        o.emax = (int)ev - 1023 - 52 + kb;
+        if (o.emax < -100) return kFrontTiny;
+        const float sc = __uint_as_float((unsigned)(127 - kb) << 23);
+#define DD(m) d[(m) + H - 1]
+        const bool wide = away > 0;
+        const int e2 = DD(-2) - 4 * DD(-1);
+        const int r3 = rne_change((unsigned)t3, wide), r2 = rne_change((unsigned)(t3 - e2), wide);
+        o.sa[0] = (float)(DD(-1) - DD(1)) * sc;
+        o.sb[0] = (float)(DD(-1) + DD(1)) * sc;
+        o.sa[1] = (float)(DD(2) - 4 * DD(1) + r3) * sc;
+        o.sb[1] = (float)(DD(2) - 2 * DD(1)) * sc;
+        o.sa[2] = (float)(e2 + r3 - r2) * sc;
+        o.sb[2] = (float)(DD(-2) - 2 * DD(-1)) * sc;
+#undef DD
+#pragma unroll
+        for (int k = 0; k < 3; k++) o.sea[k] = o.seb[k] = 0.0f;
+        o.zs = 1.6e-30f;
+#pragma unroll
+        for (int j = 0; j < W; j++) o.f[j] = (float)d[j] * sc;
+        return kFrontReady;
+    }
+    const unsigned eb = (ev - 127u) << 23;
+    float h0, l0, M = 0.0f;
+#pragma unroll
+    for (int jj = 0; jj < W; jj++) {
+        const int j = jj == 0 ? H - 1 : (jj <= H - 1 ? jj - 1 : jj);
+        const unsigned hi = (unsigned)__double2hiint(v[j]), lo = (unsigned)__double2loint(v[j]);
+        const unsigned x = __funnelshift_l(lo, hi, 3) - eb;
+        const unsigned hb = (x & 0x7fffffffu) | (hi & 0x80000000u);
+        const unsigned es = (hb & 0xff800000u) - (23u << 23);
+        float l = __uint_as_float(((lo >> 6) & 0x7fffffu) | es) - __uint_as_float(es);
+        float h = __uint_as_float(hb);
+        if (((hi & 0x7fffffffu) >> 20) + 100u < ev) h = l = 0.0f;
+        if (jj == 0) {
+            h0 = h;
+            l0 = l;
+            o.f[j] = 0.0f;
+        } else {
+            o.f[j] = (h - h0) + (l - l0);
+            M = fmaxf(M, fabsf(o.f[j]));
+        }
+    }
+    if (!(M >= 9.5367431640625e-7f)) return kFrontOpen;
+    const int em = (int)(__float_as_uint(M) >> 23) - 127;            // -20 .. 1
+    const float sc = __uint_as_float((unsigned)(127 - em) << 23);
+    o.emax = (int)ev - 1023 + em;
+    if (o.emax < -100) return kFrontTiny;
+    o.zs = 5.7e-14f * sc;                                              // 2^-44
+#pragma unroll
+    for (int j = 0; j < W; j++) o.f[j] *= sc;
+    small_in_shifted<H>(o, 1.7763568394002505e-15f * sc);            // 2^-49
+    return kFrontReady;
+#undef FF
+}
+
+// The inputs by FP64 subtraction, for every form front_bits leaves open.
+template <int H>
+__device__ __forceinline__ int front_fp64(const double (&v)[2 * H], FilterInput<H> &o)
+{
+    constexpr int W = 2 * H;
 #define VV(m) v[(m) + H - 1]
+    double s[W];
+#pragma unroll
+    for (int j = 0; j < W; j++) s[j] = v[j] - v[H - 1];
     // Common scale: the largest exponent among the shifted values (the
     // largest biased exponent field: zero for zeros and subnormals, 0x7FF for
     // non-finite values, which the range test below sends on).
@@ -342,21 +602,70 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const doub
     for (int j = 0; j < W; j++)
         if (j != H - 1) efield = max(efield, (__double2hiint(s[j]) >> 20) & 0x7FF);
     const int emax = efield - 1023;
+    o.emax = emax;
     if (efield == 0) {
-        // No shifted value above the subnormal range.  All values bit-identical:
+        // no shifted value above the subnormal range
+        bool all_eq = true;
+#pragma unroll
+        for (int j = 0; j < W; j++) all_eq = all_eq && dbits_equal(v[j], v[H - 1]);
+        return all_eq ? kFrontFlat : kFrontOpen;
+    }
+    if (emax < -100) return kFrontTiny;
+    if (emax > 50) return kFrontOpen;
+#pragma unroll
+    for (int j = 0; j < W; j++) o.f[j] = (j == H - 1) ? 0.0f : d2f_scaled(s[j], emax);
+    o.zs = 1.6e-30f;                         // > 2^-100: flushed-value error
+    // The exact path evaluates the small indicators on the unshifted values:
+    // its rounding is relative to max |v| (bound 2^(ev - emax - 50) scaled).
+    // |v_m| <= |v_0| + |v_m - v_0| < 2^(e_0 + 1) + 2^(emax + 1) (1 + 2^-52)
+    // with e_0 the exponent of v_0, so ev = max(e_0, emax) + 1 bounds the
+    // exponent of every v_m.
+    const int ecell = (__double2hiint(VV(0)) & 0x7FF00000) != 0 ? dexp(VV(0)) : -1100;
+    const int ev = max(ecell, emax) + 1;
+    if (ev - emax > 60) return kFrontOpen;
+    const float eo = ev < -900 ? 0.0f : __uint_as_float((unsigned)(max(ev - emax - 50, -126) + 127) << 23);
+    if (ev - emax >= 30) {
+        // values within 2^-30 of one another relative to their size: the
+        // exact path's rounding on the unshifted values is then as large as
+        // their differences, so take its own FP64 inputs (the same
+        // operations: bitwise its values) and bound only their conversion
+        small_in_exact(VV(-1) - VV(1), emax, o.sa[0], o.sea[0]);
+        small_in_exact((VV(-1) - 2.0 * VV(0)) + VV(1), emax, o.sb[0], o.seb[0]);
+        small_in_exact((3.0 * VV(0) - 4.0 * VV(1)) + VV(2), emax, o.sa[1], o.sea[1]);
+        small_in_exact((VV(0) - 2.0 * VV(1)) + VV(2), emax, o.sb[1], o.seb[1]);
+        small_in_exact((VV(-2) - 4.0 * VV(-1)) + 3.0 * VV(0), emax, o.sa[2], o.sea[2]);
+        small_in_exact((VV(-2) - 2.0 * VV(-1)) + VV(0), emax, o.sb[2], o.seb[2]);
+    } else {
+        small_in_shifted<H>(o, eo);
+    }
+    return kFrontReady;
+#undef VV
+}
+
+// The filter.  v: the 2H values (FP64); need_ct: the caller records the
+// decision byte, so its C_T exponent must be known.  Returns true with the
+// decision byte (the exact path's encoding) when every decision is certain.
+template <int H>
+__device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const FastK &F, uint8_t &flag,
+                                            bool need_ct)
+{
+#define VV(m) v[(m) + H - 1]
+    FilterInput<H> o;
+    int front = front_bits<H>(v, o);
+    if (front == kFrontOpen) front = front_fp64<H>(v, o);
+    if (front == kFrontOpen) return false;
+    if (front == kFrontFlat) {
+        // All values bit-identical:
         // the exact path's beta_0 and beta_p are 0 and beta_1 = beta_2 (the
         // rounding of 3 v_0), so chi_p lies in [1/4, 1/2] (or is NaN for
         // eps = 0, which also keeps S_p), and eta = eps/eps = 1 (m = 0 when
         // C_r <= 1; NaN for eps = 0, m = 0 too): S_p with the smooth exponent
         // when C_T <= 0.1 there.  Anything else goes to the exact path.
-        bool all_eq = F.flat_ok != 0;
-#pragma unroll
-        for (int j = 0; j < W; j++) all_eq = all_eq && dbits_equal(v[j], v[H - 1]);
-        if (!all_eq) return false;
+        if (!F.flat_ok) return false;
         flag = (uint8_t)(large_code(H) | (((F.nexp_smooth - 7) & 7) << 5));
         return true;
     }
-    if (emax < -100) {
+    if (front == kFrontTiny) {
         // Every shifted value below 2^-100, not all zero: distinct doubles that
         // close are below 2^-46 in size, so every indicator the exact path
         // forms, its own rounding included, is below 2^-177 (the largest
@@ -369,10 +678,7 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const doub
         flag = (uint8_t)(large_code(H) | (((F.nexp_smooth - 7) & 7) << 5));
         return true;
     }
-    if (emax > 50) return false;
-    float f[W];
-#pragma unroll
-    for (int j = 0; j < W; j++) f[j] = (j == H - 1) ? 0.0f : d2f_scaled(s[j], emax);
+    const int emax = o.emax;
     // floor of every x_k: 2^-140 in original units (the exact path's
     // (beta+eps)^7 stays normal), at least 2^-120 scaled (FP32 stays normal)
     const int tb = max(-140 - 2 * emax, -120);
@@ -389,53 +695,11 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const doub
         }
     }
     const float u23 = 1.1920929e-7f * 1.0001f, u24 = 5.9604645e-8f * 1.0001f;
-    const float z100 = 1.6e-30f;             // > 2^-100: flushed-value error
-    // The exact path evaluates the small indicators on the unshifted values:
-    // its rounding is relative to max |v| (bound 2^(ev - emax - 50) scaled).
-    // |v_m| <= |v_0| + |v_m - v_0| < 2^(e_0 + 1) + 2^(emax + 1) (1 + 2^-52)
-    // with e_0 the exponent of v_0, so ev = max(e_0, emax) + 1 bounds the
-    // exponent of every v_m.
-    const int ecell = (__double2hiint(VV(0)) & 0x7FF00000) != 0 ? dexp(VV(0)) : -1100;
-    const int ev = max(ecell, emax) + 1;
-    if (ev - emax > 60) return false;
-    const float eo = ev < -900 ? 0.0f : __uint_as_float((unsigned)(max(ev - emax - 50, -126) + 127) << 23);
-#define FF(m) f[(m) + H - 1]
-
-    // Inputs a_k, b_k of the three small indicators with absolute error
-    // bounds (scaled units).
-    float sa[3], sea[3], sb[3], seb[3];
-    if (ev - emax >= 30) {
-        // values within 2^-30 of one another relative to their size: the
-        // exact path's rounding on the unshifted values is then as large as
-        // their differences, so take its own FP64 inputs (the same
-        // operations: bitwise its values) and bound only their conversion
-        small_in_exact(VV(-1) - VV(1), emax, sa[0], sea[0]);
-        small_in_exact((VV(-1) - 2.0 * VV(0)) + VV(1), emax, sb[0], seb[0]);
-        small_in_exact((3.0 * VV(0) - 4.0 * VV(1)) + VV(2), emax, sa[1], sea[1]);
-        small_in_exact((VV(0) - 2.0 * VV(1)) + VV(2), emax, sb[1], seb[1]);
-        small_in_exact((VV(-2) - 4.0 * VV(-1)) + 3.0 * VV(0), emax, sa[2], sea[2]);
-        small_in_exact((VV(-2) - 2.0 * VV(-1)) + VV(0), emax, sb[2], seb[2]);
-    } else {
-        // on the shifted values (s_0 = 0); the slack holds the exact path's
-        // rounding on the unshifted values
-        const float sl0 = 2.0f * z100 + 4.0f * eo, sl1 = 5.0f * z100 + 8.0f * eo;
-        sa[0] = FF(-1) - FF(1);
-        sea[0] = u23 * (fabsf(FF(-1)) + fabsf(FF(1))) + u24 * fabsf(sa[0]) + sl0;
-        sb[0] = FF(-1) + FF(1);
-        seb[0] = u23 * (fabsf(FF(-1)) + fabsf(FF(1))) + u24 * fabsf(sb[0]) + sl0;
-        sa[1] = FF(2) - 4.0f * FF(1);
-        sea[1] = u23 * (fabsf(FF(2)) + 4.0f * fabsf(FF(1))) + u24 * fabsf(sa[1]) + sl1;
-        sb[1] = FF(2) - 2.0f * FF(1);
-        seb[1] = u23 * (fabsf(FF(2)) + 2.0f * fabsf(FF(1))) + u24 * fabsf(sb[1]) + sl1;
-        sa[2] = FF(-2) - 4.0f * FF(-1);
-        sea[2] = u23 * (fabsf(FF(-2)) + 4.0f * fabsf(FF(-1))) + u24 * fabsf(sa[2]) + sl1;
-        sb[2] = FF(-2) - 2.0f * FF(-1);
-        seb[2] = u23 * (fabsf(FF(-2)) + 2.0f * fabsf(FF(-1))) + u24 * fabsf(sb[2]) + sl1;
-    }
+#define FF(m) o.f[(m) + H - 1]
     float b0, e0, b1, e1, b2, e2;
-    small_beta(sa[0], sea[0], sb[0], seb[0], b0, e0);
-    small_beta(sa[1], sea[1], sb[1], seb[1], b1, e1);
-    small_beta(sa[2], sea[2], sb[2], seb[2], b2, e2);
+    small_beta(o.sa[0], o.sea[0], o.sb[0], o.seb[0], b0, e0);
+    small_beta(o.sa[1], o.sea[1], o.sb[1], o.seb[1], b1, e1);
+    small_beta(o.sa[2], o.sea[2], o.sb[2], o.seb[2], b2, e2);
     // x_k = beta_k + eps: lower and upper bounds, the lower ones at tiny2 or above
     const float x0 = x_lower(b0 - e0, ebl), x1 = x_lower(b1 - e1, ebl), x2 = x_lower(b2 - e2, ebl);
     if (!(x0 >= tiny2) || !(x1 >= tiny2) || !(x2 >= tiny2)) return false;
@@ -447,7 +711,7 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const doub
     // leaves the eta measure out for most reconstructions.  The C_T bits of
     // the byte are then zero (the byte is not stored).
     float blo, bhi;                           // bounds of beta_p, for both tests
-    beta_large_bounds<H, H>(f, blo, bhi);
+    beta_large_bounds<H, H>(o.f, blo, bhi);
     if (!need_ct) {
         // sum_k (x_p / x_k)^7 <= 3 (x_p / min_k x_k)^7: one division for the
         // common case (a looser bound only sends borderline cases on)
@@ -466,7 +730,7 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const doub
     for (int m = -2; m <= 2; m++) {
         const float a = FF(m + 1), b = FF(m);
         dl[m + 2] = a - b;
-        el[m + 2] = u23 * (fabsf(a) + fabsf(b)) + u24 * fabsf(dl[m + 2]) + 2.0f * z100;
+        el[m + 2] = u23 * (fabsf(a) + fabsf(b)) + u24 * fabsf(dl[m + 2]) + 2.0f * o.zs;
         zl[m + 2] = dbits_equal(VV(m + 1), VV(m));
     }
     float emin_lo = 1.0f, emin_hi = 1.0f;
@@ -499,7 +763,7 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const doub
     const float thr = F.thr[nexp], thr_rej = F.thr_rej[nexp];
 
     // Targeted selection, largest group first (Sec. 3.3).
-    const int sel = select_large<H, H>(f, blo, bhi, tiny2, ebl, ebh, x0, x1, x2, X0, X1, X2, thr,
+    const int sel = select_large<H, H>(o.f, blo, bhi, tiny2, ebl, ebh, x0, x1, x2, X0, X1, X2, thr,
                                        thr_rej);
     if (sel < 0) return false;
     if (sel > 0) {
@@ -526,7 +790,6 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const doub
     flag = (uint8_t)(((d[0] | (d[1] << 1) | (d[2] << 2)) << 2) | fct);
     return true;
 #undef FF
-#undef SV
 #undef VV
 }
 
