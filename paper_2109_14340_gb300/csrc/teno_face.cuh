@@ -83,7 +83,7 @@ struct SweepBuf {
     uint32_t *xlist;       // [nt per_tile] entries left to the exact path
     uint32_t *count;       // [nt] queue lengths
     double *R;             // [2 nc][nt 32] reconstructed values
-    double *RO;            // [nd + 2][nt 32] Roe velocity, enthalpy, sound speed
+    double *RO;            // [nd + 4][nt 32] Roe velocity, enthalpy, sound speed, |u|^2, u_d c
     double *RL;            // [4 nc + 1][nt 32] limiter: halved U, F of cells i, i+1, and the
                            // Lax-Friedrichs speed; nullptr without a limiter
     uint8_t *RD;           // [2 nc][nt 32] decision bytes; nullptr without a record
@@ -106,7 +106,7 @@ inline size_t sweep_buf_layout(SweepBuf &b, char *p, int64_t nt, int nd, int W, 
     b.qslot = (uint16_t *)take(sizeof(uint16_t) * q);
     b.count = (uint32_t *)take(sizeof(uint32_t) * nt);
     b.R = (double *)take(sizeof(double) * 2 * nc * f);
-    b.RO = (double *)take(sizeof(double) * (nd + 2) * f);
+    b.RO = (double *)take(sizeof(double) * (nd + 4) * f);
     b.RD = (uint8_t *)take(2 * nc * f);
     b.RL = limiter ? (double *)take(sizeof(double) * (4 * nc + 1) * f) : nullptr;
     return off;
@@ -430,6 +430,8 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
         for (int k = 0; k < ND; k++) B.RO[k * nf + cf] = rs.ut[k];
         B.RO[ND * nf + cf] = rs.Ht;
         B.RO[(ND + 1) * nf + cf] = rs.ct;
+        B.RO[(ND + 2) * nf + cf] = rs.q2;
+        B.RO[(ND + 3) * nf + cf] = rs.unct;
         if (a.limiter) {
 #pragma unroll
             for (int c = 0; c < nc; c++) {
@@ -542,58 +544,6 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
 #undef TMP
 }
 
-// |x| in FP32, rounded up; infinity for what FP32 does not hold and for NaN.
-__device__ __forceinline__ float abs_up(double x)
-{
-    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu, e = hi >> 20;
-    if (e < 897u) return 1.17549435e-38f;
-    if (e > 1149u) return INFINITY;
-    return __uint_as_float((__funnelshift_l((unsigned)__double2loint(x), hi, 3) - (896u << 23)) + 1u);
-}
-
-// True only if the positivity limiter certainly leaves this flux as it is.  Both
-// one-sided updates U_i -+ 2 lam (F - F_i) with the whole flux are formed
-// (halved); the limiter's own come from the same terms by way of the
-// Lax-Friedrichs flux, so each component of theirs is within 2^-49 of S_c, the
-// sum of the sizes of all terms.  Density and rho p above 1e-13 times
-// those sizes (and the limiter's eps) therefore pass its tests too, with
-// theta = 1.  Some 34 FP64 instructions where the limiter's own test takes
-// about 215 (3D Noh, 64^3: 0.46 ms a stage for the finish kernel).
-template <int ND>
-__device__ __forceinline__ bool limiter_calm(const double (&Fo)[ND + 2], double lam, const Consts &K,
-                                             const SweepBuf &B, int64_t nf, int64_t cf)
-{
-    constexpr int nc = ND + 2, last = nc - 1;
-    const float af = abs_up(B.RL[4 * nc * nf + cf]), lf = abs_up(lam);
-    double ul[nc], ur[nc];
-    float S[nc];
-#pragma unroll
-    for (int c = 0; c < nc; c++) {
-        const double hUl = B.RL[(4 * c) * nf + cf], hFl = B.RL[(4 * c + 1) * nf + cf];
-        const double hUr = B.RL[(4 * c + 2) * nf + cf], hFr = B.RL[(4 * c + 3) * nf + cf];
-        ul[c] = fma(-lam, fma(-2.0, hFl, Fo[c]), hUl);
-        ur[c] = fma(lam, fma(-2.0, hFr, Fo[c]), hUr);
-        const float u = abs_up(hUl) + abs_up(hUr);
-        S[c] = u + lf * (abs_up(Fo[c]) + 2.0f * (abs_up(hFl) + abs_up(hFr)) + 2.0f * af * u);
-    }
-    float k = 2.0f * S[last] * S[0];
-#pragma unroll
-    for (int a = 0; a < ND; a++) k = fmaf(S[1 + a], S[1 + a], k);
-    const double rho_min = (double)(1.0e-13f * S[0]) + K.lim_eps;
-    const double q_min = K.gm1 * (double)(1.0e-13f * k), e2 = 2.0 * K.lim_eps;
-    bool calm = isfinite(k);
-#pragma unroll
-    for (int side = 0; side < 2; side++) {
-        const double(&u)[nc] = side ? ur : ul;
-        double q = -(u[1] * u[1]);                     // rho p / (2 (gamma - 1))
-#pragma unroll
-        for (int a = 1; a < ND; a++) q = fma(-u[1 + a], u[1 + a], q);
-        q = fma(2.0 * u[last], u[0], q);
-        calm = calm && u[0] > rho_min && K.gm1 * q > fma(e2, u[0], q_min);
-    }
-    return calm;
-}
-
 // Back-projection of a face, the limiter, and what it leaves: the flux, the
 // limiter's byte and the decision bytes of the record.
 template <int ND, int D, int MODE>
@@ -603,15 +553,13 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
     constexpr int nc = ND + 2, last = nc - 1;
     const int64_t nf = B.nt * kTileFaces;
     if (!TENO_IN(st, flin, da.nfaces)) return;
-    RoeScalars<ND> rs;                 // the entries r_entry reads, as roe_state forms them
+    RoeScalars<ND> rs;                 // what r_entry reads
 #pragma unroll
     for (int k = 0; k < ND; k++) rs.ut[k] = B.RO[k * nf + cf];
     rs.Ht = B.RO[ND * nf + cf];
     rs.ct = B.RO[(ND + 1) * nf + cf];
-    rs.q2 = rs.ut[0] * rs.ut[0];
-#pragma unroll
-    for (int k = 1; k < ND; k++) rs.q2 = fma(rs.ut[k], rs.ut[k], rs.q2);
-    rs.unct = rs.ut[D] * rs.ct;
+    rs.q2 = B.RO[(ND + 2) * nf + cf];
+    rs.unct = B.RO[(ND + 3) * nf + cf];
     // F = sum_k r_k (f+_k + f-_k), fields ascending; the zero and unit entries
     // of the shear columns are skipped.
     double Fo[nc];
@@ -633,9 +581,7 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
         }
     }
 
-    if (limiter && limiter_calm<ND>(Fo, *da.lam, K, B, nf, cf)) {
-        if constexpr (MODE == kSweepRecord) da.limrec[flin] = 0;
-    } else if (limiter) {
+    if (limiter) {
         // Positivity-preserving flux limiter (cited in Sec. 5.3): blend toward
         // the Lax-Friedrichs flux so that the one-sided half updates of cells i
         // and i+1 keep rho >= eps and p >= eps.
@@ -644,16 +590,15 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
 #pragma unroll
         for (int c = 0; c < nc; c++) {
             // staged halves: FL = (F_l + F_r)/2 - af (U_r - U_l)/2 exactly as
-            // ((F_l + F_r) - af (U_r - U_l)) / 2
+            // ((F_l + F_r) - af (U_r - U_l)) / 2; a doubled half joins a sum in one fma
             const double hUl = B.RL[(4 * c) * nf + cf], hFl = B.RL[(4 * c + 1) * nf + cf];
             const double hUr = B.RL[(4 * c + 2) * nf + cf], hFr = B.RL[(4 * c + 3) * nf + cf];
-            const double Ul = 2.0 * hUl, Ur = 2.0 * hUr, Fl = 2.0 * hFl, Fr = 2.0 * hFr;
             FL[c] = (hFl + hFr) - af * (hUr - hUl);
             dF[c] = Fo[c] - FL[c];
-            UL[c] = Ul - lam2 * (FL[c] - Fl);
-            UR[c] = Ur + lam2 * (FL[c] - Fr);
-            dUL[c] = -(lam2 * dF[c]);
+            UL[c] = fma(2.0, hUl, -(lam2 * fma(-2.0, hFl, FL[c])));
+            UR[c] = fma(2.0, hUr, lam2 * fma(-2.0, hFr, FL[c]));
             dUR[c] = lam2 * dF[c];
+            dUL[c] = -dUR[c];
         }
         double th = 1.0;
 #pragma unroll
@@ -673,7 +618,8 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
 #pragma unroll
             for (int c = 0; c < nc; c++) {
                 Us[c] = side ? UR[c] : UL[c];
-                Ut[c] = Us[c] + th * (side ? dUR[c] : dUL[c]);
+                const double dU = side ? dUR[c] : dUL[c];
+                Ut[c] = Us[c] + (th == 1.0 ? dU : th * dU);
             }
             const double pt = pressure_of<ND>(Ut, K.gm1);
             if (pt < eps) {
@@ -920,10 +866,10 @@ cudaError_t launch_decisions(const SweepBuf &B, int32_t tiles, int nc, int fast,
                              unsigned *nexact, unsigned long long *exact_count, const FastK &FK,
                              const Consts &K, Status *st, cudaStream_t s)
 {
-    // warps enough to fill the chip (24 on each of 152 SMs) before tiles share one
+    // at least four waves of warps (24 on each of 152 SMs) before tiles share one
     const int64_t fill = 152 * 24;
     int group = 1, split = 1;
-    while (group < kDecideMostTiles && tiles > fill * group) group *= 2;
+    while (group < kDecideMostTiles && tiles >= 8 * fill * group) group *= 2;
     while (group == 1 && split < 2 * nc && (int64_t)tiles * split * 2 <= fill) split *= 2;
     const int64_t units = (int64_t)((tiles + group - 1) / group) * split;
     decide_kernel<H, RECORD><<<(unsigned)((units + kDecideWarps - 1) / kDecideWarps), 32 * kDecideWarps, 0, s>>>(

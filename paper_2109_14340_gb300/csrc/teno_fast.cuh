@@ -65,8 +65,10 @@ struct FastK {
     int flat_ok;                 // C_r <= 1 and C_T at m = 0 at most 0.1 (the flat cases'
                                  // answer, S_p with the smooth exponent, holds)
     int tiny_ok;                 // flat_ok, and both epsilons at least 2^-136
-    float rho;                   // 3 rho^7 <= thr[nexp_min]: x_p <= rho min_k x_k accepts S_p
-                                 // whatever the exponent (0: never)
+    float rho_acc[23];           // 3 rho_acc[n]^7 <= thr[n]: x <= rho_acc[n] min_k x_k accepts
+                                 // (0: never)
+    float rho_rej[23];           // rho_rej[n]^7 >= thr_rej[n]: x >= rho_rej[n] min_k x_k rejects
+    float cr_up;                 // C_r (1 + 1e-5) rounded up
 };
 
 // Filter switch (teno_set_decision_filter), process-wide.
@@ -125,8 +127,12 @@ inline FastK fastk_make(double cr, double alpha1, double alpha2, double eps_beta
         if ((double)tu < tr) tu = nextafterf(tu, INFINITY);
         F.thr_rej[n] = nextafterf(tu, INFINITY);
     }
-    const double t3 = (double)F.thr[F.nexp_min] / 3.0;
-    F.rho = t3 > 0.0 ? (float)(pow(t3, 1.0 / 7.0) * (1.0 - 1.0e-6)) : 0.0f;
+    for (int n = 0; n < 23; n++) {
+        const double ta = (double)F.thr[n] / 3.0, tr = (double)F.thr_rej[n];
+        F.rho_acc[n] = ta > 0.0 ? (float)(pow(ta, 1.0 / 7.0) * (1.0 - 1.0e-6)) : 0.0f;
+        F.rho_rej[n] = tr > 0.0 ? (float)(pow(tr, 1.0 / 7.0) * (1.0 + 1.0e-6)) : 1.0f;
+    }
+    F.cr_up = nextafterf((float)(cr * (1.0 + 1.0e-5)), INFINITY);
     return F;
 }
 
@@ -304,16 +310,24 @@ __device__ __forceinline__ float x_lower(float lo, float elo)
 template <int H, int L>
 __device__ __forceinline__ int select_large(const float (&f)[2 * H], float lo, float hi, float tiny2,
                                             float elo, float ehi, float x0, float x1, float x2,
-                                            float X0, float X1, float X2, float thr, float thr_rej)
+                                            float X0, float X1, float X2, float thr, float thr_rej,
+                                            float acc, float rej)
 {
-    if (pow7_sum(x_upper(hi, ehi), x0, x1, x2, true) <= thr) return L - 2;
-    const float xl = x_lower(lo, elo);
-    if (!(xl >= tiny2) || !(pow7_sum(xl, X0, X1, X2, false) > thr_rej)) return -1;
+    // acc, rej: acc min_k x_k below which the sum of three is at most thr, and rej
+    // min_k X_k above which one of them alone exceeds thr_rej; the sums
+    // themselves are needed only between (ratios within 3^(1/7) = 1.17)
+    const float xu = x_upper(hi, ehi), xl = x_lower(lo, elo);
+    if (xu <= acc) return L - 2;
+    if (!(xl >= tiny2)) return pow7_sum(xu, x0, x1, x2, true) <= thr ? L - 2 : -1;
+    if (!(xl >= rej)) {
+        if (pow7_sum(xu, x0, x1, x2, true) <= thr) return L - 2;
+        if (!(pow7_sum(xl, X0, X1, X2, false) > thr_rej)) return -1;
+    }
     if constexpr (L > 3) {
         float lo1, hi1;
         beta_large_bounds<H, L - 1>(f, lo1, hi1);
         return select_large<H, L - 1>(f, lo1, hi1, tiny2, elo, ehi, x0, x1, x2, X0, X1, X2, thr,
-                                      thr_rej);
+                                      thr_rej, acc, rej);
     } else {
         return 0;
     }
@@ -338,10 +352,14 @@ __device__ __forceinline__ constexpr float sos_bound(int which)
 
 // First test of a reconstruction whose C_T exponent is not recorded: true
 // only if S_p is certain to be accepted, whatever the exponent (chi_p >= C_T
-// holds if sum_k (x_p / x_k)^7 <= 3 (x_p / min_k x_k)^7 <= thr[nexp_min]).
-// Most reconstructions of a resolved flow end here, so it uses no FP64
-// operation at all and few others; whatever it leaves open goes to
-// fast_decide.
+// holds if sum_k (x_p / x_k)^7 <= 3 (x_p / min_k x_k)^7 <= thr[nexp_min]), or
+// at the smooth exponent where eta >= C_r (m = 0) is certain.  Most
+// reconstructions of a resolved flow end here, so it uses no FP64 operation at
+// all and few others; whatever it leaves open goes to fast_decide.
+//
+// eta >= C_r: with e a bound of the differences' errors, 2 (|a| - e)(|b| - e) >=
+// C_r ((|a| + e)^2 + (|b| + e)^2) for the four pairs of neighbouring differences
+// (its epsilon only raises eta).
 //
 // The shifted values come from the bit patterns: every value, scaled by a
 // power of two to below 2, is cut exactly into h (24 bits) and l (the next
@@ -371,7 +389,7 @@ __device__ __forceinline__ bool quick_large(const double (&v)[2 * H], const Fast
     // every exponent within 100 of the largest: no zero, subnormal, NaN or infinity
     const bool range = ev >= 993u && ev <= 1072u && (hmin >> 20) + 100u >= ev;
     const unsigned eb = (ev - 127u) << 23;
-    float h0, l0, s[W];
+    float h0, lo0, s[W];
     // offset 0 first, then the others against it
 #pragma unroll
     for (int jj = 0; jj < W; jj++) {
@@ -384,10 +402,10 @@ __device__ __forceinline__ bool quick_large(const double (&v)[2 * H], const Fast
         const float h = __uint_as_float(hb);
         if (jj == 0) {
             h0 = h;
-            l0 = l;
+            lo0 = l;
             s[j] = 0.0f;
         } else {
-            s[j] = (h - h0) + (l - l0);
+            s[j] = (h - h0) + (l - lo0);
         }
     }
 #define SS(m) s[(m) + H - 1]
@@ -420,8 +438,23 @@ __device__ __forceinline__ bool quick_large(const double (&v)[2 * H], const Fast
     const float E = fmaf(sos_bound<H>(0) * M, sqrt_approx(bt),
                          fmaf(bt, (float)(n + 3) * 5.9604645e-8f, sos_bound<H>(1) * (M * M)));
     const float xp = fmaf(bt + E, 1.0f + 4.0e-6f, 2.0e-22f);
+    const float xs = (1.0f - 2.0e-6f) * xk;
+    // 2^-23 (|s| + |s|) + 2^-24 |difference| + 2^-43 for |s| <= m3, rounded up
+    const float m3 = fmaxf(ms, fabsf(SS(3))), e = fmaf(m3, 4.0e-7f, 1.2e-13f);
+    const float d0 = fabsf(SS(-1) - SS(-2)), d1 = fabsf(SS(-1)), d2 = fabsf(SS(1));
+    const float d3 = fabsf(SS(2) - SS(1)), d4 = fabsf(SS(3) - SS(2));
+    // the same test of each pair with its own sizes: q(a, b) >= 0
+    const float l0 = d0 - e, l1 = d1 - e, l2 = d2 - e, l3 = d3 - e, l4 = d4 - e;
+    const float u0 = d0 + e, u1 = d1 + e, u2 = d2 + e, u3 = d3 + e, u4 = d4 + e;
+    const float q0 = u0 * u0, q1 = u1 * u1, q2 = u2 * u2, q3 = u3 * u3, q4 = u4 * u4;
+    const float c = F.cr_up;
+    const bool smooth = fminf(fminf(l0, l1), fminf(l2, fminf(l3, l4))) > 0.0f &&
+                        2.0f * (l0 * l1) >= c * (q0 + q1) && 2.0f * (l1 * l2) >= c * (q1 + q2) &&
+                        2.0f * (l2 * l3) >= c * (q2 + q3) && 2.0f * (l3 * l4) >= c * (q3 + q4);
 #undef SS
-    return range && M >= 9.5367431640625e-7f && xp <= (F.rho * (1.0f - 2.0e-6f)) * xk;
+    const float rho = smooth ? fmaxf(F.rho_acc[F.nexp_min], F.rho_acc[F.nexp_smooth])
+                             : F.rho_acc[F.nexp_min];
+    return range && M >= 9.5367431640625e-7f && xp <= rho * xs;
 }
 
 // A small indicator's FP64 input as the exact path forms it, converted to
@@ -712,15 +745,13 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const Fast
     // the byte are then zero (the byte is not stored).
     float blo, bhi;                           // bounds of beta_p, for both tests
     beta_large_bounds<H, H>(o.f, blo, bhi);
-    if (!need_ct) {
-        // sum_k (x_p / x_k)^7 <= 3 (x_p / min_k x_k)^7: one division for the
-        // common case (a looser bound only sends borderline cases on)
-        const float r = __fdividef(x_upper(bhi, ebh), fminf(x0, fminf(x1, x2))) * (1.0f + 5e-7f);
-        const float q = r * r;
-        if (3.0f * (q * q * q * r) * (1.0f + 4e-6f) <= F.thr[F.nexp_min]) {
-            flag = (uint8_t)large_code(H);
-            return true;
-        }
+    const float xmin = fminf(x0, fminf(x1, x2)) * (1.0f - 2.0e-6f);
+    const float Xmin = fminf(X0, fminf(X1, X2)) * (1.0f + 2.0e-6f);
+    if (!need_ct && x_upper(bhi, ebh) <= F.rho_acc[F.nexp_min] * xmin) {
+        // sum_k (x_p / x_k)^7 <= 3 (x_p / min_k x_k)^7 <= thr (a looser bound only
+        // sends borderline cases on)
+        flag = (uint8_t)large_code(H);
+        return true;
     }
 
     // eta measure over cells -1..2 from the differences Delta_{m+1/2}, m=-2..2.
@@ -763,8 +794,9 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const Fast
     const float thr = F.thr[nexp], thr_rej = F.thr_rej[nexp];
 
     // Targeted selection, largest group first (Sec. 3.3).
+    const float acc = F.rho_acc[nexp], rej = F.rho_rej[nexp];
     const int sel = select_large<H, H>(o.f, blo, bhi, tiny2, ebl, ebh, x0, x1, x2, X0, X1, X2, thr,
-                                       thr_rej);
+                                       thr_rej, acc * xmin, rej * Xmin);
     if (sel < 0) return false;
     if (sel > 0) {
         if constexpr (H == 6)
@@ -782,7 +814,10 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const Fast
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             const int j1 = k == 0 ? 1 : 0, j2 = k == 2 ? 1 : 2;
-            if (pow7_sum2(xu[k], xl[j1], xl[j2], true) <= thr) d[k] = 1;
+            // as in select_large, with the two others' smaller one
+            if (xu[k] <= acc * (fminf(xl[j1], xl[j2]) * (1.0f - 2.0e-6f))) d[k] = 1;
+            else if (xl[k] >= rej * (fminf(xu[j1], xu[j2]) * (1.0f + 2.0e-6f))) d[k] = 0;
+            else if (pow7_sum2(xu[k], xl[j1], xl[j2], true) <= thr) d[k] = 1;
             else if (pow7_sum2(xl[k], xu[j1], xu[j2], false) > thr_rej) d[k] = 0;
             else return false;
         }
