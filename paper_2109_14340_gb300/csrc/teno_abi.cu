@@ -47,6 +47,8 @@ struct CombineArgs {
                              // next evaluation's input, with its non-physical
                              // cells counted here), or nullptr
     Status *st;
+    const double *dt_dev;    // RK modes: the time step, or nullptr for dt
+    double dt;
     int64_t n[3];
     int64_t ncell;
     int mode;                // 0: rhs, 1..3: RK stage 0..2
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(256) combine_kernel(CombineArgs a)
         double Uc[nc], Uo[nc];
 #pragma unroll
         for (int c = 0; c < nc; c++) Uc[c] = a.Uk[c * a.ncell + id];
-        const double dt = a.st->dt;
+        const double dt = a.dt_dev ? *a.dt_dev : a.dt;
 #pragma unroll
         for (int c = 0; c < nc; c++) {
             double acc = 0.0;
@@ -140,9 +142,11 @@ __global__ void __launch_bounds__(256) prims_kernel(const double *U, int64_t nce
 
 // A_d = max over cells of |u_d| + c, accumulated as bit patterns (the
 // ordering of non-negative doubles); NaN never enters.  Optionally counts
-// non-physical cells.
+// non-physical cells.  cfl > 0: the last block to add its maxima also forms the
+// time step dt = cfl / sum_d A_d / dx_d (written to the status block and *dt_out).
 template <int ND>
-__global__ void wave_max_kernel(const double *U, int64_t ncell, Consts K, Status *st, int count)
+__global__ void wave_max_kernel(const double *U, int64_t ncell, Consts K, Status *st, int count,
+                                double cfl, double3 inv_dx, double *dt_out, int accumulate)
 {
     constexpr int nc = ND + 2;
     double m[ND];
@@ -177,23 +181,27 @@ __global__ void wave_max_kernel(const double *U, int64_t ncell, Consts K, Status
         for (int o = 16; o > 0; o >>= 1) bad += __shfl_down_sync(0xffffffffu, bad, o);
         if ((threadIdx.x & 31) == 0 && bad) atomicAdd(&st->nonphys, bad);
     }
-}
-
-// dt = cfl / sum_d A_d / dx_d (written to *dt_out and the status block).
-__global__ void cfl_finalize_kernel(Status *st, int nd, double cfl, double3 inv_dx, double *dt_out,
-                                    int accumulate)
-{
-    const double idx[3] = {inv_dx.x, inv_dx.y, inv_dx.z};
-    double S = __longlong_as_double((long long)st->amax[0]) * idx[0];
-    for (int d = 1; d < nd; d++) S = S + __longlong_as_double((long long)st->amax[d]) * idx[d];
-    const double dt = cfl / S;
-    st->dt = dt;
-    if (dt_out) *dt_out = dt;
-    if (accumulate) st->t_accum = st->t_accum + dt;
+    if (!(cfl > 0.0)) return;
+    __threadfence();                       // this thread's maxima before the block's count
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&st->blocks, 1ull) == gridDim.x - 1) {
+        __threadfence();
+        const double idx[3] = {inv_dx.x, inv_dx.y, inv_dx.z};
+        double S = 0.0;
+#pragma unroll
+        for (int d = 0; d < ND; d++) {
+            const double A = __longlong_as_double((long long)atomicMax(&st->amax[d], 0ull));
+            S = d == 0 ? A * idx[0] : S + A * idx[d];
+        }
+        const double dt = cfl / S;
+        st->dt = dt;
+        if (dt_out) *dt_out = dt;
+        if (accumulate) st->t_accum = st->t_accum + dt;
+    }
 }
 
 // dt = cfl / sum_d A_d / dx_d with A_d the largest of ncopies rows of maxima
-// (sub-domains): the arithmetic of cfl_finalize_kernel on the combined maxima.
+// (sub-domains): the arithmetic of wave_max_kernel on the combined maxima.
 __global__ void dt_from_speeds_kernel(const double *amax, int ncopies, int nd, double cfl,
                                       double3 inv_dx, double *dt_out)
 {
@@ -209,8 +217,7 @@ __global__ void dt_from_speeds_kernel(const double *amax, int ncopies, int nd, d
     *dt_out = cfl / S;
 }
 
-// Stage preparation: dt from the host value or a device scalar, and the
-// limiter's effective dt/dx per direction: dt/dx in 1D; (dt S) / A_d with
+// Stage preparation: the limiter's effective dt/dx per direction: dt/dx in 1D; (dt S) / A_d with
 // S = sum_d A_d/dx_d in several dimensions (each direction's one-sided
 // updates get the share A_d/dx_d / S of the update).
 // The block also zeroes the stage's counters (one per chunk of the sweeps).
@@ -220,7 +227,6 @@ __global__ void prepare_kernel(Status *st, int nd, double dt_host, const double 
     for (int i = threadIdx.x; i < ncounters; i += blockDim.x) counters[i] = 0u;
     if (threadIdx.x) return;
     const double dt = dt_dev ? *dt_dev : dt_host;
-    st->dt = dt;
     if (!limiter) return;
     const double idx[3] = {inv_dx.x, inv_dx.y, inv_dx.z};
     if (nd == 1) {
@@ -433,25 +439,39 @@ static int grid_for(int64_t n, int block)
         if ((x) != cudaSuccess) return TENO_ECUDA;    \
     } while (0)
 
+static double3 inv_dx_of(const teno_params *p);
+
 static cudaError_t launch_wave_max(const teno_params *p, const double *U, Status *st,
-                                   int count, cudaStream_t s)
+                                   int count, cudaStream_t s, double cfl = 0.0,
+                                   double *dt_out = nullptr, int accumulate = 0)
 {
     const Consts K = consts_of(p);
     const int64_t N = ncells(p);
     const int blk = 256, grd = grid_for(N, blk);
-    cudaError_t e = cudaMemsetAsync(st->amax, 0, sizeof(st->amax), s);
+    const double3 idx = inv_dx_of(p);
+    static_assert(offsetof(Status, blocks) == offsetof(Status, amax) + sizeof(Status::amax), "zeroed together");
+    cudaError_t e = cudaMemsetAsync(st->amax, 0, sizeof(st->amax) + sizeof(st->blocks), s);
     if (e != cudaSuccess) return e;
-    if (p->ndim == 1) wave_max_kernel<1><<<grd, blk, 0, s>>>(U, N, K, st, count);
-    else if (p->ndim == 2) wave_max_kernel<2><<<grd, blk, 0, s>>>(U, N, K, st, count);
-    else wave_max_kernel<3><<<grd, blk, 0, s>>>(U, N, K, st, count);
+    if (p->ndim == 1) wave_max_kernel<1><<<grd, blk, 0, s>>>(U, N, K, st, count, cfl, idx, dt_out, accumulate);
+    else if (p->ndim == 2) wave_max_kernel<2><<<grd, blk, 0, s>>>(U, N, K, st, count, cfl, idx, dt_out, accumulate);
+    else wave_max_kernel<3><<<grd, blk, 0, s>>>(U, N, K, st, count, cfl, idx, dt_out, accumulate);
     return cudaGetLastError();
 }
 
-// Primitives of U into the workspace's primitive rows (non-physical cells
-// counted); returns their address.
-static cudaError_t launch_prims(const teno_params *p, const double *U, char *ws, cudaStream_t s,
-                                double **P_out)
+// Whether an evaluation takes the single launch for few tiles: its tiles stage
+// (and count) the cells themselves, so it needs no stored primitives.
+static bool small_path(const teno_params *p, const void *frozen)
 {
+    return !frozen && small_evaluation(all_tiles(p), p->ndim, p->scheme / 2);
+}
+
+// Primitives of U into the workspace's primitive rows (non-physical cells
+// counted); returns their address (nullptr where the sweeps need none).
+static cudaError_t launch_prims(const teno_params *p, const double *U, char *ws, cudaStream_t s,
+                                double **P_out, const void *frozen = nullptr)
+{
+    *P_out = nullptr;
+    if (small_path(p, frozen)) return cudaSuccess;
     NvtxRange range("teno primitives");
     const Layout L = layout(p);
     Status *st = (Status *)(ws + L.status);
@@ -513,7 +533,9 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
     const int nd = p->ndim, nc = ncons(p);
     const SweepMem M = sm ? *sm : sweep_mem(p, ws + L.sweep, kChunkTiles);
     if (p->limiter && nd > 1) CUDA_TRY(launch_wave_max(p, Uk, st, 0, s));
-    prepare_kernel<<<1, M.nchunks > 32 ? 256 : 32, 0, s>>>(st, nd, dt_host, dt_dev, idx, p->limiter,
+    const int small = small_path(p, frozen);
+    if (!small || p->limiter)         // counters to zero, the limiter's dt/dx
+        prepare_kernel<<<1, M.nchunks > 32 ? 256 : 32, 0, s>>>(st, nd, dt_host, dt_dev, idx, p->limiter,
                                                          M.counters, (int)M.nchunks);
     CUDA_TRY(cudaGetLastError());
     uint8_t *fl = flags;
@@ -539,6 +561,7 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
                                       // unless its primitives were stored
     a.g.limiter = p->limiter;
     a.g.tag = 0;
+    a.small = small;
     a.exact_count = g_prof.on ? g_prof.exact : nullptr;
     a.FK = fastk_of(p);
     a.K = K;
@@ -618,6 +641,8 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
     c.out = out;
     c.P = P_out;
     c.st = st;
+    c.dt_dev = dt_dev;
+    c.dt = dt_host;
     for (int k = 0; k < 3; k++) c.n[k] = p->n[k];
     c.ncell = ncells(p);
     c.mode = mode;
@@ -756,7 +781,7 @@ int teno_rhs_frozen(const teno_params *p, const double *U, double *rhs, double d
     if (p->limiter && !(dt_limiter >= 0.0)) return TENO_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     double *P = nullptr;
-    CUDA_TRY(launch_prims(p, U, (char *)ws, s, &P));
+    CUDA_TRY(launch_prims(p, U, (char *)ws, s, &P, decisions));
     return stage(p, U, U, rhs, 0, dt_limiter, nullptr, nullptr, (char *)ws, s, decisions, P,
                  nullptr);
 }
@@ -774,7 +799,7 @@ int teno_rk3_step_frozen(const teno_params *p, double *U, double dt, const uint8
     double *Us = (double *)((char *)ws + L.stage);
     cudaStream_t s = (cudaStream_t)stream;
     double *P = nullptr;
-    CUDA_TRY(launch_prims(p, U, (char *)ws, s, &P));
+    CUDA_TRY(launch_prims(p, U, (char *)ws, s, &P, decisions));
     if ((r = stage(p, U, U, Us, 1, dt, nullptr, nullptr, (char *)ws, s, decisions, P, P))) return r;
     if ((r = stage(p, Us, U, Us, 2, dt, nullptr, nullptr, (char *)ws, s, decisions + flb, P, P)))
         return r;
@@ -792,9 +817,7 @@ int teno_cfl_dt(const teno_params *p, const double *U, double cfl, double *dt_de
     Status *st = (Status *)((char *)ws + layout(p).status);
     cudaStream_t s = (cudaStream_t)stream;
     NvtxRange range("teno cfl dt");
-    CUDA_TRY(launch_wave_max(p, U, st, 0, s));
-    cfl_finalize_kernel<<<1, 1, 0, s>>>(st, p->ndim, cfl, inv_dx_of(p), dt_device, 0);
-    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(launch_wave_max(p, U, st, 0, s, cfl, dt_device));
     return TENO_OK;
 }
 
@@ -808,7 +831,7 @@ int teno_rk3_stage(const teno_params *p, int stage_k, double *U, double *Us, dou
     if (stage_k < 1 || stage_k > 3 || ws_bytes < layout(p).total) return TENO_EINVAL;
     if (!dt_device && !(dt >= 0.0)) return TENO_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    double *P = (double *)((char *)ws + layout(p).prims);
+    double *P = small_path(p, nullptr) ? nullptr : (double *)((char *)ws + layout(p).prims);
     // the stages of teno_rk3_step, the primitives carried in the workspace
     if (stage_k == 1) {
         CUDA_TRY(launch_prims(p, U, (char *)ws, s, &P));
@@ -878,9 +901,7 @@ int teno_advance_host(const teno_params *p, double *U_host, double *U_dev, int n
     CUDA_TRY(cudaMemcpyAsync(U_dev, U_host, bytes, cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaMemsetAsync(&st->t_accum, 0, sizeof(double), s));
     for (int k = 0; k < nsteps; k++) {
-        CUDA_TRY(launch_wave_max(p, U_dev, st, 0, s));
-        cfl_finalize_kernel<<<1, 1, 0, s>>>(st, p->ndim, cfl, inv_dx_of(p), nullptr, 1);
-        CUDA_TRY(cudaGetLastError());
+        CUDA_TRY(launch_wave_max(p, U_dev, st, 0, s, cfl, nullptr, 1));
         if ((r = teno_rk3_step(p, U_dev, 0.0, &st->dt, ws, ws_bytes, stream))) return r;
     }
     CUDA_TRY(cudaMemcpyAsync(U_host, U_dev, bytes, cudaMemcpyDeviceToHost, s));

@@ -16,12 +16,13 @@ namespace teno {
 struct Status {
     unsigned long long nonphys;    // non-physical cells + faces (teno_status)
     unsigned long long amax[3];    // bit patterns of A_d = max(|u_d| + c) >= 0
+    unsigned long long blocks;     // blocks that have added theirs (zeroed with amax)
     double dt;                     // time step of the current call
     double lam[3];                 // limiter: effective dt/dx of each direction
     double t_accum;                // summed dt of teno_advance_host
     unsigned long long oob_count;  // debug build: out-of-range accesses skipped
     long long oob_line, oob_index, oob_extent;   // the first one's source line, index, extent
-    double pad[19];
+    double pad[18];
 };
 static_assert(sizeof(Status) == 256, "status block is 256 bytes");
 

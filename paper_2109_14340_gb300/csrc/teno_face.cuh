@@ -124,6 +124,7 @@ struct SweepArgs {
     DirArgs dir[3];
     SweepPart part[3];
     int32_t nparts, tiles;
+    int small;                         // 1: the single launch for few tiles
     unsigned *nexact;                  // length of the exact path's list (zeroed beforehand)
     unsigned long long *exact_count;   // adds the exact-path reconstructions, or nullptr
     SweepBuf buf;
@@ -151,6 +152,17 @@ inline void tile_shape(DirArgs &d, int64_t faces, int64_t pencils, int H)
         }
         if (pencils == 1) break;
     }
+}
+
+// Whether an evaluation of so many tiles takes the single launch (small_kernel)
+// rather than the four kernels.  Measured per right-hand side, four kernels
+// against one: 1D 400 cells 58 against 34 us, 100 000 cells (3126 tiles) 163
+// against 154; 2D ten-point 128^2 (1088 tiles) 123 against 110, 256^2 (4200) 314
+// against 316; 2D twelve-point 96^2 (620) 124 against 107, 160^2 (1640) 151
+// against 183; 3D 20^3 (900) 131 against 138, 28^3 216 against 289.
+inline bool small_evaluation(int64_t tiles, int nd, int H)
+{
+    return tiles <= (nd == 1 ? 4096 : (nd == 2 ? (H == 6 ? 1024 : 3072) : 512));
 }
 
 // Tile t of direction D: first face f0 and the position of its first pencil.  x
@@ -305,30 +317,23 @@ __device__ __forceinline__ double half_of(double x)
 // limrec), and one that applies recorded decisions (frozen, frozen_argmax).
 enum { kSweepPlain = 0, kSweepRecord = 1, kSweepFrozen = 2 };
 
-// One tile by one warp: the faces from f0 along D of the pencils from (x, y, z);
-// tile: its index in the chunk's buffers; sm: the warp's slice.  Every lane of
-// the warp calls it; it returns with the warp in step, its values, queue and
-// Roe states in the buffers.
-template <int ND, int H, int D, int MODE>
-__device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da, const FastK &FK,
-                                           const Consts &K, const SweepBuf &B, int64_t f0, int64_t x,
-                                           int64_t y, int64_t z, int64_t tile, double *sm)
+// Stages the cells of a tile from f0-H along D, pencil by pencil in the x sweep,
+// pencils side by side in the others: cells first, first + step, ...
+template <int ND, int H, int D>
+__device__ __forceinline__ void stage_cells(const GridArgs &a, const DirArgs &da, const Consts &K,
+                                            int64_t f0, int64_t x, int64_t y, int64_t z, double *sm,
+                                            int first, int step)
 {
     using SL = FaceSmem<ND, H>;
-    constexpr int nc = ND + 2, last = nc - 1, W = 2 * H, NS = SL::NS;
-    const int lane = threadIdx.x & 31;
+    constexpr int nc = ND + 2, last = nc - 1, NS = SL::NS;
     double2 *UF = (double2 *)sm;
 #define TMP(q, j) sm[SL::TMP + (q) * NS + (j)]
-
     const int64_t n0 = a.n[0], n1 = a.n[1], nD = a.n[D];
     const int tps = ND == 1 ? 0 : da.tps, tp = 1 << tps;
     const int nsf = (kTileFaces >> tps) + 2 * H - 1;   // cells of one pencil
     const int64_t npen = D == 0 ? n1 - y : n0 - x;     // pencils from the first one on
     const int64_t cstride = D == 0 ? 1 : (D == 1 ? n0 : n0 * n1);
-
-    // Stage the cells from f0-H along D, pencil by pencil in the x sweep, pencils
-    // side by side in the others.
-    for (int idx = lane; idx < tp * nsf; idx += 32) {
+    for (int idx = first; idx < tp * nsf; idx += step) {
         int j, pp;
         if (D == 0) {
             pp = (idx >= nsf) + (idx >= 2 * nsf) + (idx >= 3 * nsf);
@@ -401,6 +406,30 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
         TMP(SL::QLP, idx) = fabs(vd + cj);
         TMP(SL::QLR, idx) = fabs(vd) + cj;
     }
+#undef TMP
+}
+
+// One tile by one warp: the faces from f0 along D of the pencils from (x, y, z);
+// tile: its index in the chunk's buffers; sm: the warp's slice.  Every lane of
+// the warp calls it; it returns with the warp in step, its values, queue and
+// Roe states in the buffers.
+template <int ND, int H, int D, int MODE>
+__device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da, const FastK &FK,
+                                           const Consts &K, const SweepBuf &B, int64_t f0, int64_t x,
+                                           int64_t y, int64_t z, int64_t tile, double *sm)
+{
+    using SL = FaceSmem<ND, H>;
+    constexpr int nc = ND + 2, last = nc - 1, W = 2 * H, NS = SL::NS;
+    const int lane = threadIdx.x & 31;
+    double2 *UF = (double2 *)sm;
+#define TMP(q, j) sm[SL::TMP + (q) * NS + (j)]
+
+    const int64_t nD = a.n[D];
+    const int tps = ND == 1 ? 0 : da.tps, tp = 1 << tps;
+    const int nsf = (kTileFaces >> tps) + 2 * H - 1;   // cells of one pencil
+    const int64_t npen = D == 0 ? a.n[1] - y : a.n[0] - x;     // pencils from the first one on
+
+    stage_cells<ND, H, D>(a, da, K, f0, x, y, z, sm, lane, 32);
     __syncwarp();
 
     int p, fo;
@@ -546,7 +575,7 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
 
 // Back-projection of a face, the limiter, and what it leaves: the flux, the
 // limiter's byte and the decision bytes of the record.
-template <int ND, int D, int MODE>
+template <int ND, int D, int MODE, bool BYTES = true>
 __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, const Consts &K,
                                             const SweepBuf &B, int64_t cf, int64_t flin, Status *st)
 {
@@ -638,7 +667,7 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
         da.limrec[flin] = 0;
     }
 
-    if constexpr (MODE == kSweepRecord) {
+    if constexpr (MODE == kSweepRecord && BYTES) {
 #pragma unroll
         for (int q = 0; q < 2 * nc; q++) da.flags[flin * nc * 2 + q] = B.RD[q * nf + cf];
     }
@@ -683,16 +712,22 @@ __global__ void __launch_bounds__(32 * kSweepWarps, kSweepBlocks<H>) sweep_kerne
     }
 }
 
-// The queued reconstructions of `group` consecutive tiles, by `split` warps that
-// take every split-th round of 32 entries.  A round takes one entry per lane
-// through the filter; its outcomes gather by kind in shared memory, and a
-// kind's values are evaluated when it has a warp's worth, the rest at the end.
-// Few tiles per warp and split > 1 shorten a small evaluation, many fill the
-// lanes of a large one.  RECORD: decision bytes are kept.  mixed: 0, or in a
-// batch of both schemes 1 for the tiles whose length has no top bit, 2 for
-// those that have it.
-constexpr int kDecideWarps = 4, kDecideMostTiles = 16;
+// What the decide and exact kernels need beside the buffers.  Arguments of both
+// schemes of a batch; a single problem uses one.
+struct DecideArgs {
+    SweepBuf B;
+    int32_t tiles;
+    int nc, fast, need_ct;
+    int group, split;      // tiles per warp, warps per group of tiles
+    unsigned *nexact[2];   // lengths of the exact path's lists (zeroed beforehand),
+    uint32_t *xlist[2];    // one per scheme
+    unsigned long long *exact_count;   // adds the exact-path reconstructions, or nullptr
+    Status *st;
+    FastK FK;
+    Consts K;
+};
 
+// A decided entry's value, to its owner's place.
 template <int H, bool RECORD>
 __device__ __forceinline__ void decided_out(const SweepBuf &B, int64_t nq, int64_t nf, uint32_t per,
                                             bool fallback, uint32_t q, uint8_t f, int nc, Status *st)
@@ -709,27 +744,32 @@ __device__ __forceinline__ void decided_out(const SweepBuf &B, int64_t nq, int64
     if (RECORD) B.RD[o] = f;
 }
 
+constexpr int kDecideWarps = 4, kDecideMostTiles = 16;
+
+// The queued reconstructions of `group` consecutive tiles, by `split` warps that
+// take every split-th round of 32 entries.  A round takes one entry per lane
+// through the filter; its outcomes gather by kind in shared memory, and a
+// kind's values are evaluated when it has a warp's worth, the rest at the end.
+// Few tiles per warp and split > 1 shorten a small evaluation, many fill the
+// lanes of a large one.  RECORD: decision bytes are kept.  mixed: -1, or in a
+// batch of both schemes the top bit of the lengths of the tiles to take.
 template <int H, bool RECORD>
-__global__ void __launch_bounds__(32 * kDecideWarps, 6) decide_kernel(
-    const SweepBuf B, int32_t tiles, int group, int split, int nc, int fast, int need_ct, int mixed,
-    unsigned *nexact, const FastK FK, Status *st)
+__device__ __forceinline__ void decide_unit(const DecideArgs &a, int64_t unit, int mixed,
+                                            uint32_t (*list)[64], uint8_t (*code)[64])
 {
     constexpr int W = 2 * H;
-    __shared__ uint32_t list_[kDecideWarps][2][64];    // gathered entries: large stencil, fallback
-    __shared__ uint8_t code_[kDecideWarps][2][64];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t(*list)[64] = list_[warp];
-    uint8_t(*code)[64] = code_[warp];
-    const int64_t unit = (int64_t)blockIdx.x * kDecideWarps + warp;
+    const SweepBuf &B = a.B;
+    const int lane = threadIdx.x & 31, nc = a.nc, group = a.group, split = a.split;
     const int64_t t0 = unit / split * group;
-    if (t0 >= tiles) return;
+    if (t0 >= a.tiles) return;
     const uint32_t per = 64u * nc;
     const int64_t nq = B.nt * per, nf = B.nt * kTileFaces;
+    const int which = mixed > 0;
     // entries before each tile of the group: lane i holds tile i's
     int before = 0, total;
     {
-        uint32_t c = lane < group && t0 + lane < tiles ? B.count[t0 + lane] : 0u;
-        if (mixed && (c >> 31) != (uint32_t)(mixed == 2)) c = 0u;
+        uint32_t c = lane < group && t0 + lane < a.tiles ? B.count[t0 + lane] : 0u;
+        if (mixed >= 0 && (int)(c >> 31) != mixed) c = 0u;
         int sum = (int)(c & 0x7fffffffu);
         const int own = sum;
 #pragma unroll
@@ -754,11 +794,11 @@ __global__ void __launch_bounds__(32 * kDecideWarps, 6) decide_kernel(
         uint8_t fl = 0;
         if (e < total) {
             kind = 2;
-            if (fast && TENO_IN(st, q, nq)) {
+            if (a.fast && TENO_IN(a.st, q, nq)) {
                 double v[W];
 #pragma unroll
                 for (int kk = 0; kk < W; kk++) v[kk] = B.qv[kk * nq + q];
-                if (fast_decide<H>(v, FK, fl, need_ct != 0))
+                if (fast_decide<H>(v, a.FK, fl, a.need_ct != 0))
                     kind = (fl & 3) != 0 || (H == 6 && (fl & 31) == 0) ? 0 : 1;
             }
         }
@@ -775,9 +815,9 @@ __global__ void __launch_bounds__(32 * kDecideWarps, 6) decide_kernel(
         n1 += __popc(m1);
         if (m2) {
             int at = 0;
-            if (lane == 0) at = (int)atomicAdd(nexact, __popc(m2));
+            if (lane == 0) at = (int)atomicAdd(a.nexact[which], __popc(m2));
             at = __shfl_sync(0xffffffffu, at, 0) + __popc(m2 & below);
-            if (kind == 2 && TENO_IN(st, at, nq)) B.xlist[at] = q;
+            if (kind == 2 && TENO_IN(a.st, at, nq)) a.xlist[which][at] = q;
         }
         __syncwarp();
         const bool end = base + 32 * split >= total;
@@ -785,44 +825,226 @@ __global__ void __launch_bounds__(32 * kDecideWarps, 6) decide_kernel(
             const int n = min(n0, 32);
             n0 -= n;
             if (lane < n)
-                decided_out<H, RECORD>(B, nq, nf, per, false, list[0][n0 + lane], code[0][n0 + lane], nc, st);
+                decided_out<H, RECORD>(B, nq, nf, per, false, list[0][n0 + lane], code[0][n0 + lane], nc, a.st);
         }
         if (n1 >= 32 || (end && n1 > 0)) {
             const int n = min(n1, 32);
             n1 -= n;
             if (lane < n)
-                decided_out<H, RECORD>(B, nq, nf, per, true, list[1][n1 + lane], code[1][n1 + lane], nc, st);
+                decided_out<H, RECORD>(B, nq, nf, per, true, list[1][n1 + lane], code[1][n1 + lane], nc, a.st);
         }
         __syncwarp();
     }
     // at most 31 of a kind are left after the last round's pass
-    if (lane < n0) decided_out<H, RECORD>(B, nq, nf, per, false, list[0][lane], code[0][lane], nc, st);
-    if (lane < n1) decided_out<H, RECORD>(B, nq, nf, per, true, list[1][lane], code[1][lane], nc, st);
+    if (lane < n0) decided_out<H, RECORD>(B, nq, nf, per, false, list[0][lane], code[0][lane], nc, a.st);
+    if (lane < n1) decided_out<H, RECORD>(B, nq, nf, per, true, list[1][lane], code[1][lane], nc, a.st);
 }
 
-// The listed reconstructions through the exact path.
-template <int H, bool RECORD>
-__global__ void __launch_bounds__(128) exact_kernel(SweepBuf B, int nc, const unsigned *nexact,
-                                                    unsigned long long *exact_count,
-                                                    const Consts K, Status *st)
+// MIX = 0: scheme 2 H; 1: a batch of eight- and ten-point problems, every other
+// unit for each scheme.
+template <int H, bool RECORD, int MIX>
+__global__ void __launch_bounds__(32 * kDecideWarps, 6) decide_kernel(const DecideArgs a, int mixed)
+{
+    __shared__ uint32_t list_[kDecideWarps][2][64];    // gathered entries: large stencil, fallback
+    __shared__ uint8_t code_[kDecideWarps][2][64];
+    const int warp = threadIdx.x >> 5;
+    const int64_t unit = (int64_t)blockIdx.x * kDecideWarps + warp;
+    if constexpr (MIX == 0) {
+        decide_unit<H, RECORD>(a, unit, mixed, list_[warp], code_[warp]);
+    } else if (unit & 1) {
+        decide_unit<5, RECORD>(a, unit >> 1, 1, list_[warp], code_[warp]);
+    } else {
+        decide_unit<4, RECORD>(a, unit >> 1, 0, list_[warp], code_[warp]);
+    }
+}
+
+// One reconstruction through the exact path by a whole warp, bitwise
+// teno_recon: an FP64 instruction costs the warp the same for one lane as for
+// 32, and a lane on its own goes through some 280 of them, 17 divisions
+// among them.  Here the rows of the quadratic forms, the four eta_j, the
+// small indicators, the separations gamma and the chi run side by side, about
+// 100 instructions in all.  Lanes 0 .. 2H-2 hold the rows of S_H's form, the
+// next 2H-3 those of S_(H-1), and so on (32 in all for H = 6); qc: the lane's
+// row of coefficients.  Every lane returns the value.
+// first lane of S_L's rows
+template <int H>
+__host__ __device__ constexpr int exact_first(int L)
+{
+    int f = 0;
+    for (int l = H; l > L; l--) f += 2 * l - 1;
+    return f;
+}
+
+template <int H, int L>
+__device__ __forceinline__ void exact_row(int lane, int &row, double (&qc)[2 * H])
+{
+    constexpr int f = exact_first<H>(L), n = 2 * L - 1;
+    if (lane >= f && lane < f + n) {
+        // rows in ascending offset without offset 0 (index L - 1)
+        const int r = lane - f + (lane - f >= L - 1 ? 1 : 0);
+        row = r + (H - L);                             // its value index in the 2H stencil
+#pragma unroll
+        for (int c = 0; c < 2 * L; c++) {
+            double q = 0.0;
+#pragma unroll
+            for (int rr = 0; rr <= c; rr++)
+                if (rr == r) q = qcoef<L>(rr, c);
+            qc[c + H - L] = q;
+        }
+    }
+    if constexpr (L > 3) exact_row<H, L - 1>(lane, row, qc);
+}
+
+// The sum over the rows, in order, as beta_large_s forms it.
+template <int H, int L>
+__device__ __forceinline__ double exact_sum(double sr, double inner)
+{
+    constexpr int f = exact_first<H>(L);
+    double acc = 0.0;
+#pragma unroll
+    for (int i = 0; i < 2 * L - 1; i++) {
+        const double s = __shfl_sync(0xffffffffu, sr, f + i);
+        const double t = __shfl_sync(0xffffffffu, inner, f + i);
+        acc = i == 0 ? s * t : fma(s, t, acc);
+    }
+    return acc;
+}
+
+template <int H>
+__device__ __forceinline__ double exact_warp(const double (&v)[2 * H], int row, const double (&qc)[2 * H],
+                                             const Consts &K, uint8_t &flag)
 {
     constexpr int W = 2 * H;
+    const unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+#define V(m) v[(m) + H - 1]
+    // rows: inner_r = q_rr s_r + sum_{c > r} q_rc s_c, ascending c, offset 0 left out
+    double sr = 0.0, inner = 0.0;
+    bool begun = false;
+#pragma unroll
+    for (int c = 0; c < W; c++) {
+        if (c == H - 1) continue;
+        const double s = v[c] - V(0);
+        if (c == row) {
+            sr = s;
+            inner = qc[c] * s;
+            begun = true;
+        } else if (begun && c < W) {
+            const double t = fma(qc[c], s, inner);
+            inner = qc[c] != 0.0 ? t : inner;          // beyond the row's stencil: no term
+        }
+    }
+    double b3 = exact_sum<H, 3>(sr, inner), b4 = exact_sum<H, 4>(sr, inner), b5 = 0.0, b6 = 0.0;
+    if constexpr (H >= 5) b5 = exact_sum<H, 5>(sr, inner);
+    if constexpr (H >= 6) b6 = exact_sum<H, 6>(sr, inner);
+    // small indicators k = 0, 1, 2: b = (x - 2 y) + z; a_0 = V(-1) - V(1),
+    // a_1 = (3 V(0) - 4 V(1)) + V(2), a_2 = (V(-2) - 4 V(-1)) + 3 V(0)
+    const int k3 = lane % 3;
+    const double t3 = 3.0 * V(0);
+    const double ax = k3 == 0 ? V(-1) : (k3 == 1 ? t3 : V(-2));
+    const double ay = k3 == 2 ? V(-1) : V(1);
+    const double ab = fma(k3 == 0 ? -1.0 : -4.0, ay, ax);
+    const double az = k3 == 1 ? V(2) : t3;
+    const double a = k3 == 0 ? ab : ab + az;
+    const double bx = k3 == 0 ? V(-1) : (k3 == 1 ? V(0) : V(-2));
+    const double by = k3 == 0 ? V(0) : (k3 == 1 ? V(1) : V(-1));
+    const double bz = k3 == 0 ? V(1) : (k3 == 1 ? V(2) : V(0));
+    const double b = fma(-2.0, by, bx) + bz;
+    const double bs = 0.25 * (a * a) + (13.0 / 12.0) * (b * b);
+    // lanes 0-2: gamma of the small stencils; 3..H: of S_3..S_H; 8-11: eta_j, j = -1..2
+    const int j = (lane & 3) - 1;
+    const double vp = j < 0 ? V(0) : (j == 0 ? V(1) : (j == 1 ? V(2) : V(3)));
+    const double vo = j < 0 ? V(-1) : (j == 0 ? V(0) : (j == 1 ? V(1) : V(2)));
+    const double vn = j < 0 ? V(-2) : (j == 0 ? V(-1) : (j == 1 ? V(0) : V(1)));
+    const double dp = vp - vo, dm = vo - vn;
+    const double num = fabs((2.0 * dp) * dm) + K.eps_eta;
+    const double den = (dp * dp + dm * dm) + K.eps_eta;
+    const double beta = lane < 3 ? bs : (lane == 3 ? b3 : (lane == 4 ? b4 : (lane == 5 ? b5 : b6)));
+    const double x = beta + K.eps_beta, x2 = x * x, x4 = x2 * x2, x7 = (x4 * x2) * x;
+    const bool eta = lane >= 8;
+    const double q1 = (eta ? num : 1.0) / (eta ? den : x7);
+    const double g0 = __shfl_sync(all, q1, 0), g1 = __shfl_sync(all, q1, 1), g2 = __shfl_sync(all, q1, 2);
+    double emin = __shfl_sync(all, q1, 8);
+#pragma unroll
+    for (int i = 1; i < 4; i++) {
+        const double e = __shfl_sync(all, q1, 8 + i);
+        if (e < emin) emin = e;
+    }
+    const double g012 = (g0 + g1) + g2;
+    // lanes 0-2: g_k / g012; 3..H: chi of S_3..S_H; 8: eta / C_r
+    const double q2 = (eta ? emin : q1) / (eta ? K.cr : (lane < 3 ? g012 : g012 + q1));
+    const double r = __shfl_sync(all, q2, 8);
+    const double m = 1.0 - (r < 1.0 ? r : 1.0);
+    const double om = 1.0 - m, om2 = om * om;
+    const double g = (om2 * om2) * (1.0 + 4.0 * m);
+    const double bct = K.alpha1 - K.alpha2 * (1.0 - g);
+    const double fln = floor(bct);
+    const int nexp = fln < 0.0 ? 0 : (fln > 22.0 ? 22 : (int)fln);
+    const unsigned keep = __ballot_sync(all, !(q2 < TENO_TENPOW[nexp]));
+    const uint8_t fct = (uint8_t)(((nexp - 7) & 7) << 5);
+    int sel = 0;
+#pragma unroll
+    for (int L = 3; L <= H; L++)
+        if (keep >> L & 1u) sel = L;
+    if (sel) {
+        flag = (uint8_t)(large_code(sel) | fct);
+        return large_value<H>(v, sel);
+    }
+    flag = (uint8_t)((keep & 7u) << 2 | fct);
+    return fallback_value<H>(v, (int)(keep & 7u));
+#undef V
+}
+
+// The listed reconstructions through the exact path: a warp for each while they
+// are few (at most kExactFew), a lane for each when they fill warps.
+constexpr unsigned kExactFew = 152 * 16;
+
+template <int H, bool RECORD>
+__device__ __forceinline__ void exact_list(const DecideArgs &a, int which, unsigned block, unsigned blocks)
+{
+    constexpr int W = 2 * H;
+    const SweepBuf &B = a.B;
+    const int nc = a.nc;
     const int64_t per = 64 * nc, nq = B.nt * per, nf = B.nt * kTileFaces;
-    const unsigned n = *nexact;
-    if (exact_count && blockIdx.x == 0 && threadIdx.x == 0 && n)
-        atomicAdd(exact_count, (unsigned long long)n);
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const uint32_t q = B.xlist[i];
-        if (!TENO_IN(st, q, nq)) continue;
+    const unsigned n = *a.nexact[which];
+    if (n == 0) return;
+    if (a.exact_count && block == 0 && threadIdx.x == 0)
+        atomicAdd(a.exact_count, (unsigned long long)n);
+    const bool few = n <= kExactFew;
+    int row = -1;
+    double qc[W];
+#pragma unroll
+    for (int c = 0; c < W; c++) qc[c] = 0.0;           // beyond the row's stencil
+    if (few) exact_row<H, H>(threadIdx.x & 31, row, qc);
+    const unsigned step = few ? blocks * (blockDim.x >> 5) : blocks * blockDim.x;
+    for (unsigned i = few ? block * (blockDim.x >> 5) + (threadIdx.x >> 5) : block * blockDim.x + threadIdx.x;
+         i < n; i += step) {
+        const uint32_t q = a.xlist[which][i];
+        if (!TENO_IN(a.st, q, nq)) continue;
         double v[W];
 #pragma unroll
         for (int kk = 0; kk < W; kk++) v[kk] = B.qv[kk * nq + q];
         const int slot = B.qslot[q];
         const int64_t o = (slot >> 5) * nf + (int64_t)(q / (uint32_t)per) * kTileFaces + (slot & 31);
-        if (!TENO_IN(st, o, 2 * nc * nf)) continue;
+        if (!TENO_IN(a.st, o, 2 * nc * nf)) continue;
         uint8_t fl;
-        B.R[o] = teno_recon<H>(v, K, fl);
-        if (RECORD) B.RD[o] = fl;
+        const double val = few ? exact_warp<H>(v, row, qc, a.K, fl) : teno_recon<H>(v, a.K, fl);
+        if (!few || (threadIdx.x & 31) == 0) {
+            B.R[o] = val;
+            if (RECORD) B.RD[o] = fl;
+        }
+    }
+}
+
+template <int H, bool RECORD, int MIX>
+__global__ void __launch_bounds__(128) exact_kernel(const DecideArgs a, int which)
+{
+    if constexpr (MIX == 0) {
+        exact_list<H, RECORD>(a, which, blockIdx.x, gridDim.x);
+    } else if (blockIdx.x & 1) {
+        exact_list<5, RECORD>(a, 1, blockIdx.x >> 1, gridDim.x >> 1);
+    } else {
+        exact_list<4, RECORD>(a, 0, blockIdx.x >> 1, gridDim.x >> 1);
     }
 }
 
@@ -860,23 +1082,296 @@ __global__ void __launch_bounds__(128) finish_kernel(const SweepArgs a)
     }
 }
 
-// The decide and exact kernels of one chunk.
-template <int H, bool RECORD>
-cudaError_t launch_decisions(const SweepBuf &B, int32_t tiles, int nc, int fast, int need_ct, int mixed,
-                             unsigned *nexact, unsigned long long *exact_count, const FastK &FK,
-                             const Consts &K, Status *st, cudaStream_t s)
+// Few tiles: a block per tile, a warp per field and sign, everything in one
+// launch.  Where tiles do not fill the chip, what counts is the longest chain
+// of one warp: a lane of the sweep goes through all fields one after the other
+// (some 390 FP64 instructions in 1D, 64 cycles each), and the decide, exact and
+// finish kernels follow it with a launch each.  Here the warps share a tile's
+// fields and signs: Roe state and splitting speeds by one warp each, w by the
+// f+ warp of a field and g by its f- warp, then each its reconstruction.  Lanes
+// of a warp may want different kinds of value, which costs FP64 instructions
+// that the four kernels save: those are the better ones for more tiles.
+template <int ND, int H>
+struct SmallSmem {
+    static constexpr int nc = ND + 2, W = 2 * H;
+    static constexpr int NW = 2 * nc;                  // warps
+    static constexpr int CELLS = 0;                    // FaceSmem
+    static constexpr int ROE = FaceSmem<ND, H>::TOTAL; // [nd + 9][32] Roe scalars, finish's rows first
+    static constexpr int SPD = ROE + (ND + 9) * 32;    // [4][32] splitting speeds
+    static constexpr int PRJ = SPD + 4 * 32;           // [2 nc][W][32] halved w and g
+    static constexpr int VAL = PRJ + NW * W * 32;      // [2 nc][32] values
+    static constexpr int BYTES = 8 * (VAL + NW * 32);
+    // the limiter's rows [4 nc + 1][32] take the projections' room once those were read
+    static_assert(4 * nc + 1 <= NW * W, "limiter rows fit in the projections' room");
+};
+
+// Roe state, its rows for the projections and the finish, and the splitting
+// speeds of a tile: warp 0 the first, warps 1-4 a speed each.
+template <int ND, int H, int D, int MODE>
+__device__ __forceinline__ void small_states(const GridArgs &a, const DirArgs &da, const Consts &K,
+                                             int warp, int b0, int bs, bool active, int64_t flin,
+                                             double *sm, uint16_t *arg)
 {
-    // at least four waves of warps (24 on each of 152 SMs) before tiles share one
-    const int64_t fill = 152 * 24;
-    int group = 1, split = 1;
-    while (group < kDecideMostTiles && tiles >= 8 * fill * group) group *= 2;
-    while (group == 1 && split < 2 * nc && (int64_t)tiles * split * 2 <= fill) split *= 2;
-    const int64_t units = (int64_t)((tiles + group - 1) / group) * split;
-    decide_kernel<H, RECORD><<<(unsigned)((units + kDecideWarps - 1) / kDecideWarps), 32 * kDecideWarps, 0, s>>>(
-        B, tiles, group, split, nc, fast, need_ct, mixed, nexact, FK, st);
-    const int64_t most = (int64_t)tiles * nc / 2;         // blocks of 128 for every entry
-    exact_kernel<H, RECORD><<<(unsigned)(most < 608 ? (most ? most : 1) : 608), 128, 0, s>>>(
-        B, nc, nexact, exact_count, K, st);
+    using SL = FaceSmem<ND, H>;
+    using SS = SmallSmem<ND, H>;
+    constexpr int W = 2 * H, NS = SL::NS;
+    const int lane = threadIdx.x & 31;
+#define TMP(q, j) sm[SL::TMP + (q) * NS + (j)]
+    if (!active) return;
+    if (warp == 0) {
+        const int bl = b0 + (H - 1) * bs, br = bl + bs;
+        RoeScalars<ND> rs;
+        double ul[ND], ur[ND];
+#pragma unroll
+        for (int k = 0; k < ND; k++) { ul[k] = TMP(SL::QV + k, bl); ur[k] = TMP(SL::QV + k, br); }
+        const double c2 = roe_state<ND, D>(ul, TMP(SL::QH, bl), TMP(SL::QSR, bl), ur, TMP(SL::QH, br),
+                                           TMP(SL::QSR, br), K.gm1, rs);
+        if (!(c2 > 0.0)) atomicAdd(&a.st->nonphys, 1ull);
+        double *r = sm + SS::ROE + lane;
+#pragma unroll
+        for (int k = 0; k < ND; k++) r[k * 32] = rs.ut[k];
+        r[ND * 32] = rs.Ht;
+        r[(ND + 1) * 32] = rs.ct;
+        r[(ND + 2) * 32] = rs.q2;
+        r[(ND + 3) * 32] = rs.unct;
+        r[(ND + 4) * 32] = rs.cinv;
+        r[(ND + 5) * 32] = rs.b1;
+        r[(ND + 6) * 32] = rs.b2;
+        r[(ND + 7) * 32] = rs.unc;
+        r[(ND + 8) * 32] = rs.bu;
+    } else if (warp <= 4) {
+        const int row = warp == 1 ? SL::QLM : (warp == 2 ? SL::QL0 : (warp == 3 ? SL::QLP : SL::QLR));
+        double m = 0.0;
+        int jm = 0;
+#pragma unroll
+        for (int j = 0; j < W; j++) {
+            const double e = TMP(row, b0 + j * bs);
+            if (j == 0 || speed_gt(e, m)) { m = e; jm = j; }
+        }
+        sm[SS::SPD + (warp - 1) * 32 + lane] = m;
+        if (MODE == kSweepRecord) arg[(warp - 1) * 32 + lane] = (uint16_t)jm;
+    }
+#undef TMP
+}
+
+// This warp's row of L applied to U (f+ warps) or F (f- warps) of the stencil.
+template <int ND, int H, int D>
+__device__ __forceinline__ void small_project(int k, int s, int b0, int bs, const double *sm, double *out)
+{
+    using SL = FaceSmem<ND, H>;
+    using SS = SmallSmem<ND, H>;
+    constexpr int nc = ND + 2, last = nc - 1, W = 2 * H, NS = SL::NS;
+    const int lane = threadIdx.x & 31;
+    const double *r = sm + SS::ROE + lane;
+    RoeScalars<ND> rs;
+#pragma unroll
+    for (int i = 0; i < ND; i++) rs.ut[i] = r[i * 32];
+    rs.cinv = r[(ND + 4) * 32];
+    rs.b1 = r[(ND + 5) * 32];
+    rs.b2 = r[(ND + 6) * 32];
+    rs.unc = r[(ND + 7) * 32];
+    rs.bu = r[(ND + 8) * 32];
+    const bool shear = (k >= 2 && k < last);
+    const int tax = shear ? shear_axis<ND, D>(k) : 0;
+    double lrow[nc];
+    l_row<ND, D>(rs, k, lrow);
+#pragma unroll
+    for (int j = 0; j < W; j++) {
+        const double *c = sm + 2 * (b0 + j * bs) + s;  // the pair's U or F
+        double w;
+        if (shear) {
+            w = c[2 * (1 + tax) * NS] + lrow[0] * c[0];
+        } else {
+            w = lrow[0] * c[0];
+#pragma unroll
+            for (int i = 1; i < nc; i++) w = fma(lrow[i], c[2 * i * NS], w);
+        }
+        out[j * 32 + lane] = w;
+    }
+}
+
+// One tile at the pencils from (x, y, z), faces from f0 of direction d, by a block.
+template <int ND, int H, int MODE>
+__device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da, const FastK &FK,
+                                           const Consts &K, int d, int64_t f0, int64_t x, int64_t y,
+                                           int64_t z, unsigned long long *exact_count, double *sm)
+{
+    using SL = FaceSmem<ND, H>;
+    using SS = SmallSmem<ND, H>;
+    constexpr int nc = ND + 2, last = nc - 1, W = 2 * H, NS = SL::NS, NT = 32 * SS::NW;
+    __shared__ uint16_t arg[4 * 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = warp >> 1, s = warp & 1;
+    const int tps = ND == 1 ? 0 : da.tps;
+    int p, fo, b0, bs;
+    int64_t flin, npen;
+    const double2 *UF = (const double2 *)sm;
+    if (d == 0) {
+        tile_lane<0>(tps, lane, p, fo);
+        b0 = p * ((kTileFaces >> tps) + 2 * H - 1) + fo;
+        bs = 1;
+        npen = a.n[1] - y;
+        flin = face_index<0>(a.n, f0 + fo, x, y + p, z);
+    } else {
+        tile_lane<1>(tps, lane, p, fo);
+        b0 = lane;
+        bs = 1 << tps;
+        npen = a.n[0] - x;
+        flin = d == 1 ? face_index<1>(a.n, f0 + fo, x + p, y, z) : face_index<2>(a.n, f0 + fo, x + p, y, z);
+    }
+    const bool active = f0 + fo <= (d == 0 ? a.n[0] : (d == 1 ? a.n[1] : a.n[2])) - da.skip_last && p < npen;
+    if (active && !TENO_IN(a.st, flin, da.nfaces)) flin = 0;     // debug build: counted, redirected
+
+    if (ND == 1 || d == 0) stage_cells<ND, H, 0>(a, da, K, f0, x, y, z, sm, threadIdx.x, NT);
+    if constexpr (ND >= 2) {
+        if (d == 1) stage_cells<ND, H, 1>(a, da, K, f0, x, y, z, sm, threadIdx.x, NT);
+    }
+    if constexpr (ND >= 3) {
+        if (d == 2) stage_cells<ND, H, 2>(a, da, K, f0, x, y, z, sm, threadIdx.x, NT);
+    }
+    __syncthreads();
+    if (ND == 1 || d == 0) small_states<ND, H, 0, MODE>(a, da, K, warp, b0, bs, active, flin, sm, arg);
+    if constexpr (ND >= 2) {
+        if (d == 1) small_states<ND, H, 1, MODE>(a, da, K, warp, b0, bs, active, flin, sm, arg);
+    }
+    if constexpr (ND >= 3) {
+        if (d == 2) small_states<ND, H, 2, MODE>(a, da, K, warp, b0, bs, active, flin, sm, arg);
+    }
+    __syncthreads();
+    double *prj = sm + SS::PRJ + warp * W * 32;
+    if (active) {
+        if (ND == 1 || d == 0) small_project<ND, H, 0>(k, s, b0, bs, sm, prj);
+        if constexpr (ND >= 2) {
+            if (d == 1) small_project<ND, H, 1>(k, s, b0, bs, sm, prj);
+        }
+        if constexpr (ND >= 3) {
+            if (d == 2) small_project<ND, H, 2>(k, s, b0, bs, sm, prj);
+        }
+    }
+    __syncthreads();
+    double v[W], val = 0.0;
+    uint8_t fl = 0;
+    bool open = false;
+    if (active) {
+        const double *hw = sm + SS::PRJ + 2 * k * W * 32 + lane, *hg = hw + W * 32;
+        const int sp = K.split ? 3 : (k == 0 ? 0 : (k == last ? 2 : 1));
+        const double al = sm[SS::SPD + sp * 32 + lane], sa = s ? -al : al;
+#pragma unroll
+        for (int kk = 0; kk < W; kk++) {
+            const int j = s ? W - 1 - kk : kk;
+            v[kk] = fma(sa, hw[j * 32], hg[j * 32]);
+        }
+        const bool need_ct = MODE == kSweepRecord && a.need_ct;
+        open = true;
+        if (a.fast) {
+            if (!need_ct && quick_large<H>(v, FK)) {
+                fl = (uint8_t)large_code(H);
+                open = false;
+            } else if (fast_decide<H>(v, FK, fl, need_ct)) {
+                open = false;
+            }
+            if (!open) val = decided_value<H>(v, fl);
+        }
+    }
+    unsigned left = __ballot_sync(0xffffffffu, open);
+    if (left) {
+        if (exact_count && lane == 0) atomicAdd(exact_count, (unsigned long long)__popc(left));
+        if (__popc(left) > 3) {                        // a lane each costs about as much as three
+            if (open) val = teno_recon<H>(v, K, fl);
+        } else {
+            int row = -1;
+            double qc[W];
+#pragma unroll
+            for (int c = 0; c < W; c++) qc[c] = 0.0;
+            exact_row<H, H>(lane, row, qc);
+            while (left) {
+                const int src = __ffs(left) - 1;
+                left &= left - 1;
+                double u[W];
+#pragma unroll
+                for (int kk = 0; kk < W; kk++) u[kk] = __shfl_sync(0xffffffffu, v[kk], src);
+                uint8_t f;
+                const double r = exact_warp<H>(u, row, qc, K, f);
+                if (lane == src) {
+                    val = r;
+                    fl = f;
+                }
+            }
+        }
+    }
+    sm[SS::VAL + warp * 32 + lane] = val;
+    if (MODE == kSweepRecord && active) da.flags[flin * nc * 2 + 2 * k + s] = fl;
+    __syncthreads();
+    if (warp == 0 && active) {
+        SweepBuf B;
+        B.nt = 1;                                      // rows of 32
+        B.R = sm + SS::VAL;
+        B.RO = sm + SS::ROE;
+        B.RL = sm + SS::PRJ;
+        if (a.limiter) {
+            const int bl = b0 + (H - 1) * bs, br = bl + bs;
+#pragma unroll
+            for (int c = 0; c < nc; c++) {
+                const double2 cl = UF[c * NS + bl], cr = UF[c * NS + br];
+                B.RL[(4 * c) * 32 + lane] = cl.x;
+                B.RL[(4 * c + 1) * 32 + lane] = cl.y;
+                B.RL[(4 * c + 2) * 32 + lane] = cr.x;
+                B.RL[(4 * c + 3) * 32 + lane] = cr.y;
+            }
+            const double sl = sm[SL::TMP + SL::QLR * NS + bl], sr = sm[SL::TMP + SL::QLR * NS + br];
+            B.RL[4 * nc * 32 + lane] = sr > sl ? sr : sl;
+        }
+        if (MODE == kSweepRecord)
+            da.argmax[flin] = (uint16_t)(arg[lane] | (arg[32 + lane] << 4) | (arg[64 + lane] << 8) |
+                                         (arg[96 + lane] << 12));
+        if (ND == 1 || d == 0) finish_face<ND, 0, MODE, false>(da, a.limiter, K, B, lane, flin, a.st);
+        if constexpr (ND >= 2) {
+            if (d == 1) finish_face<ND, 1, MODE, false>(da, a.limiter, K, B, lane, flin, a.st);
+        }
+        if constexpr (ND >= 3) {
+            if (d == 2) finish_face<ND, 2, MODE, false>(da, a.limiter, K, B, lane, flin, a.st);
+        }
+    }
+}
+
+// 24 warps per SM at least (20 in 3D), 80 registers (96).
+template <int ND, int H, int MODE>
+__global__ void __launch_bounds__(64 * (ND + 2), ND == 1 ? 4 : (ND == 2 ? 3 : 2))
+    small_kernel(const SweepArgs a)
+{
+    extern __shared__ double sm[];
+    const int32_t tile = (int32_t)blockIdx.x;
+    int i = 0;
+    while (i + 1 < a.nparts && tile >= a.part[i + 1].first) i++;
+    const int64_t t = a.part[i].t0 + (tile - a.part[i].first);
+    const int d = a.part[i].d;
+    int64_t f0, x, y, z;
+    if (ND == 1 || d == 0) tile_at<ND, 0>(a.g.n, a.dir[0], t, f0, x, y, z);
+    if constexpr (ND >= 2) {
+        if (d == 1) tile_at<ND, 1>(a.g.n, a.dir[1], t, f0, x, y, z);
+    }
+    if constexpr (ND >= 3) {
+        if (d == 2) tile_at<ND, 2>(a.g.n, a.dir[2], t, f0, x, y, z);
+    }
+    small_tile<ND, H, MODE>(a.g, a.dir[d], a.FK, a.K, d, f0, x, y, z, a.exact_count, sm);
+}
+
+// The decide and exact kernels of one chunk (a's group and split are set here).
+// mixed: in a batch of both schemes, the one to take (MIX = 0).
+template <int H, bool RECORD, int MIX>
+cudaError_t launch_decisions(DecideArgs &a, cudaStream_t s, int mixed = -1)
+{
+    // at least four waves of warps (24 on each of 152 SMs) before tiles share
+    // one; a small evaluation's rounds go to a warp each while that is about two
+    // waves (a round takes some 5 us, alone or beside 23 others)
+    const int64_t fill = 152 * 24, sides = MIX ? 2 : 1;
+    a.group = a.split = 1;
+    while (a.group < kDecideMostTiles && a.tiles * sides >= 8 * fill * a.group) a.group *= 2;
+    while (a.group == 1 && a.split < 2 * a.nc && a.tiles * sides * a.split <= fill) a.split *= 2;
+    const int64_t units = (int64_t)((a.tiles + a.group - 1) / a.group) * a.split * sides;
+    decide_kernel<H, RECORD, MIX><<<(unsigned)((units + kDecideWarps - 1) / kDecideWarps),
+                                    32 * kDecideWarps, 0, s>>>(a, mixed);
+    const int64_t most = ((int64_t)a.tiles * a.nc + 1) / 2;   // blocks of 128 lanes for every entry
+    exact_kernel<H, RECORD, MIX><<<(unsigned)(sides * (most < 608 ? most : 608)), 128, 0, s>>>(a, mixed > 0);
     return cudaGetLastError();
 }
 
@@ -891,12 +1386,36 @@ cudaError_t launch_chunk_mode(const SweepArgs &a, cudaStream_t s)
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
+    if constexpr (MODE != kSweepFrozen) {
+        if (a.small) {
+            constexpr size_t bytes = SmallSmem<ND, H>::BYTES;
+            static bool small_done = false;
+            if (!small_done) {
+                cudaError_t e = cudaFuncSetAttribute(small_kernel<ND, H, MODE>,
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                if (e != cudaSuccess) return e;
+                small_done = true;
+            }
+            small_kernel<ND, H, MODE><<<(unsigned)a.tiles, 64 * (ND + 2), bytes, s>>>(a);
+            return cudaGetLastError();
+        }
+    }
     const unsigned blocks = (unsigned)((a.tiles + kSweepWarps - 1) / kSweepWarps);
     sweep_kernel<ND, H, MODE><<<blocks, 32 * kSweepWarps, smem, s>>>(a);
     if (MODE != kSweepFrozen) {
-        cudaError_t e = launch_decisions<H, MODE == kSweepRecord>(
-            a.buf, a.tiles, ND + 2, a.g.fast, a.g.need_ct, 0, a.nexact, a.exact_count, a.FK, a.K,
-            a.g.st, s);
+        DecideArgs d;
+        d.B = a.buf;
+        d.tiles = a.tiles;
+        d.nc = ND + 2;
+        d.fast = a.g.fast;
+        d.need_ct = a.g.need_ct;
+        d.nexact[0] = d.nexact[1] = a.nexact;
+        d.xlist[0] = d.xlist[1] = a.buf.xlist;
+        d.exact_count = a.exact_count;
+        d.st = a.g.st;
+        d.FK = a.FK;
+        d.K = a.K;
+        cudaError_t e = launch_decisions<H, MODE == kSweepRecord, 0>(d, s);
         if (e != cudaSuccess) return e;
     }
     finish_kernel<ND, MODE><<<(unsigned)((a.tiles + 3) / 4), 128, 0, s>>>(a);
