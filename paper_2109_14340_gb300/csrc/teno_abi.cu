@@ -92,15 +92,8 @@ __global__ void __launch_bounds__(256) combine_kernel(CombineArgs a)
                                   TENO_LOAD(a.st, Fd, flo[d], a.nfaces[d])) * a.inv_dx[d];
                 acc = acc - t;
             }
-            double o;
-            if (a.mode == 0) {
-                o = acc;
-            } else {
-                const double t = Uc[c] + dt * acc;
-                if (a.mode == 1) o = t;
-                else if (a.mode == 2) o = 0.75 * a.Un[c * a.ncell + id] + 0.25 * t;
-                else o = (1.0 / 3.0) * a.Un[c * a.ncell + id] + (2.0 / 3.0) * t;
-            }
+            const double o = stage_value(a.mode, acc, Uc[c],
+                                         a.mode > 1 ? a.Un[c * a.ncell + id] : 0.0, dt);
             a.out[c * a.ncell + id] = o;
             Uo[c] = o;
         }
@@ -241,8 +234,7 @@ __global__ void prepare_kernel(Status *st, int nd, double dt_host, const double 
 }
 
 // Scalar reconstruction of caller-provided stencils (teno_reconstruct): the
-// certified filter first when enabled (its first test too where no decision
-// byte is asked for, as in the sweeps), else / then the exact path.
+// certified filter first when enabled, else / then the exact path.
 template <int H>
 __global__ void recon_kernel(const double *v, int64_t count, double *out, uint8_t *flags, Consts K,
                              FastK FK, int fast)
@@ -255,7 +247,7 @@ __global__ void recon_kernel(const double *v, int64_t count, double *out, uint8_
         for (int m = 0; m < W; m++) vv[m] = v[i * W + m];
         uint8_t fl = 0;
         double r;
-        if (fast && !flags && quick_large<H>(vv, FK)) r = flux_large<H, H>(vv);
+        if (fast && quick_large<H>(vv, FK, flags != nullptr, fl)) r = flux_large<H, H>(vv);
         else if (fast && fast_decide<H>(vv, FK, fl, flags != nullptr)) r = decided_value<H>(vv, fl);
         else r = teno_recon<H>(vv, K, fl);
         out[i] = r;
@@ -465,6 +457,20 @@ static bool small_path(const teno_params *p, const void *frozen)
     return !frozen && small_evaluation(all_tiles(p), p->ndim, p->scheme / 2);
 }
 
+// In 1D that launch also forms the stage's result, where it may write an array
+// that it does not read.
+static bool fused_path(const teno_params *p, const void *frozen)
+{
+    return p->ndim == 1 && small_path(p, frozen);
+}
+
+// The stage-2 state of a step: in place of the stage-1 state, or in the fluxes'
+// room, which fused stages leave unused.
+static double *second_stage(const teno_params *p, char *ws, double *Us, const void *frozen)
+{
+    return fused_path(p, frozen) ? (double *)(ws + layout(p).flux[0]) : Us;
+}
+
 // Primitives of U into the workspace's primitive rows (non-physical cells
 // counted); returns their address (nullptr where the sweeps need none).
 static cudaError_t launch_prims(const teno_params *p, const double *U, char *ws, cudaStream_t s,
@@ -534,7 +540,8 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
     const SweepMem M = sm ? *sm : sweep_mem(p, ws + L.sweep, kChunkTiles);
     if (p->limiter && nd > 1) CUDA_TRY(launch_wave_max(p, Uk, st, 0, s));
     const int small = small_path(p, frozen);
-    if (!small || p->limiter)         // counters to zero, the limiter's dt/dx
+    const bool fused = fused_path(p, frozen) && Uk != out;
+    if (!small || (p->limiter && !fused))         // counters to zero, the limiter's dt/dx
         prepare_kernel<<<1, M.nchunks > 32 ? 256 : 32, 0, s>>>(st, nd, dt_host, dt_dev, idx, p->limiter,
                                                          M.counters, (int)M.nchunks);
     CUDA_TRY(cudaGetLastError());
@@ -583,13 +590,26 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
         D.lam = &st->lam[d];
         D.skip_last = (p->bc_lo[d] == TENO_BC_PERIODIC && !fl && !fz) ? 1 : 0;
         tiles[d] = shape_tiles(p, d, D.skip_last, D);
+        if (fused) {                  // every face, tiles overlapping by one
+            D.skip_last = 0;
+            D.own = kTileFaces - 1;
+            tiles[d] = D.line_tiles = (p->n[d] + D.own - 1) / D.own;
+        }
         if (fl) fl += (size_t)face_grid(p, d) * nc * 2;
         if (fz) fz += (size_t)face_grid(p, d) * nc * 2;
         if (am) am += face_grid(p, d);
         if (fam) fam += face_grid(p, d);
         if (lr) lr += face_grid(p, d);
     }
-    // all directions' tiles in order, cut into chunks that fit the buffers
+    a.fuse.mode = fused ? mode : -1;
+    a.fuse.Un = Un;
+    a.fuse.out = out;
+    a.fuse.dt_dev = dt_dev;
+    a.fuse.dt = dt_host;
+    a.fuse.inv_dx = idx.x;
+    // all directions' tiles in order, cut into chunks that fit the buffers (the
+    // single launch uses none)
+    const int64_t chunk_tiles = small ? all_tiles(p) + tiles[0] : M.nt;
     int d = 0;
     int64_t done = 0;                 // tiles of direction d already in a chunk
     for (int64_t chunk = 0; d < nd; chunk++) {
@@ -597,8 +617,8 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
         a.tiles = 0;
         a.nexact = M.counters + chunk;
         int64_t faces = 0;            // computed by this chunk (for the profile)
-        while (d < nd && a.tiles < M.nt) {
-            const int64_t room = M.nt - a.tiles, left = tiles[d] - done;
+        while (d < nd && a.tiles < chunk_tiles) {
+            const int64_t room = chunk_tiles - a.tiles, left = tiles[d] - done;
             const int64_t take = left < room ? left : room;
             const int64_t fd = a.g.ncell / p->n[d] * (p->n[d] + 1 - a.dir[d].skip_last);
             SweepPart &q = a.part[a.nparts++];
@@ -627,6 +647,7 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
         if (e != cudaSuccess) return TENO_ECUDA;
         if (slot >= 0) CUDA_TRY(profile_mark(1, slot, s));
     }
+    if (fused) return TENO_OK;
     CombineArgs c;
     for (int d = 0; d < 3; d++) {
         c.F[d] = (const double *)(ws + L.flux[d]);
@@ -733,9 +754,10 @@ int teno_rk3_step(const teno_params *p, double *U, double dt, const double *dt_d
     // each stage's combine stores the primitives of the next stage's input
     double *P = nullptr;
     CUDA_TRY(launch_prims(p, U, (char *)ws, s, &P));
+    double *U2 = second_stage(p, (char *)ws, Us, nullptr);
     if ((r = stage(p, U, U, Us, 1, dt, dt_device, nullptr, (char *)ws, s, nullptr, P, P))) return r;
-    if ((r = stage(p, Us, U, Us, 2, dt, dt_device, nullptr, (char *)ws, s, nullptr, P, P))) return r;
-    return stage(p, Us, U, U, 3, dt, dt_device, nullptr, (char *)ws, s, nullptr, P, nullptr);
+    if ((r = stage(p, Us, U, U2, 2, dt, dt_device, nullptr, (char *)ws, s, nullptr, P, P))) return r;
+    return stage(p, U2, U, U, 3, dt, dt_device, nullptr, (char *)ws, s, nullptr, P, nullptr);
 }
 
 static int rk3_step_record(const teno_params *p, double *U, double dt, double *U1, double *U2,

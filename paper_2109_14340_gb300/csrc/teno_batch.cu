@@ -30,9 +30,15 @@ struct BatchSlot {
 
 constexpr int kCellTile = 256;
 constexpr int kMixedTiles = 4096;
+// Tiles up to which the fused stage is the better one: two steps of 200 problems of
+// 64 to 512 cells (1860 tiles) take 1055 us against 1142, of 400 (3700) 1893
+// against 1634.
+constexpr int kSmallBatch = 2400;
 constexpr int kTiles[3] = {64, 128, 256};   // faces in flight per block (a warp: 32)
 constexpr int kBatchSlice =                 // doubles of shared memory per warp
     FaceSmem<1, 5>::TOTAL > FaceSmem<1, 4>::TOTAL ? FaceSmem<1, 5>::TOTAL : FaceSmem<1, 4>::TOTAL;
+constexpr size_t kBatchSmallBytes =
+    SmallSmem<1, 5>::BYTES > SmallSmem<1, 4>::BYTES ? SmallSmem<1, 5>::BYTES : SmallSmem<1, 4>::BYTES;
 constexpr size_t batch_smem(int TF) { return sizeof(double) * kBatchSlice * (TF / 32); }
 
 // Item -> problem by binary search in an exclusive prefix of per-problem item
@@ -88,7 +94,7 @@ __global__ void __launch_bounds__(kCellTile) batch_wave_max_kernel(
 }
 
 // dt = cfl / (A / dx) and the limiter's dt/dx per problem, exactly as
-// cfl_finalize_kernel + prepare_kernel do for one 1D problem.
+// wave_max_kernel and prepare_kernel do for one 1D problem.
 __global__ void batch_finalize_kernel(const BatchProb *probs, int nprob, BatchSlot *slots,
                                       double cfl)
 {
@@ -138,10 +144,56 @@ __global__ void __launch_bounds__(TF, 512 / TF) batch_sweep_kernel(
         a.bcs_lo = nullptr;
         a.bcs_hi = nullptr;
         a.skip_last = 0;
+        a.tps = 0;
+        a.own = kTileFaces;
         const int64_t f0 = (int64_t)(first + it - fprefix[p]) * kTileFaces;
         if (d.scheme == 10) sweep_tile<1, 5, 0, kSweepPlain>(g, a, FK, K, B, f0, 0, 0, 0, it, slice);
         else sweep_tile<1, 4, 0, kSweepPlain>(g, a, FK, K, B, f0, 0, 0, 0, it, slice);
     }
+}
+
+// Few tiles: the fused 1D stage, a block per item (31 cells of a problem).  Each
+// item's cells are counted with the input of stages 2 and 3; the wave-maximum
+// pass counts the first's.
+__global__ void __launch_bounds__(192, 4) batch_small_kernel(
+    const BatchProb *probs, int nprob, const int32_t *sprefix, const double *Uk, const double *Un,
+    double *out, const BatchSlot *slots, Status *st, Consts K, FastK FK, int fast, int mode)
+{
+    extern __shared__ double sm[];
+    const int it = blockIdx.x;
+    const int p = find_problem(sprefix, nprob, it);
+    const BatchProb d = probs[p];
+    GridArgs g;
+    g.U = Uk + d.u_off;
+    g.P = nullptr;
+    g.st = st;
+    g.n[0] = d.n; g.n[1] = 1; g.n[2] = 1;
+    g.ncell = d.n;
+    g.fast = fast;
+    g.need_ct = 0;
+    g.count_cells = mode > 1;
+    g.limiter = d.limiter;
+    g.tag = 0;
+    DirArgs a;
+    a.nfaces = d.n + 1;
+    a.bc_lo = d.bc_lo;
+    a.bc_hi = d.bc_hi;
+    a.bcs_lo = nullptr;
+    a.bcs_hi = nullptr;
+    a.lam = nullptr;
+    a.skip_last = 0;
+    a.tps = 0;
+    a.own = kTileFaces - 1;
+    FuseArgs f;
+    f.Un = Un + d.u_off;
+    f.out = out + d.u_off;
+    f.dt_dev = &slots[p].dt;
+    f.dt = 0.0;
+    f.inv_dx = d.inv_dx;
+    f.mode = mode;
+    const int64_t f0 = (int64_t)(it - sprefix[p]) * a.own;
+    if (d.scheme == 10) small_tile<1, 5, kSweepPlain>(g, a, FK, K, 0, f0, 0, 0, 0, nullptr, sm, f);
+    else small_tile<1, 4, kSweepPlain>(g, a, FK, K, 0, f0, 0, 0, 0, nullptr, sm, f);
 }
 
 __global__ void __launch_bounds__(128) batch_finish_kernel(
@@ -187,11 +239,7 @@ __global__ void __launch_bounds__(kCellTile) batch_combine_kernel(
             double acc = 0.0;
             const double t = (Fd[i + 1] - Fd[i]) * d.inv_dx;
             acc = acc - t;
-            const double s = Uc[c] + dt * acc;
-            double o;
-            if (mode == 1) o = s;
-            else if (mode == 2) o = 0.75 * Un[d.u_off + c * d.n + i] + 0.25 * s;
-            else o = (1.0 / 3.0) * Un[d.u_off + c * d.n + i] + (2.0 / 3.0) * s;
+            const double o = stage_value(mode, acc, Uc[c], mode > 1 ? Un[d.u_off + c * d.n + i] : 0.0, dt);
             out[d.u_off + c * d.n + i] = o;
             Uo[c] = o;
         }
@@ -212,13 +260,14 @@ struct teno_batch {
     teno_params common;
     std::vector<teno_batch_problem> probs;
     std::vector<BatchProb> desc;
-    std::vector<int32_t> fprefix;
+    std::vector<int32_t> fprefix, sprefix;      // 32-face tiles; 31-cell tiles of the fused stage
+    bool small() const { return sprefix.back() <= kSmallBatch; }
     std::vector<int32_t> cprefix;
     size_t u_len = 0, f_len = 0, p_len = 0;
     int64_t chunk_tiles = 0;    // tiles per pass through the sweep's buffers
     bool has8 = false, has10 = false, has_limiter = false;
     int nchunks() const { return (int)((fprefix.back() + chunk_tiles - 1) / chunk_tiles); }
-    size_t off_slots = 0, off_counters = 0, off_desc = 0, off_fprefix = 0,
+    size_t off_slots = 0, off_counters = 0, off_desc = 0, off_fprefix = 0, off_sprefix = 0,
            off_cprefix = 0, off_F = 0, off_Us = 0, off_P = 0, off_sweep = 0, off_xlist10 = 0, off_single = 0, total = 0;
     size_t single_bytes = 0;
     int tile_idx = 1;           // index into kTiles
@@ -295,6 +344,8 @@ int upload(teno_batch *b, char *ws, cudaStream_t s)
                              cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaMemcpyAsync(ws + b->off_fprefix, b->fprefix.data(), sizeof(int32_t) * (np + 1),
                              cudaMemcpyHostToDevice, s));
+    CUDA_TRY(cudaMemcpyAsync(ws + b->off_sprefix, b->sprefix.data(), sizeof(int32_t) * (np + 1),
+                             cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaMemcpyAsync(ws + b->off_cprefix, b->cprefix.data(), sizeof(int32_t) * (np + 1),
                              cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaStreamSynchronize(s));     // the host vectors are pageable
@@ -304,6 +355,8 @@ int upload(teno_batch *b, char *ws, cudaStream_t s)
     CUDA_TRY(set_face_attr<64>());
     CUDA_TRY(set_face_attr<128>());
     CUDA_TRY(set_face_attr<256>());
+    CUDA_TRY(cudaFuncSetAttribute(batch_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)kBatchSmallBytes));
     b->uploaded_ws = ws;
     b->uploaded_dev = dev;
     return TENO_OK;
@@ -341,6 +394,17 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
     const FastK FK = fastk_make(b->common.ct_cr, b->common.ct_alpha1, b->common.ct_alpha2,
                                 b->common.eps_beta, b->common.eps_eta);
     const int fast = g_fast_filter && fast_filter_valid(b->common.eps_beta, b->common.eps_eta);
+    if (b->small()) {
+        // U -> Us -> the fluxes' room -> U: a stage reads its neighbours' cells, so it
+        // never writes the array it reads
+        double *const seq[4] = {U, Us, (double *)(ws + b->off_F), U};
+        const int32_t *spre = (const int32_t *)(ws + b->off_sprefix);
+        for (int stg = 0; stg < 3; stg++)
+            batch_small_kernel<<<b->sprefix.back(), 192, kBatchSmallBytes, s>>>(
+                desc, np, spre, seq[stg], U, seq[stg + 1], slots, st, K, FK, fast, stg + 1);
+        CUDA_TRY(cudaGetLastError());
+        return TENO_OK;
+    }
     for (int stg = 0; stg < 3; stg++) {
         const double *Uin = stg == 0 ? U : Us;
         for (int c = 0; c < nchunks; c++) {
@@ -419,8 +483,9 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
     b->common.ndim = 1;
     b->probs.assign(probs, probs + nprob);
     size_t f_off = 0, p_off = 0, u_end = 0, single = 0;
-    int64_t ftiles = 0, ctiles = 0;
+    int64_t ftiles = 0, stiles = 0, ctiles = 0;
     b->fprefix.push_back(0);
+    b->sprefix.push_back(0);
     b->cprefix.push_back(0);
     for (int p = 0; p < nprob; p++) {
         const teno_batch_problem &q = probs[p];
@@ -455,6 +520,8 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
         u_end = std::max(u_end, (size_t)(q.offset + 3 * q.n));
         ftiles += (q.n + 1 + kTileFaces - 1) / kTileFaces;
         b->fprefix.push_back((int32_t)ftiles);
+        stiles += (q.n + kTileFaces - 2) / (kTileFaces - 1);
+        b->sprefix.push_back((int32_t)std::min<int64_t>(stiles, 1 << 30));
         ctiles += (q.n + kCellTile - 1) / kCellTile;
         b->cprefix.push_back((int32_t)ctiles);
         if (ftiles > (int64_t)1 << 30 || ctiles > (int64_t)1 << 30) {
@@ -482,10 +549,12 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
     off += a256(sizeof(BatchProb) * nprob);
     b->off_fprefix = off;
     off += a256(sizeof(int32_t) * (nprob + 1));
+    b->off_sprefix = off;
+    off += a256(sizeof(int32_t) * (nprob + 1));
     b->off_cprefix = off;
     off += a256(sizeof(int32_t) * (nprob + 1));
     b->off_F = off;
-    off += a256(sizeof(double) * b->f_len);
+    off += a256(sizeof(double) * std::max(b->f_len, b->u_len));
     b->off_Us = off;
     off += a256(sizeof(double) * b->u_len);
     b->off_P = off;

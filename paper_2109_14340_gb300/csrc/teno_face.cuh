@@ -56,6 +56,8 @@ struct DirArgs {
     // A tile is 2^tps pencils (side by side in x, in y for the x sweep) by 32 >> tps
     // faces; tiles per line of faces, and groups of 2^tps pencils along that axis.
     int tps;
+    int own;               // faces a tile owns along the line: all, or one fewer where tiles
+                           // overlap by a face (the fused 1D stage)
     int64_t line_tiles, groups;
 };
 
@@ -119,6 +121,17 @@ struct SweepPart {
     int32_t first, count, d;
 };
 
+// The fused 1D stage: a tile's faces also give its cells their update, which the
+// tile writes in place of its fluxes (tiles overlap by a face; the input and the
+// output are different arrays).
+struct FuseArgs {
+    const double *Un;      // state at t^n (RK modes), [3][n]
+    double *out;           // rhs (mode 0) or next stage state, [3][n]
+    const double *dt_dev;  // time step, or nullptr for dt
+    double dt, inv_dx;
+    int mode;              // -1: not fused; 0: rhs; 1..3: RK stage 0..2
+};
+
 struct SweepArgs {
     GridArgs g;
     DirArgs dir[3];
@@ -127,6 +140,7 @@ struct SweepArgs {
     int small;                         // 1: the single launch for few tiles
     unsigned *nexact;                  // length of the exact path's list (zeroed beforehand)
     unsigned long long *exact_count;   // adds the exact-path reconstructions, or nullptr
+    FuseArgs fuse;
     SweepBuf buf;
     FastK FK;
     Consts K;
@@ -147,6 +161,7 @@ inline void tile_shape(DirArgs &d, int64_t faces, int64_t pencils, int H)
         if (tps == 0 || cost < best) {
             best = cost;
             d.tps = tps;
+            d.own = (int)tf;
             d.line_tiles = lt;
             d.groups = gr;
         }
@@ -189,7 +204,7 @@ __device__ __forceinline__ void tile_at(const int64_t (&n)[3], const DirArgs &da
             else y = o;
         }
     }
-    f0 = ft * (kTileFaces >> da.tps);
+    f0 = ft * da.own;
 }
 
 // The lane's face within its tile: pencil p and offset fo along D.
@@ -365,8 +380,14 @@ __device__ __forceinline__ void stage_cells(const GridArgs &a, const DirArgs &da
             const bool ok = TENO_IN(a.st, id, a.ncell);
 #pragma unroll
             for (int c = 0; c < nc; c++) Uc[c] = ok ? a.U[c * a.ncell + id] : 0.0;
-            if (!rule && a.P && ok) {
-                load_prims<ND>(a.P, a.ncell, id, q);      // stored for this input
+            if (rule < 3 && a.P && ok) {
+                // stored for this input; a mirror image has its cell's, velocities
+                // (all or the wall-normal one) with the other sign, bit for bit
+                load_prims<ND>(a.P, a.ncell, id, q);
+                apply_ghost_rule<ND, D>(Uc, rule, nullptr, nullptr, 0, 0, K.gm1);
+#pragma unroll
+                for (int k = 0; k < ND; k++)
+                    if (rule == 2 || (rule == 1 && k == D)) q.u[k] = -q.u[k];
             } else {
                 if (rule) {
                     // boundary-face index among the faces of this side (other axes, x fastest)
@@ -381,7 +402,7 @@ __device__ __forceinline__ void stage_cells(const GridArgs &a, const DirArgs &da
         if (D == 0 && a.count_cells) {
             // interior cells of this tile's own face range: each cell once
             const int64_t ci = f0 - H + j;
-            if (ci >= f0 && ci < f0 + (kTileFaces >> tps) && ci < nD && nonphysical_cell<ND>(Uc[0], q))
+            if (ci >= f0 && ci < f0 + da.own && ci < nD && nonphysical_cell<ND>(Uc[0], q))
                 atomicAdd(&a.st->nonphys, 1ull);
         }
         // halves of U and of the flux along D: each product and sum of
@@ -546,11 +567,11 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
                 if constexpr (MODE == kSweepFrozen) {
                     *r = frozen_recon<H>(v, da.frozen[(flin * nc + k) * 2 + s]);
                 } else {
-                    open = !(a.fast && !(MODE == kSweepRecord && a.need_ct) && quick_large<H>(v, FK));
+                    uint8_t fl;
+                    open = !(a.fast && quick_large<H>(v, FK, MODE == kSweepRecord && a.need_ct, fl));
                     if (!open) {
                         *r = flux_large<H, H>(v);
-                        if constexpr (MODE == kSweepRecord)
-                            B.RD[(2 * k + s) * nf + cf] = (uint8_t)large_code(H);
+                        if constexpr (MODE == kSweepRecord) B.RD[(2 * k + s) * nf + cf] = fl;
                     }
                 }
             }
@@ -573,15 +594,15 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
 #undef TMP
 }
 
-// Back-projection of a face, the limiter, and what it leaves: the flux, the
-// limiter's byte and the decision bytes of the record.
-template <int ND, int D, int MODE, bool BYTES = true>
-__device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, const Consts &K,
-                                            const SweepBuf &B, int64_t cf, int64_t flin, Status *st)
+// Back-projection of a face and the limiter: the flux Fo (and the limiter's byte
+// of the record).  lam: the limiter's dt/dx.
+template <int ND, int D, int MODE>
+__device__ __forceinline__ void face_flux(const DirArgs &da, int limiter, double lam, const Consts &K,
+                                          const SweepBuf &B, int64_t cf, int64_t flin,
+                                          double (&Fo)[ND + 2])
 {
     constexpr int nc = ND + 2, last = nc - 1;
     const int64_t nf = B.nt * kTileFaces;
-    if (!TENO_IN(st, flin, da.nfaces)) return;
     RoeScalars<ND> rs;                 // what r_entry reads
 #pragma unroll
     for (int k = 0; k < ND; k++) rs.ut[k] = B.RO[k * nf + cf];
@@ -591,7 +612,6 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
     rs.unct = B.RO[(ND + 3) * nf + cf];
     // F = sum_k r_k (f+_k + f-_k), fields ascending; the zero and unit entries
     // of the shear columns are skipped.
-    double Fo[nc];
 #pragma unroll
     for (int k = 0; k < nc; k++) {
         const double hsum = B.R[(2 * k) * nf + cf] + B.R[(2 * k + 1) * nf + cf];
@@ -614,7 +634,7 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
         // Positivity-preserving flux limiter (cited in Sec. 5.3): blend toward
         // the Lax-Friedrichs flux so that the one-sided half updates of cells i
         // and i+1 keep rho >= eps and p >= eps.
-        const double eps = K.lim_eps, lam2 = 2.0 * (*da.lam), af = B.RL[4 * nc * nf + cf];
+        const double eps = K.lim_eps, lam2 = 2.0 * lam, af = B.RL[4 * nc * nf + cf];
         double FL[nc], dF[nc], UL[nc], UR[nc], dUL[nc], dUR[nc];
 #pragma unroll
         for (int c = 0; c < nc; c++) {
@@ -667,6 +687,19 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
         da.limrec[flin] = 0;
     }
 
+}
+
+// That and what else the face leaves: the flux in its array and (BYTES) its
+// decision bytes in the record.
+template <int ND, int D, int MODE, bool BYTES = true>
+__device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, const Consts &K,
+                                            const SweepBuf &B, int64_t cf, int64_t flin, Status *st)
+{
+    constexpr int nc = ND + 2;
+    const int64_t nf = B.nt * kTileFaces;
+    if (!TENO_IN(st, flin, da.nfaces)) return;
+    double Fo[nc];
+    face_flux<ND, D, MODE>(da, limiter, limiter ? *da.lam : 0.0, K, B, cf, flin, Fo);
     if constexpr (MODE == kSweepRecord && BYTES) {
 #pragma unroll
         for (int q = 0; q < 2 * nc; q++) da.flags[flin * nc * 2 + q] = B.RD[q * nf + cf];
@@ -676,13 +709,14 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
 }
 
 // Warps per block of the sweep (pencils side by side in the y and z sweeps) and
-// the blocks per SM that its registers are bounded for.
+// the blocks per SM that its registers are bounded for: 16 warps keep the FP64
+// unit 90 % busy; 20 (102 registers) gain nothing (128^3 TENO10 +0.7 %, TENO8
+// -0.1 %).
 constexpr int kSweepWarps = 4;
-template <int H>
 constexpr int kSweepBlocks = 4;
 
 template <int ND, int H, int MODE>
-__global__ void __launch_bounds__(32 * kSweepWarps, kSweepBlocks<H>) sweep_kernel(const SweepArgs a)
+__global__ void __launch_bounds__(32 * kSweepWarps, kSweepBlocks) sweep_kernel(const SweepArgs a)
 {
     extern __shared__ double sm[];
     const int w = threadIdx.x >> 5;
@@ -1105,11 +1139,22 @@ struct SmallSmem {
     static_assert(4 * nc + 1 <= NW * W, "limiter rows fit in the projections' room");
 };
 
+// Flux difference of one component of a cell and the stage's combination, as
+// combine_kernel forms them.
+__device__ __forceinline__ double stage_value(int mode, double acc, double U, double Un, double dt)
+{
+    if (mode == 0) return acc;
+    const double t = U + dt * acc;
+    if (mode == 1) return t;
+    if (mode == 2) return 0.75 * Un + 0.25 * t;
+    return (1.0 / 3.0) * Un + (2.0 / 3.0) * t;
+}
+
 // Roe state, its rows for the projections and the finish, and the splitting
 // speeds of a tile: warp 0 the first, warps 1-4 a speed each.
 template <int ND, int H, int D, int MODE>
 __device__ __forceinline__ void small_states(const GridArgs &a, const DirArgs &da, const Consts &K,
-                                             int warp, int b0, int bs, bool active, int64_t flin,
+                                             int warp, int b0, int bs, bool active, bool own,
                                              double *sm, uint16_t *arg)
 {
     using SL = FaceSmem<ND, H>;
@@ -1126,7 +1171,7 @@ __device__ __forceinline__ void small_states(const GridArgs &a, const DirArgs &d
         for (int k = 0; k < ND; k++) { ul[k] = TMP(SL::QV + k, bl); ur[k] = TMP(SL::QV + k, br); }
         const double c2 = roe_state<ND, D>(ul, TMP(SL::QH, bl), TMP(SL::QSR, bl), ur, TMP(SL::QH, br),
                                            TMP(SL::QSR, br), K.gm1, rs);
-        if (!(c2 > 0.0)) atomicAdd(&a.st->nonphys, 1ull);
+        if (own && !(c2 > 0.0)) atomicAdd(&a.st->nonphys, 1ull);
         double *r = sm + SS::ROE + lane;
 #pragma unroll
         for (int k = 0; k < ND; k++) r[k * 32] = rs.ut[k];
@@ -1194,11 +1239,13 @@ __device__ __forceinline__ void small_project(int k, int s, int b0, int bs, cons
 template <int ND, int H, int MODE>
 __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da, const FastK &FK,
                                            const Consts &K, int d, int64_t f0, int64_t x, int64_t y,
-                                           int64_t z, unsigned long long *exact_count, double *sm)
+                                           int64_t z, unsigned long long *exact_count, double *sm,
+                                           const FuseArgs &fuse)
 {
     using SL = FaceSmem<ND, H>;
     using SS = SmallSmem<ND, H>;
     constexpr int nc = ND + 2, last = nc - 1, W = 2 * H, NS = SL::NS, NT = 32 * SS::NW;
+    const bool fused = ND == 1 && fuse.mode >= 0;
     __shared__ uint16_t arg[4 * 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = warp >> 1, s = warp & 1;
     const int tps = ND == 1 ? 0 : da.tps;
@@ -1220,6 +1267,19 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
     }
     const bool active = f0 + fo <= (d == 0 ? a.n[0] : (d == 1 ? a.n[1] : a.n[2])) - da.skip_last && p < npen;
     if (active && !TENO_IN(a.st, flin, da.nfaces)) flin = 0;     // debug build: counted, redirected
+    const bool own = fo < da.own || f0 + fo == a.n[0];           // (all, unless tiles overlap)
+    // the fused update's inputs, on their way while the fluxes are computed
+    double Uk[nc], Un[nc], dt = 0.0;
+    const int64_t ic = f0 + lane;                                 // the lane's cell
+    const bool mine = fused && warp == 0 && lane < da.own && ic < a.n[0];
+    if (fused && warp == 0) dt = fuse.dt_dev ? *fuse.dt_dev : fuse.dt;
+    if (mine) {
+#pragma unroll
+        for (int c = 0; c < nc; c++) {
+            Uk[c] = fuse.mode > 0 ? a.U[c * a.ncell + ic] : 0.0;
+            Un[c] = fuse.mode > 1 ? fuse.Un[c * a.ncell + ic] : 0.0;
+        }
+    }
 
     if (ND == 1 || d == 0) stage_cells<ND, H, 0>(a, da, K, f0, x, y, z, sm, threadIdx.x, NT);
     if constexpr (ND >= 2) {
@@ -1229,12 +1289,12 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
         if (d == 2) stage_cells<ND, H, 2>(a, da, K, f0, x, y, z, sm, threadIdx.x, NT);
     }
     __syncthreads();
-    if (ND == 1 || d == 0) small_states<ND, H, 0, MODE>(a, da, K, warp, b0, bs, active, flin, sm, arg);
+    if (ND == 1 || d == 0) small_states<ND, H, 0, MODE>(a, da, K, warp, b0, bs, active, own, sm, arg);
     if constexpr (ND >= 2) {
-        if (d == 1) small_states<ND, H, 1, MODE>(a, da, K, warp, b0, bs, active, flin, sm, arg);
+        if (d == 1) small_states<ND, H, 1, MODE>(a, da, K, warp, b0, bs, active, own, sm, arg);
     }
     if constexpr (ND >= 3) {
-        if (d == 2) small_states<ND, H, 2, MODE>(a, da, K, warp, b0, bs, active, flin, sm, arg);
+        if (d == 2) small_states<ND, H, 2, MODE>(a, da, K, warp, b0, bs, active, own, sm, arg);
     }
     __syncthreads();
     double *prj = sm + SS::PRJ + warp * W * 32;
@@ -1263,18 +1323,14 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
         const bool need_ct = MODE == kSweepRecord && a.need_ct;
         open = true;
         if (a.fast) {
-            if (!need_ct && quick_large<H>(v, FK)) {
-                fl = (uint8_t)large_code(H);
-                open = false;
-            } else if (fast_decide<H>(v, FK, fl, need_ct)) {
-                open = false;
-            }
+            open = !quick_large<H>(v, FK, need_ct, fl) && !fast_decide<H>(v, FK, fl, need_ct);
             if (!open) val = decided_value<H>(v, fl);
         }
     }
     unsigned left = __ballot_sync(0xffffffffu, open);
     if (left) {
-        if (exact_count && lane == 0) atomicAdd(exact_count, (unsigned long long)__popc(left));
+        const unsigned owned = __ballot_sync(0xffffffffu, own);
+        if (exact_count && lane == 0) atomicAdd(exact_count, (unsigned long long)__popc(left & owned));
         if (__popc(left) > 3) {                        // a lane each costs about as much as three
             if (open) val = teno_recon<H>(v, K, fl);
         } else {
@@ -1301,7 +1357,9 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
     sm[SS::VAL + warp * 32 + lane] = val;
     if (MODE == kSweepRecord && active) da.flags[flin * nc * 2 + 2 * k + s] = fl;
     __syncthreads();
-    if (warp == 0 && active) {
+    if (warp) return;
+    double Fo[nc];
+    if (active) {
         SweepBuf B;
         B.nt = 1;                                      // rows of 32
         B.R = sm + SS::VAL;
@@ -1323,12 +1381,29 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
         if (MODE == kSweepRecord)
             da.argmax[flin] = (uint16_t)(arg[lane] | (arg[32 + lane] << 4) | (arg[64 + lane] << 8) |
                                          (arg[96 + lane] << 12));
-        if (ND == 1 || d == 0) finish_face<ND, 0, MODE, false>(da, a.limiter, K, B, lane, flin, a.st);
+        // the fused stage's limiter forms dt/dx itself (1D)
+        const double lam = fused ? dt * fuse.inv_dx : (a.limiter ? *da.lam : 0.0);
+        if (ND == 1 || d == 0) face_flux<ND, 0, MODE>(da, a.limiter, lam, K, B, lane, flin, Fo);
         if constexpr (ND >= 2) {
-            if (d == 1) finish_face<ND, 1, MODE, false>(da, a.limiter, K, B, lane, flin, a.st);
+            if (d == 1) face_flux<ND, 1, MODE>(da, a.limiter, lam, K, B, lane, flin, Fo);
         }
         if constexpr (ND >= 3) {
-            if (d == 2) finish_face<ND, 2, MODE, false>(da, a.limiter, K, B, lane, flin, a.st);
+            if (d == 2) face_flux<ND, 2, MODE>(da, a.limiter, lam, K, B, lane, flin, Fo);
+        }
+        if (!fused) {
+#pragma unroll
+            for (int c = 0; c < nc; c++) da.F[c * da.nfaces + flin] = Fo[c];
+        }
+    }
+    if (ND == 1 && fused) {
+#pragma unroll
+        for (int c = 0; c < nc; c++) {
+            const double Fr = __shfl_down_sync(0xffffffffu, Fo[c], 1);
+            const double t = (Fr - Fo[c]) * fuse.inv_dx;
+            double acc = 0.0;
+            acc = acc - t;
+            if (mine && TENO_IN(a.st, ic, a.ncell))
+                fuse.out[c * a.ncell + ic] = stage_value(fuse.mode, acc, Uk[c], Un[c], dt);
         }
     }
 }
@@ -1352,7 +1427,7 @@ __global__ void __launch_bounds__(64 * (ND + 2), ND == 1 ? 4 : (ND == 2 ? 3 : 2)
     if constexpr (ND >= 3) {
         if (d == 2) tile_at<ND, 2>(a.g.n, a.dir[2], t, f0, x, y, z);
     }
-    small_tile<ND, H, MODE>(a.g, a.dir[d], a.FK, a.K, d, f0, x, y, z, a.exact_count, sm);
+    small_tile<ND, H, MODE>(a.g, a.dir[d], a.FK, a.K, d, f0, x, y, z, a.exact_count, sm, a.fuse);
 }
 
 // The decide and exact kernels of one chunk (a's group and split are set here).

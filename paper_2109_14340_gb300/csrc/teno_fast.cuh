@@ -350,11 +350,12 @@ __device__ __forceinline__ constexpr float sos_bound(int which)
     else return which ? TENO_SOS12_K0 : TENO_SOS12_TAU2 * TENO_SOS12_KAPPA;
 }
 
-// First test of a reconstruction whose C_T exponent is not recorded: true
-// only if S_p is certain to be accepted, whatever the exponent (chi_p >= C_T
-// holds if sum_k (x_p / x_k)^7 <= 3 (x_p / min_k x_k)^7 <= thr[nexp_min]), or
-// at the smooth exponent where eta >= C_r (m = 0) is certain.  Most
-// reconstructions of a resolved flow end here, so it uses no FP64 operation at
+// First test of a reconstruction: true only if S_p is certain to be accepted,
+// whatever the exponent (chi_p >= C_T holds if sum_k (x_p / x_k)^7 <=
+// 3 (x_p / min_k x_k)^7 <= thr[nexp_min]), or at the smooth exponent where
+// eta >= C_r (m = 0) is certain; only the latter where the exponent is recorded
+// (need_ct).  flag: the decision byte.  Most reconstructions of a resolved flow
+// end here, so it uses no FP64 operation at
 // all and few others; whatever it leaves open goes to fast_decide.
 //
 // eta >= C_r: with e a bound of the differences' errors, 2 (|a| - e)(|b| - e) >=
@@ -375,7 +376,8 @@ __device__ __forceinline__ constexpr float sos_bound(int which)
 // is below 2e-22 in scaled units and (beta + eps)^7 is a normal number with
 // a normal reciprocal for every beta at or above 2e-22 / rho there.
 template <int H>
-__device__ __forceinline__ bool quick_large(const double (&v)[2 * H], const FastK &F)
+__device__ __forceinline__ bool quick_large(const double (&v)[2 * H], const FastK &F, bool need_ct,
+                                            uint8_t &flag)
 {
     constexpr int W = 2 * H;
     unsigned hmax = 0u, hmin = 0x7fffffffu;
@@ -452,8 +454,9 @@ __device__ __forceinline__ bool quick_large(const double (&v)[2 * H], const Fast
                         2.0f * (l0 * l1) >= c * (q0 + q1) && 2.0f * (l1 * l2) >= c * (q1 + q2) &&
                         2.0f * (l2 * l3) >= c * (q2 + q3) && 2.0f * (l3 * l4) >= c * (q3 + q4);
 #undef SS
-    const float rho = smooth ? fmaxf(F.rho_acc[F.nexp_min], F.rho_acc[F.nexp_smooth])
-                             : F.rho_acc[F.nexp_min];
+    const float any = need_ct ? 0.0f : F.rho_acc[F.nexp_min];
+    const float rho = smooth ? fmaxf(any, F.rho_acc[F.nexp_smooth]) : any;
+    flag = (uint8_t)(large_code(H) | (need_ct ? ((F.nexp_smooth - 7) & 7) << 5 : 0));
     return range && M >= 9.5367431640625e-7f && xp <= rho * xs;
 }
 
