@@ -62,6 +62,8 @@ struct CombineArgs {
 template <int ND>
 __global__ void __launch_bounds__(256) combine_kernel(CombineArgs a)
 {
+    chain_next();
+    chain_wait();
     constexpr int nc = ND + 2;
     // one thread per cell; x from the block's row, y and z from the grid
     const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -117,6 +119,8 @@ template <int ND>
 __global__ void __launch_bounds__(256) prims_kernel(const double *U, int64_t ncell, Consts K,
                                                     double *P, Status *st)
 {
+    chain_next();
+    chain_wait();
     constexpr int nc = ND + 2;
     unsigned long long bad = 0;
     for (int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; id < ncell;
@@ -141,6 +145,8 @@ template <int ND>
 __global__ void wave_max_kernel(const double *U, int64_t ncell, Consts K, Status *st, int count,
                                 double cfl, double3 inv_dx, double *dt_out, int accumulate)
 {
+    chain_next();
+    chain_wait();
     constexpr int nc = ND + 2;
     double m[ND];
 #pragma unroll
@@ -217,6 +223,8 @@ __global__ void dt_from_speeds_kernel(const double *amax, int ncopies, int nd, d
 __global__ void prepare_kernel(Status *st, int nd, double dt_host, const double *dt_dev,
                                double3 inv_dx, int limiter, unsigned *counters, int ncounters)
 {
+    chain_next();
+    chain_wait();
     for (int i = threadIdx.x; i < ncounters; i += blockDim.x) counters[i] = 0u;
     if (threadIdx.x) return;
     const double dt = dt_dev ? *dt_dev : dt_host;
@@ -444,10 +452,10 @@ static cudaError_t launch_wave_max(const teno_params *p, const double *U, Status
     static_assert(offsetof(Status, blocks) == offsetof(Status, amax) + sizeof(Status::amax), "zeroed together");
     cudaError_t e = cudaMemsetAsync(st->amax, 0, sizeof(st->amax) + sizeof(st->blocks), s);
     if (e != cudaSuccess) return e;
-    if (p->ndim == 1) wave_max_kernel<1><<<grd, blk, 0, s>>>(U, N, K, st, count, cfl, idx, dt_out, accumulate);
-    else if (p->ndim == 2) wave_max_kernel<2><<<grd, blk, 0, s>>>(U, N, K, st, count, cfl, idx, dt_out, accumulate);
-    else wave_max_kernel<3><<<grd, blk, 0, s>>>(U, N, K, st, count, cfl, idx, dt_out, accumulate);
-    return cudaGetLastError();
+    if (p->ndim == 1) e = launch_chained(wave_max_kernel<1>, grd, blk, 0, s, U, N, K, st, count, cfl, idx, dt_out, accumulate);
+    else if (p->ndim == 2) e = launch_chained(wave_max_kernel<2>, grd, blk, 0, s, U, N, K, st, count, cfl, idx, dt_out, accumulate);
+    else e = launch_chained(wave_max_kernel<3>, grd, blk, 0, s, U, N, K, st, count, cfl, idx, dt_out, accumulate);
+    return e;
 }
 
 // Whether an evaluation takes the single launch for few tiles: its tiles stage
@@ -485,11 +493,12 @@ static cudaError_t launch_prims(const teno_params *p, const double *U, char *ws,
     const Consts K = consts_of(p);
     const int64_t N = ncells(p);
     const int blk = 256, grd = grid_for(N, blk);
-    if (p->ndim == 1) prims_kernel<1><<<grd, blk, 0, s>>>(U, N, K, P, st);
-    else if (p->ndim == 2) prims_kernel<2><<<grd, blk, 0, s>>>(U, N, K, P, st);
-    else prims_kernel<3><<<grd, blk, 0, s>>>(U, N, K, P, st);
+    cudaError_t e;
+    if (p->ndim == 1) e = launch_chained(prims_kernel<1>, grd, blk, 0, s, U, N, K, P, st);
+    else if (p->ndim == 2) e = launch_chained(prims_kernel<2>, grd, blk, 0, s, U, N, K, P, st);
+    else e = launch_chained(prims_kernel<3>, grd, blk, 0, s, U, N, K, P, st);
     *P_out = P;
-    return cudaGetLastError();
+    return e;
 }
 
 // Event record of the face-sweep launches (teno_profile_*).
@@ -542,9 +551,8 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
     const int small = small_path(p, frozen);
     const bool fused = fused_path(p, frozen) && Uk != out;
     if (!small || (p->limiter && !fused))         // counters to zero, the limiter's dt/dx
-        prepare_kernel<<<1, M.nchunks > 32 ? 256 : 32, 0, s>>>(st, nd, dt_host, dt_dev, idx, p->limiter,
-                                                         M.counters, (int)M.nchunks);
-    CUDA_TRY(cudaGetLastError());
+        CUDA_TRY(launch_chained(prepare_kernel, 1, M.nchunks > 32 ? 256 : 32, 0, s, st, nd, dt_host, dt_dev,
+                                idx, p->limiter, M.counters, (int)M.nchunks));
     uint8_t *fl = flags;
     const uint8_t *fz = frozen;
     // the decision record: all directions' decision bytes, then all
@@ -671,9 +679,9 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
     const int blk = 256;
     const dim3 grd((unsigned)((p->n[0] + blk - 1) / blk), (unsigned)p->n[1], (unsigned)p->n[2]);
     NvtxRange crange("teno combine");
-    if (nd == 1) combine_kernel<1><<<grd, blk, 0, s>>>(c);
-    else if (nd == 2) combine_kernel<2><<<grd, blk, 0, s>>>(c);
-    else combine_kernel<3><<<grd, blk, 0, s>>>(c);
+    if (nd == 1) CUDA_TRY(launch_chained(combine_kernel<1>, grd, blk, 0, s, c));
+    else if (nd == 2) CUDA_TRY(launch_chained(combine_kernel<2>, grd, blk, 0, s, c));
+    else CUDA_TRY(launch_chained(combine_kernel<3>, grd, blk, 0, s, c));
     CUDA_TRY(cudaGetLastError());
     return TENO_OK;
 }

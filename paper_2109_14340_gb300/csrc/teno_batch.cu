@@ -61,6 +61,8 @@ __global__ void __launch_bounds__(kCellTile) batch_wave_max_kernel(
     double *P, Status *st, Consts K)
 {
     __shared__ double red[kCellTile / 32];
+    chain_next();
+    chain_wait();
     const int nitems = cprefix[nprob];
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int p = find_problem(cprefix, nprob, it);
@@ -98,6 +100,8 @@ __global__ void __launch_bounds__(kCellTile) batch_wave_max_kernel(
 __global__ void batch_finalize_kernel(const BatchProb *probs, int nprob, BatchSlot *slots,
                                       double cfl)
 {
+    chain_next();
+    chain_wait();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= nprob) return;
     const double idx = probs[p].inv_dx;
@@ -119,6 +123,8 @@ __global__ void __launch_bounds__(TF, 512 / TF) batch_sweep_kernel(
 {
     extern __shared__ double sm[];
     double *slice = sm + (size_t)(threadIdx.x >> 5) * kBatchSlice;
+    chain_next();
+    chain_wait();
     for (;;) {
         int it = 0;
         if ((threadIdx.x & 31) == 0) it = atomicAdd(counter, 1);
@@ -160,6 +166,8 @@ __global__ void __launch_bounds__(192, 4) batch_small_kernel(
     double *out, const BatchSlot *slots, Status *st, Consts K, FastK FK, int fast, int mode)
 {
     extern __shared__ double sm[];
+    chain_next();
+    chain_wait();
     const int it = blockIdx.x;
     const int p = find_problem(sprefix, nprob, it);
     const BatchProb d = probs[p];
@@ -200,6 +208,8 @@ __global__ void __launch_bounds__(128) batch_finish_kernel(
     const BatchProb *probs, int nprob, const int32_t *fprefix, int first, int count, double *F,
     SweepBuf B, const BatchSlot *slots, Status *st, Consts K)
 {
+    chain_next();
+    chain_wait();
     const int it = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (it >= count) return;
     const int p = find_problem(fprefix, nprob, first + it);
@@ -222,6 +232,8 @@ __global__ void __launch_bounds__(kCellTile) batch_combine_kernel(
     const BatchProb *probs, int nprob, const int32_t *cprefix, const double *Uk, const double *Un,
     double *out, const double *F, const BatchSlot *slots, double *P, Status *st, Consts K, int mode)
 {
+    chain_next();
+    chain_wait();
     const int nitems = cprefix[nprob];
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int p = find_problem(cprefix, nprob, it);
@@ -385,10 +397,8 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
     // per stage and chunk: the sweep's item counter, the two schemes' exact-path lists
     const int nchunks = b->nchunks();
     CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(int) * 9 * nchunks, s));
-    batch_wave_max_kernel<<<grid_c, kCellTile, 0, s>>>(desc, np, cpre, U, slots, P, st, K);
-    CUDA_TRY(cudaGetLastError());
-    batch_finalize_kernel<<<(np + 127) / 128, 128, 0, s>>>(desc, np, slots, cfl);
-    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(launch_chained(batch_wave_max_kernel, grid_c, kCellTile, 0, s, desc, np, cpre, U, slots, P, st, K));
+    CUDA_TRY(launch_chained(batch_finalize_kernel, (np + 127) / 128, 128, 0, s, desc, np, slots, cfl));
     const int TF = kTiles[tile_idx];
     const int grid_f = b->num_sms * bps;
     const FastK FK = fastk_make(b->common.ct_cr, b->common.ct_alpha1, b->common.ct_alpha2,
@@ -400,9 +410,8 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
         double *const seq[4] = {U, Us, (double *)(ws + b->off_F), U};
         const int32_t *spre = (const int32_t *)(ws + b->off_sprefix);
         for (int stg = 0; stg < 3; stg++)
-            batch_small_kernel<<<b->sprefix.back(), 192, kBatchSmallBytes, s>>>(
-                desc, np, spre, seq[stg], U, seq[stg + 1], slots, st, K, FK, fast, stg + 1);
-        CUDA_TRY(cudaGetLastError());
+            CUDA_TRY(launch_chained(batch_small_kernel, b->sprefix.back(), 192, kBatchSmallBytes, s, desc, np,
+                                    spre, seq[stg], U, seq[stg + 1], slots, st, K, FK, fast, stg + 1));
         return TENO_OK;
     }
     for (int stg = 0; stg < 3; stg++) {
@@ -412,12 +421,11 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
             const int first = c * (int)b->chunk_tiles;
             const int count = std::min((int)b->chunk_tiles, b->fprefix[np] - first);
             if (TF == 64)
-                batch_sweep_kernel<64><<<grid_f, 64, batch_smem(64), s>>>(desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt);
+                CUDA_TRY(launch_chained(batch_sweep_kernel<64>, grid_f, 64, batch_smem(64), s, desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt));
             else if (TF == 128)
-                batch_sweep_kernel<128><<<grid_f, 128, batch_smem(128), s>>>(desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt);
+                CUDA_TRY(launch_chained(batch_sweep_kernel<128>, grid_f, 128, batch_smem(128), s, desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt));
             else
-                batch_sweep_kernel<256><<<grid_f, 256, batch_smem(256), s>>>(desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt);
-            CUDA_TRY(cudaGetLastError());
+                CUDA_TRY(launch_chained(batch_sweep_kernel<256>, grid_f, 256, batch_smem(256), s, desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt));
             DecideArgs d;
             d.B = B;
             d.tiles = count;
@@ -441,12 +449,11 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
                 if (b->has8) CUDA_TRY((launch_decisions<4, false, 0>(d, s, mixed ? 0 : -1)));
                 if (b->has10) CUDA_TRY((launch_decisions<5, false, 0>(d, s, mixed ? 1 : -1)));
             }
-            batch_finish_kernel<<<(count + 3) / 4, 128, 0, s>>>(desc, np, fpre, first, count, F, B, slots, st, K);
-            CUDA_TRY(cudaGetLastError());
+            CUDA_TRY(launch_chained(batch_finish_kernel, (count + 3) / 4, 128, 0, s, desc, np, fpre, first, count, F,
+                                    B, slots, st, K));
         }
-        batch_combine_kernel<<<grid_c, kCellTile, 0, s>>>(desc, np, cpre, Uin, U, stg == 2 ? U : Us, F,
-                                                         slots, P, st, K, stg + 1);
-        CUDA_TRY(cudaGetLastError());
+        CUDA_TRY(launch_chained(batch_combine_kernel, grid_c, kCellTile, 0, s, desc, np, cpre, Uin, U,
+                                stg == 2 ? U : Us, F, slots, P, st, K, stg + 1));
     }
     return TENO_OK;
 }

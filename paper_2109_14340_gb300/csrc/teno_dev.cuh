@@ -12,6 +12,31 @@
 
 namespace teno {
 
+// Kernels of one call follow one another through programmatic launches: the next
+// one's blocks are set up while the last blocks of its predecessor run, and wait
+// for its end (and its writes) in chain_wait, which every kernel launched by
+// launch_chained calls before its first access to global memory.  Some 1 to 3 us
+// less between two short kernels.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t s, A &&...args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Workspace header (first 256 bytes of every workspace).
 struct Status {
     unsigned long long nonphys;    // non-physical cells + faces (teno_status)

@@ -220,6 +220,24 @@ __device__ __forceinline__ void tile_lane(int tps, int lane, int &p, int &fo)
     }
 }
 
+// A record's 16-bit words: a step's records lie back to back, and an odd number
+// of bytes each puts the second's words at odd addresses.
+__device__ __forceinline__ void put_word(uint16_t *p, unsigned v)
+{
+    if ((uintptr_t)p & 1) {
+        ((uint8_t *)p)[0] = (uint8_t)v;
+        ((uint8_t *)p)[1] = (uint8_t)(v >> 8);
+    } else {
+        *p = (uint16_t)v;
+    }
+}
+
+__device__ __forceinline__ unsigned get_word(const uint16_t *p)
+{
+    const uint8_t *b = (const uint8_t *)p;
+    return (uintptr_t)p & 1 ? b[0] | (unsigned)b[1] << 8 : *p;
+}
+
 // Index of face f of the pencil at (x, y, z) in direction D's face grid.
 template <int D>
 __device__ __forceinline__ int64_t face_index(const int64_t (&n)[3], int64_t f, int64_t x, int64_t y,
@@ -496,7 +514,7 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
         }
         // Splitting speeds over the stencil (first maximum), or at recorded cells.
         if constexpr (MODE == kSweepFrozen) {
-            unsigned w = da.frozen_argmax[flin];
+            unsigned w = get_word(da.frozen_argmax + flin);
             if (!TENO_IN(a.st, (int)(w & 15), W) || !TENO_IN(a.st, (int)((w >> 4) & 15), W) ||
                 !TENO_IN(a.st, (int)((w >> 8) & 15), W) || !TENO_IN(a.st, (int)(w >> 12), W))
                 w = 0;
@@ -516,7 +534,7 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
                 if (j == 0 || speed_gt(er, ar)) { ar = er; jr_ = j; }
             }
             if constexpr (MODE == kSweepRecord)
-                da.argmax[flin] = (uint16_t)(jm | (j0 << 4) | (jp << 8) | (jr_ << 12));
+                put_word(da.argmax + flin, jm | (j0 << 4) | (jp << 8) | (jr_ << 12));
         }
         if (K.split) am = a0 = ap = ar;               // Rusanov: one speed for every field
     }
@@ -719,6 +737,8 @@ template <int ND, int H, int MODE>
 __global__ void __launch_bounds__(32 * kSweepWarps, kSweepBlocks) sweep_kernel(const SweepArgs a)
 {
     extern __shared__ double sm[];
+    chain_next();
+    chain_wait();
     const int w = threadIdx.x >> 5;
     const int32_t tile = (int32_t)blockIdx.x * kSweepWarps + w;
     if (tile >= a.tiles) return;
@@ -881,6 +901,8 @@ __global__ void __launch_bounds__(32 * kDecideWarps, 6) decide_kernel(const Deci
 {
     __shared__ uint32_t list_[kDecideWarps][2][64];    // gathered entries: large stencil, fallback
     __shared__ uint8_t code_[kDecideWarps][2][64];
+    chain_next();
+    chain_wait();
     const int warp = threadIdx.x >> 5;
     const int64_t unit = (int64_t)blockIdx.x * kDecideWarps + warp;
     if constexpr (MIX == 0) {
@@ -1073,6 +1095,8 @@ __device__ __forceinline__ void exact_list(const DecideArgs &a, int which, unsig
 template <int H, bool RECORD, int MIX>
 __global__ void __launch_bounds__(128) exact_kernel(const DecideArgs a, int which)
 {
+    chain_next();
+    chain_wait();
     if constexpr (MIX == 0) {
         exact_list<H, RECORD>(a, which, blockIdx.x, gridDim.x);
     } else if (blockIdx.x & 1) {
@@ -1100,6 +1124,8 @@ __device__ __forceinline__ void finish_lane(const SweepArgs &a, int64_t t, int l
 template <int ND, int MODE>
 __global__ void __launch_bounds__(128) finish_kernel(const SweepArgs a)
 {
+    chain_next();
+    chain_wait();
     const int32_t tile = (int32_t)blockIdx.x * 4 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (tile >= a.tiles) return;
@@ -1379,8 +1405,8 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
             B.RL[4 * nc * 32 + lane] = sr > sl ? sr : sl;
         }
         if (MODE == kSweepRecord)
-            da.argmax[flin] = (uint16_t)(arg[lane] | (arg[32 + lane] << 4) | (arg[64 + lane] << 8) |
-                                         (arg[96 + lane] << 12));
+            put_word(da.argmax + flin, arg[lane] | (arg[32 + lane] << 4) | (arg[64 + lane] << 8) |
+                                           (arg[96 + lane] << 12));
         // the fused stage's limiter forms dt/dx itself (1D)
         const double lam = fused ? dt * fuse.inv_dx : (a.limiter ? *da.lam : 0.0);
         if (ND == 1 || d == 0) face_flux<ND, 0, MODE>(da, a.limiter, lam, K, B, lane, flin, Fo);
@@ -1414,6 +1440,8 @@ __global__ void __launch_bounds__(64 * (ND + 2), ND == 1 ? 4 : (ND == 2 ? 3 : 2)
     small_kernel(const SweepArgs a)
 {
     extern __shared__ double sm[];
+    chain_next();
+    chain_wait();
     const int32_t tile = (int32_t)blockIdx.x;
     int i = 0;
     while (i + 1 < a.nparts && tile >= a.part[i + 1].first) i++;
@@ -1443,11 +1471,13 @@ cudaError_t launch_decisions(DecideArgs &a, cudaStream_t s, int mixed = -1)
     while (a.group < kDecideMostTiles && a.tiles * sides >= 8 * fill * a.group) a.group *= 2;
     while (a.group == 1 && a.split < 2 * a.nc && a.tiles * sides * a.split <= fill) a.split *= 2;
     const int64_t units = (int64_t)((a.tiles + a.group - 1) / a.group) * a.split * sides;
-    decide_kernel<H, RECORD, MIX><<<(unsigned)((units + kDecideWarps - 1) / kDecideWarps),
-                                    32 * kDecideWarps, 0, s>>>(a, mixed);
+    cudaError_t e = launch_chained(decide_kernel<H, RECORD, MIX>,
+                                   (unsigned)((units + kDecideWarps - 1) / kDecideWarps),
+                                   32 * kDecideWarps, 0, s, a, mixed);
+    if (e != cudaSuccess) return e;
     const int64_t most = ((int64_t)a.tiles * a.nc + 1) / 2;   // blocks of 128 lanes for every entry
-    exact_kernel<H, RECORD, MIX><<<(unsigned)(sides * (most < 608 ? most : 608)), 128, 0, s>>>(a, mixed > 0);
-    return cudaGetLastError();
+    return launch_chained(exact_kernel<H, RECORD, MIX>, (unsigned)(sides * (most < 608 ? most : 608)), 128,
+                          0, s, a, (int)(mixed > 0));
 }
 
 template <int ND, int H, int MODE>
@@ -1471,12 +1501,12 @@ cudaError_t launch_chunk_mode(const SweepArgs &a, cudaStream_t s)
                 if (e != cudaSuccess) return e;
                 small_done = true;
             }
-            small_kernel<ND, H, MODE><<<(unsigned)a.tiles, 64 * (ND + 2), bytes, s>>>(a);
-            return cudaGetLastError();
+            return launch_chained(small_kernel<ND, H, MODE>, (unsigned)a.tiles, 64 * (ND + 2), bytes, s, a);
         }
     }
     const unsigned blocks = (unsigned)((a.tiles + kSweepWarps - 1) / kSweepWarps);
-    sweep_kernel<ND, H, MODE><<<blocks, 32 * kSweepWarps, smem, s>>>(a);
+    cudaError_t e = launch_chained(sweep_kernel<ND, H, MODE>, blocks, 32 * kSweepWarps, smem, s, a);
+    if (e != cudaSuccess) return e;
     if (MODE != kSweepFrozen) {
         DecideArgs d;
         d.B = a.buf;
@@ -1490,11 +1520,10 @@ cudaError_t launch_chunk_mode(const SweepArgs &a, cudaStream_t s)
         d.st = a.g.st;
         d.FK = a.FK;
         d.K = a.K;
-        cudaError_t e = launch_decisions<H, MODE == kSweepRecord, 0>(d, s);
+        e = launch_decisions<H, MODE == kSweepRecord, 0>(d, s);
         if (e != cudaSuccess) return e;
     }
-    finish_kernel<ND, MODE><<<(unsigned)((a.tiles + 3) / 4), 128, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(finish_kernel<ND, MODE>, (unsigned)((a.tiles + 3) / 4), 128, 0, s, a);
 }
 
 // One chunk's fluxes, in the mode its arguments ask for (a decision record to
