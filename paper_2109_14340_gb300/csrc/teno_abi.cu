@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(256) combine_kernel(CombineArgs a)
                                                                     : flo[d] + a.fstride[d];
                 const double t = (TENO_LOAD(a.st, Fd, fr, a.nfaces[d]) -
                                   TENO_LOAD(a.st, Fd, flo[d], a.nfaces[d])) * a.inv_dx[d];
-                acc = acc - t;
+                acc = d == 0 ? zero_minus(t) : acc - t;
             }
             const double o = stage_value(a.mode, acc, Uc[c],
                                          a.mode > 1 ? a.Un[c * a.ncell + id] : 0.0, dt);
@@ -441,6 +441,8 @@ static int grid_for(int64_t n, int block)
 
 static double3 inv_dx_of(const teno_params *p);
 
+static bool chained(const teno_params *p) { return all_tiles(p) <= kChainTiles; }
+
 static cudaError_t launch_wave_max(const teno_params *p, const double *U, Status *st,
                                    int count, cudaStream_t s, double cfl = 0.0,
                                    double *dt_out = nullptr, int accumulate = 0)
@@ -452,9 +454,9 @@ static cudaError_t launch_wave_max(const teno_params *p, const double *U, Status
     static_assert(offsetof(Status, blocks) == offsetof(Status, amax) + sizeof(Status::amax), "zeroed together");
     cudaError_t e = cudaMemsetAsync(st->amax, 0, sizeof(st->amax) + sizeof(st->blocks), s);
     if (e != cudaSuccess) return e;
-    if (p->ndim == 1) e = launch_chained(wave_max_kernel<1>, grd, blk, 0, s, U, N, K, st, count, cfl, idx, dt_out, accumulate);
-    else if (p->ndim == 2) e = launch_chained(wave_max_kernel<2>, grd, blk, 0, s, U, N, K, st, count, cfl, idx, dt_out, accumulate);
-    else e = launch_chained(wave_max_kernel<3>, grd, blk, 0, s, U, N, K, st, count, cfl, idx, dt_out, accumulate);
+    if (p->ndim == 1) e = launch_chained(chained(p), wave_max_kernel<1>, grd, blk, 0, s, U, N, K, st, count, cfl, idx, dt_out, accumulate);
+    else if (p->ndim == 2) e = launch_chained(chained(p), wave_max_kernel<2>, grd, blk, 0, s, U, N, K, st, count, cfl, idx, dt_out, accumulate);
+    else e = launch_chained(chained(p), wave_max_kernel<3>, grd, blk, 0, s, U, N, K, st, count, cfl, idx, dt_out, accumulate);
     return e;
 }
 
@@ -494,9 +496,9 @@ static cudaError_t launch_prims(const teno_params *p, const double *U, char *ws,
     const int64_t N = ncells(p);
     const int blk = 256, grd = grid_for(N, blk);
     cudaError_t e;
-    if (p->ndim == 1) e = launch_chained(prims_kernel<1>, grd, blk, 0, s, U, N, K, P, st);
-    else if (p->ndim == 2) e = launch_chained(prims_kernel<2>, grd, blk, 0, s, U, N, K, P, st);
-    else e = launch_chained(prims_kernel<3>, grd, blk, 0, s, U, N, K, P, st);
+    if (p->ndim == 1) e = launch_chained(chained(p), prims_kernel<1>, grd, blk, 0, s, U, N, K, P, st);
+    else if (p->ndim == 2) e = launch_chained(chained(p), prims_kernel<2>, grd, blk, 0, s, U, N, K, P, st);
+    else e = launch_chained(chained(p), prims_kernel<3>, grd, blk, 0, s, U, N, K, P, st);
     *P_out = P;
     return e;
 }
@@ -551,7 +553,7 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
     const int small = small_path(p, frozen);
     const bool fused = fused_path(p, frozen) && Uk != out;
     if (!small || (p->limiter && !fused))         // counters to zero, the limiter's dt/dx
-        CUDA_TRY(launch_chained(prepare_kernel, 1, M.nchunks > 32 ? 256 : 32, 0, s, st, nd, dt_host, dt_dev,
+        CUDA_TRY(launch_chained(chained(p), prepare_kernel, 1, M.nchunks > 32 ? 256 : 32, 0, s, st, nd, dt_host, dt_dev,
                                 idx, p->limiter, M.counters, (int)M.nchunks));
     uint8_t *fl = flags;
     const uint8_t *fz = frozen;
@@ -679,9 +681,9 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
     const int blk = 256;
     const dim3 grd((unsigned)((p->n[0] + blk - 1) / blk), (unsigned)p->n[1], (unsigned)p->n[2]);
     NvtxRange crange("teno combine");
-    if (nd == 1) CUDA_TRY(launch_chained(combine_kernel<1>, grd, blk, 0, s, c));
-    else if (nd == 2) CUDA_TRY(launch_chained(combine_kernel<2>, grd, blk, 0, s, c));
-    else CUDA_TRY(launch_chained(combine_kernel<3>, grd, blk, 0, s, c));
+    if (nd == 1) CUDA_TRY(launch_chained(chained(p), combine_kernel<1>, grd, blk, 0, s, c));
+    else if (nd == 2) CUDA_TRY(launch_chained(chained(p), combine_kernel<2>, grd, blk, 0, s, c));
+    else CUDA_TRY(launch_chained(chained(p), combine_kernel<3>, grd, blk, 0, s, c));
     CUDA_TRY(cudaGetLastError());
     return TENO_OK;
 }

@@ -248,9 +248,8 @@ __global__ void __launch_bounds__(kCellTile) batch_combine_kernel(
 #pragma unroll
         for (int c = 0; c < 3; c++) {
             const double *Fd = Fp + c * (d.n + 1);
-            double acc = 0.0;
             const double t = (Fd[i + 1] - Fd[i]) * d.inv_dx;
-            acc = acc - t;
+            const double acc = zero_minus(t);
             const double o = stage_value(mode, acc, Uc[c], mode > 1 ? Un[d.u_off + c * d.n + i] : 0.0, dt);
             out[d.u_off + c * d.n + i] = o;
             Uo[c] = o;
@@ -274,6 +273,7 @@ struct teno_batch {
     std::vector<BatchProb> desc;
     std::vector<int32_t> fprefix, sprefix;      // 32-face tiles; 31-cell tiles of the fused stage
     bool small() const { return sprefix.back() <= kSmallBatch; }
+    bool chained() const { return fprefix.back() <= kChainTiles; }
     std::vector<int32_t> cprefix;
     size_t u_len = 0, f_len = 0, p_len = 0;
     int64_t chunk_tiles = 0;    // tiles per pass through the sweep's buffers
@@ -397,8 +397,8 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
     // per stage and chunk: the sweep's item counter, the two schemes' exact-path lists
     const int nchunks = b->nchunks();
     CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(int) * 9 * nchunks, s));
-    CUDA_TRY(launch_chained(batch_wave_max_kernel, grid_c, kCellTile, 0, s, desc, np, cpre, U, slots, P, st, K));
-    CUDA_TRY(launch_chained(batch_finalize_kernel, (np + 127) / 128, 128, 0, s, desc, np, slots, cfl));
+    CUDA_TRY(launch_chained(b->chained(), batch_wave_max_kernel, grid_c, kCellTile, 0, s, desc, np, cpre, U, slots, P, st, K));
+    CUDA_TRY(launch_chained(b->chained(), batch_finalize_kernel, (np + 127) / 128, 128, 0, s, desc, np, slots, cfl));
     const int TF = kTiles[tile_idx];
     const int grid_f = b->num_sms * bps;
     const FastK FK = fastk_make(b->common.ct_cr, b->common.ct_alpha1, b->common.ct_alpha2,
@@ -410,7 +410,7 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
         double *const seq[4] = {U, Us, (double *)(ws + b->off_F), U};
         const int32_t *spre = (const int32_t *)(ws + b->off_sprefix);
         for (int stg = 0; stg < 3; stg++)
-            CUDA_TRY(launch_chained(batch_small_kernel, b->sprefix.back(), 192, kBatchSmallBytes, s, desc, np,
+            CUDA_TRY(launch_chained(b->chained(), batch_small_kernel, b->sprefix.back(), 192, kBatchSmallBytes, s, desc, np,
                                     spre, seq[stg], U, seq[stg + 1], slots, st, K, FK, fast, stg + 1));
         return TENO_OK;
     }
@@ -421,11 +421,11 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
             const int first = c * (int)b->chunk_tiles;
             const int count = std::min((int)b->chunk_tiles, b->fprefix[np] - first);
             if (TF == 64)
-                CUDA_TRY(launch_chained(batch_sweep_kernel<64>, grid_f, 64, batch_smem(64), s, desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt));
+                CUDA_TRY(launch_chained(b->chained(), batch_sweep_kernel<64>, grid_f, 64, batch_smem(64), s, desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt));
             else if (TF == 128)
-                CUDA_TRY(launch_chained(batch_sweep_kernel<128>, grid_f, 128, batch_smem(128), s, desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt));
+                CUDA_TRY(launch_chained(b->chained(), batch_sweep_kernel<128>, grid_f, 128, batch_smem(128), s, desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt));
             else
-                CUDA_TRY(launch_chained(batch_sweep_kernel<256>, grid_f, 256, batch_smem(256), s, desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt));
+                CUDA_TRY(launch_chained(b->chained(), batch_sweep_kernel<256>, grid_f, 256, batch_smem(256), s, desc, np, fpre, first, count, Uin, P, B, st, K, FK, fast, cnt));
             DecideArgs d;
             d.B = B;
             d.tiles = count;
@@ -449,10 +449,10 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
                 if (b->has8) CUDA_TRY((launch_decisions<4, false, 0>(d, s, mixed ? 0 : -1)));
                 if (b->has10) CUDA_TRY((launch_decisions<5, false, 0>(d, s, mixed ? 1 : -1)));
             }
-            CUDA_TRY(launch_chained(batch_finish_kernel, (count + 3) / 4, 128, 0, s, desc, np, fpre, first, count, F,
+            CUDA_TRY(launch_chained(b->chained(), batch_finish_kernel, (count + 3) / 4, 128, 0, s, desc, np, fpre, first, count, F,
                                     B, slots, st, K));
         }
-        CUDA_TRY(launch_chained(batch_combine_kernel, grid_c, kCellTile, 0, s, desc, np, cpre, Uin, U,
+        CUDA_TRY(launch_chained(b->chained(), batch_combine_kernel, grid_c, kCellTile, 0, s, desc, np, cpre, Uin, U,
                                 stg == 2 ? U : Us, F, slots, P, st, K, stg + 1));
     }
     return TENO_OK;

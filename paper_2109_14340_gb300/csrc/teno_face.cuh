@@ -336,15 +336,6 @@ struct FaceSmem {
     static constexpr int TOTAL = (TMP + NT * NS + 1) & ~1;         // 16-byte slices
 };
 
-// x / 2 on the exponent bits (no FP64 operation): exact where x / 2 is normal,
-// and for zeros; anything else takes the multiplication.
-__device__ __forceinline__ double half_of(double x)
-{
-    const unsigned hi = (unsigned)__double2hiint(x), e = hi & 0x7ff00000u;
-    if (e - 0x00200000u > 0x7fe00000u - 0x00200000u && __double_as_longlong(x) << 1) return x * 0.5;
-    return __hiloint2double((int)(e ? hi - 0x00100000u : hi), __double2loint(x));
-}
-
 // Sweep modes, a compile-time choice so that each kernel holds only its own
 // code: a plain sweep, one that writes the decision record (flags, argmax,
 // limrec), and one that applies recorded decisions (frozen, frozen_argmax).
@@ -1426,8 +1417,7 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
         for (int c = 0; c < nc; c++) {
             const double Fr = __shfl_down_sync(0xffffffffu, Fo[c], 1);
             const double t = (Fr - Fo[c]) * fuse.inv_dx;
-            double acc = 0.0;
-            acc = acc - t;
+            const double acc = zero_minus(t);
             if (mine && TENO_IN(a.st, ic, a.ncell))
                 fuse.out[c * a.ncell + ic] = stage_value(fuse.mode, acc, Uk[c], Un[c], dt);
         }
@@ -1471,13 +1461,13 @@ cudaError_t launch_decisions(DecideArgs &a, cudaStream_t s, int mixed = -1)
     while (a.group < kDecideMostTiles && a.tiles * sides >= 8 * fill * a.group) a.group *= 2;
     while (a.group == 1 && a.split < 2 * a.nc && a.tiles * sides * a.split <= fill) a.split *= 2;
     const int64_t units = (int64_t)((a.tiles + a.group - 1) / a.group) * a.split * sides;
-    cudaError_t e = launch_chained(decide_kernel<H, RECORD, MIX>,
+    cudaError_t e = launch_chained(a.tiles <= kChainTiles, decide_kernel<H, RECORD, MIX>,
                                    (unsigned)((units + kDecideWarps - 1) / kDecideWarps),
                                    32 * kDecideWarps, 0, s, a, mixed);
     if (e != cudaSuccess) return e;
     const int64_t most = ((int64_t)a.tiles * a.nc + 1) / 2;   // blocks of 128 lanes for every entry
-    return launch_chained(exact_kernel<H, RECORD, MIX>, (unsigned)(sides * (most < 608 ? most : 608)), 128,
-                          0, s, a, (int)(mixed > 0));
+    return launch_chained(a.tiles <= kChainTiles, exact_kernel<H, RECORD, MIX>,
+                          (unsigned)(sides * (most < 608 ? most : 608)), 128, 0, s, a, (int)(mixed > 0));
 }
 
 template <int ND, int H, int MODE>
@@ -1501,11 +1491,12 @@ cudaError_t launch_chunk_mode(const SweepArgs &a, cudaStream_t s)
                 if (e != cudaSuccess) return e;
                 small_done = true;
             }
-            return launch_chained(small_kernel<ND, H, MODE>, (unsigned)a.tiles, 64 * (ND + 2), bytes, s, a);
+            return launch_chained(a.tiles <= kChainTiles, small_kernel<ND, H, MODE>, (unsigned)a.tiles,
+                                  64 * (ND + 2), bytes, s, a);
         }
     }
     const unsigned blocks = (unsigned)((a.tiles + kSweepWarps - 1) / kSweepWarps);
-    cudaError_t e = launch_chained(sweep_kernel<ND, H, MODE>, blocks, 32 * kSweepWarps, smem, s, a);
+    cudaError_t e = launch_chained(a.tiles <= kChainTiles, sweep_kernel<ND, H, MODE>, blocks, 32 * kSweepWarps, smem, s, a);
     if (e != cudaSuccess) return e;
     if (MODE != kSweepFrozen) {
         DecideArgs d;
@@ -1523,7 +1514,8 @@ cudaError_t launch_chunk_mode(const SweepArgs &a, cudaStream_t s)
         e = launch_decisions<H, MODE == kSweepRecord, 0>(d, s);
         if (e != cudaSuccess) return e;
     }
-    return launch_chained(finish_kernel<ND, MODE>, (unsigned)((a.tiles + 3) / 4), 128, 0, s, a);
+    return launch_chained(a.tiles <= kChainTiles, finish_kernel<ND, MODE>, (unsigned)((a.tiles + 3) / 4), 128, 0,
+                          s, a);
 }
 
 // One chunk's fluxes, in the mode its arguments ask for (a decision record to
