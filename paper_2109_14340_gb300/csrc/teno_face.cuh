@@ -828,13 +828,16 @@ __device__ __forceinline__ void decide_unit(const DecideArgs &a, int64_t unit, i
     int n0 = 0, n1 = 0;                                // gathered, per kind (warp-uniform)
     for (int base = (int)(unit % split) * 32; base < total; base += 32 * split) {
         const int e = base + lane;
-        int i = 0;
+        uint32_t q = (uint32_t)(t0 * per) + (uint32_t)e;
+        if (group > 1) {                               // the entry's tile in the group
+            int i = 0;
 #pragma unroll
-        for (int b = kDecideMostTiles / 2; b > 0; b >>= 1) {
-            const int f = __shfl_sync(0xffffffffu, before, i + b);
-            if (i + b < group && e >= f) i += b;
+            for (int b = kDecideMostTiles / 2; b > 0; b >>= 1) {
+                const int f = __shfl_sync(0xffffffffu, before, i + b);
+                if (i + b < group && e >= f) i += b;
+            }
+            q = (uint32_t)((t0 + i) * per) + (uint32_t)(e - __shfl_sync(0xffffffffu, before, i));
         }
-        const uint32_t q = (uint32_t)((t0 + i) * per) + (uint32_t)(e - __shfl_sync(0xffffffffu, before, i));
         int kind = -1;                                 // 0 large stencil, 1 fallback, 2 exact path
         uint8_t fl = 0;
         if (e < total) {
@@ -1424,9 +1427,9 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
     }
 }
 
-// 24 warps per SM at least (20 in 3D), 80 registers (96).
+// 24 warps per SM at least (30 in 1D, 20 in 3D), 80 registers (64, 96).
 template <int ND, int H, int MODE>
-__global__ void __launch_bounds__(64 * (ND + 2), ND == 1 ? 4 : (ND == 2 ? 3 : 2))
+__global__ void __launch_bounds__(64 * (ND + 2), ND == 1 ? 5 : (ND == 2 ? 3 : 2))
     small_kernel(const SweepArgs a)
 {
     extern __shared__ double sm[];

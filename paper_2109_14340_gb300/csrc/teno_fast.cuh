@@ -67,6 +67,7 @@ struct FastK {
     int tiny_ok;                 // flat_ok, and both epsilons at least 2^-136
     float rho_acc[23];           // 3 rho_acc[n]^7 <= thr[n]: x <= rho_acc[n] min_k x_k accepts
                                  // (0: never)
+    float rho_acc2[23];          // 2 rho_acc2[n]^7 <= thr[n]: the same of two others
     float rho_rej[23];           // rho_rej[n]^7 >= thr_rej[n]: x >= rho_rej[n] min_k x_k rejects
     float cr_up;                 // C_r (1 + 1e-5) rounded up
 };
@@ -130,6 +131,7 @@ inline FastK fastk_make(double cr, double alpha1, double alpha2, double eps_beta
     for (int n = 0; n < 23; n++) {
         const double ta = (double)F.thr[n] / 3.0, tr = (double)F.thr_rej[n];
         F.rho_acc[n] = ta > 0.0 ? (float)(pow(ta, 1.0 / 7.0) * (1.0 - 1.0e-6)) : 0.0f;
+        F.rho_acc2[n] = ta > 0.0 ? (float)(pow(1.5 * ta, 1.0 / 7.0) * (1.0 - 1.0e-6)) : 0.0f;
         F.rho_rej[n] = tr > 0.0 ? (float)(pow(tr, 1.0 / 7.0) * (1.0 + 1.0e-6)) : 1.0f;
     }
     F.cr_up = nextafterf((float)(cr * (1.0 + 1.0e-5)), INFINITY);
@@ -165,31 +167,20 @@ __device__ __forceinline__ bool dbits_equal(double a, double b)
 // Bounds [lo, hi] of eta = (|2ab| + eps)/(a^2 + b^2 + eps) from FP32 values
 // a, b with absolute error bounds ea, eb (scaled units), and the exact-zero
 // knowledge of the FP64 differences.  With N = |2ab| <= D = a^2 + b^2,
-// eta - N/D = eps (D - N) / (D (D + eps)) lies in [0, eps/D]; eps_hi: an
-// upper bound of the scaled epsilon.  Squares below 2^-120 give up (hi = 1).
+// N / D <= eta <= (N + eps) / D: the smallest N over the largest D and the other
+// way round (1e-37 for what underflows in it).  eps_hi: an upper bound of the
+// scaled epsilon.  Squares below 2^-120 give up (hi = 1).
 __device__ __forceinline__ void eta_bounds(float a, float ea, bool za, float b, float eb, bool zb,
                                            float eps_hi, float &lo, float &hi)
 {
-    const float tiny = 7.52316385e-37f;                      // 2^-120
-    if (za && zb) { lo = 1.0f; hi = 1.0f; return; }          // (0 + eps) / (0 + eps)
-    if (za || zb) {                                           // eps / (d^2 + eps)
-        const float d = za ? fabsf(b) - eb : fabsf(a) - ea;
-        lo = 0.0f;
-        hi = (d > 0.0f && d * d >= tiny)
-                 ? fminf(__fdividef(eps_hi, d * d) * (1.0f + 1.0e-5f) + 1e-9f, 1.0f) : 1.0f;
-        return;
-    }
-    const float al = fabsf(a) - ea, ah = fabsf(a) + ea;
-    const float bl = fabsf(b) - eb, bh = fabsf(b) + eb;
-    if (!(al > 1e-30f) || !(bl > 1e-30f)) { lo = 0.0f; hi = 1.0f; return; }
-    const float t1 = __fdividef(bl, ah), t2 = __fdividef(bh, al);   // t1 <= t2
-    const float e1 = __fdividef(2.0f * t1, 1.0f + t1 * t1);
-    const float e2 = __fdividef(2.0f * t2, 1.0f + t2 * t2);
-    lo = fminf(e1, e2) * (1.0f - 1.0e-5f);
-    float h = (t1 <= 1.0f && t2 >= 1.0f) ? 1.0f : fmaxf(e1, e2) * (1.0f + 1.0e-5f);
-    const float D = al * al + bl * bl;
-    h = D >= tiny ? h + __fdividef(eps_hi, D) * (1.0f + 1.0e-5f) : 1.0f;
-    hi = fminf(h + 1e-9f, 1.0f);
+    const float aa = za ? 0.0f : fabsf(a), ab = zb ? 0.0f : fabsf(b);
+    const float xa = za ? 0.0f : ea, xb = zb ? 0.0f : eb;
+    const float al = fmaxf(aa - xa, 0.0f), ah = aa + xa, bl = fmaxf(ab - xb, 0.0f), bh = ab + xb;
+    const float Dl = fmaf(al, al, bl * bl), Dh = fmaf(ah, ah, bh * bh) + 1.0e-37f;
+    lo = __fdividef(2.0f * (al * bl), Dh) * (1.0f - 1.0e-5f);
+    hi = Dl >= 7.52316385e-37f                                          // 2^-120
+             ? fminf(__fdividef(fmaf(2.0f * ah, bh, eps_hi), Dl) * (1.0f + 1.0e-5f) + 1e-9f, 1.0f) : 1.0f;
+    if (za && zb) lo = hi = 1.0f;                            // (0 + eps) / (0 + eps)
 }
 
 // g(m) = ((1-m)^2)^2 (1+4m) in FP32.
@@ -797,7 +788,7 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const Fast
     const float thr = F.thr[nexp], thr_rej = F.thr_rej[nexp];
 
     // Targeted selection, largest group first (Sec. 3.3).
-    const float acc = F.rho_acc[nexp], rej = F.rho_rej[nexp];
+    const float acc = F.rho_acc[nexp], acc2 = F.rho_acc2[nexp], rej = F.rho_rej[nexp];
     const int sel = select_large<H, H>(o.f, blo, bhi, tiny2, ebl, ebh, x0, x1, x2, X0, X1, X2, thr,
                                        thr_rej, acc * xmin, rej * Xmin);
     if (sel < 0) return false;
@@ -818,7 +809,7 @@ __device__ __forceinline__ bool fast_decide(const double (&v)[2 * H], const Fast
         for (int k = 0; k < 3; k++) {
             const int j1 = k == 0 ? 1 : 0, j2 = k == 2 ? 1 : 2;
             // as in select_large, with the two others' smaller one
-            if (xu[k] <= acc * (fminf(xl[j1], xl[j2]) * (1.0f - 2.0e-6f))) d[k] = 1;
+            if (xu[k] <= acc2 * (fminf(xl[j1], xl[j2]) * (1.0f - 2.0e-6f))) d[k] = 1;
             else if (xl[k] >= rej * (fminf(xu[j1], xu[j2]) * (1.0f + 2.0e-6f))) d[k] = 0;
             else if (pow7_sum2(xu[k], xl[j1], xl[j2], true) <= thr) d[k] = 1;
             else if (pow7_sum2(xl[k], xu[j1], xu[j2], false) > thr_rej) d[k] = 0;
