@@ -128,7 +128,10 @@ typedef struct teno_params {
  * TENO8-AA, LLF, no limiter, periodic 1D grid of one cell (caller sets n, dx). */
 void teno_params_init(teno_params *p);
 
-/* Workspace bytes needed by every call below for these parameters.
+/* Workspace bytes needed by every call below for these parameters: status
+ * header, face fluxes, one stage state, the primitive rows, and the buffers of
+ * the face sweeps' queue (0.5 to 1.4 KB per face, up to 2.1 million faces at a
+ * time: 1.1 to 2.8 GB for every larger grid).
  * Returns TENO_EINVAL for invalid parameters (then *bytes is untouched). */
 int teno_workspace_bytes(const teno_params *p, size_t *bytes);
 
@@ -230,7 +233,7 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
 int teno_batch_workspace_bytes(const teno_batch *b, size_t *bytes);
 
 /* Autotuner: times one step (TENO_BATCH_STREAM) of every candidate tile width
- * (64/128/256 faces, i.e. 2/4/8 warps per pencil tile) and persistent grid size
+ * (64/128/256 faces in flight, i.e. 2/4/8 warps) and persistent grid size
  * (1/2/3/4/6 blocks per SM) on U_scratch (advanced in place: pass a copy) and keeps
  * the fastest in the plan.  Results do not depend on the choice.
  * *chosen_tile and *chosen_blocks_per_sm (nullable) report it. */
@@ -344,7 +347,7 @@ int teno_wave_speeds(const teno_params *p, const double *U, double *amax_device,
 int teno_dt_from_speeds(const teno_params *p, const double *amax_device, int32_t ncopies,
                         double cfl, double *dt_device, void *stream);
 
-/* Size of the device array behind teno_rhs_static: 16 MiB. */
+/* Size of the device array that bounds teno_rhs_static's grids: 16 MiB. */
 #define TENO_RHS_STATIC_SCRATCH_BYTES (16u << 20)
 
 /* teno_rhs without a workspace, for callers that cannot allocate device
@@ -353,8 +356,10 @@ int teno_dt_from_speeds(const teno_params *p, const double *amax_device, int32_t
  * fixed at start-up, code that must not call cudaMalloc while a CUDA graph
  * is captured).  The paper has no counterpart; this is an integration aid.
  *   Same arguments and result as teno_rhs, minus ws / ws_bytes.  Scratch is
- *   one file-scope device array of TENO_RHS_STATIC_SCRATCH_BYTES, present on
- *   every GPU where the library's kernels are loaded until the process exits.
+ *   one file-scope device array of TENO_RHS_STATIC_SCRATCH_BYTES, and a second
+ *   one of 32 MiB that the face sweeps work through in pieces (it limits no
+ *   grid), present on every GPU where the library's kernels are loaded until
+ *   the process exits.
  *   Problems whose status header plus face-flux buffers (256 bytes + 8 *
  *   ncons * sum over directions of the face-grid size, each part rounded up
  *   to 256 bytes) exceed it are rejected with TENO_EINVAL before anything is
@@ -365,9 +370,9 @@ int teno_dt_from_speeds(const teno_params *p, const double *amax_device, int32_t
  *   the id of the context it came from and resolved again when another
  *   context is current (after cudaDeviceReset, which unloads the array with
  *   the context), so that first-call rule applies again after a reset.
- *   All calls share the one array and each zeroes its status header: calls
+ *   All calls share the arrays and each zeroes the status header: calls
  *   whose work overlaps on the GPU (different streams, or different host
- *   threads without ordering) race on it and must be serialised by the
+ *   threads without ordering) race on them and must be serialised by the
  *   caller.  The non-physical counter is not reported (teno_status needs a
  *   workspace). */
 int teno_rhs_static(const teno_params *p, const double *U, double *rhs, double dt_limiter,
@@ -397,9 +402,10 @@ int teno_reconstruct(const teno_params *p, const double *v, int64_t count, doubl
  * with concurrent launches. */
 int teno_set_decision_filter(int on);
 
-/* Live timing of the dominant kernel (the face-sweep kernel) for roofline
- * reporting.  teno_profile_enable(1) clears the record and from then on
- * brackets every face-sweep launch with a pair of CUDA events recorded on
+/* Live timing of the dominant kernels (the face fluxes' sweep, decide, exact
+ * and finish kernels) for roofline reporting.  teno_profile_enable(1) clears
+ * the record and from then on brackets every group of face-flux launches (up to
+ * 2.1 million faces) with a pair of CUDA events recorded on
  * the launch's stream (at most 8192 launches are recorded); (0) stops.
  * teno_profile_read synchronises the recorded events and returns the summed
  * device milliseconds, the number of launches, the number of faces they

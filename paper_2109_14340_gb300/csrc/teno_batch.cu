@@ -2,11 +2,14 @@
 // Euler problems of uneven size advanced together with per-problem CFL steps.
 //
 // One step = per-problem wave-speed maxima (persistent, one block per
-// (problem, 256-cell tile)) -> per-problem dt -> three stages, each a
-// persistent face sweep that pulls (problem, face tile) items from an atomic
-// counter, then a combine over (problem, cell tile) items.  The face and cell
-// arithmetic is the single-problem code (face_block, cell_quantities), so the
-// results are bitwise those of teno_cfl_dt + teno_rk3_step per problem.
+// (problem, 256-cell tile)) -> per-problem dt -> three stages.  A stage is a
+// persistent sweep whose warps pull (problem, 32-face tile) items from an atomic
+// counter, the decisions and values of what the sweep queued, the
+// back-projection, and a combine over (problem, cell tile) items; batches of few
+// tiles take a stage in one launch (batch_small_kernel).  The face and cell
+// arithmetic is the single-problem code (sweep_tile, small_tile, finish_face,
+// cell_quantities), so the results are bitwise those of teno_cfl_dt +
+// teno_rk3_step per problem.
 #include <algorithm>
 #include <cstring>
 #include <new>

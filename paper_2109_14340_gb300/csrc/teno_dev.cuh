@@ -642,28 +642,4 @@ __device__ __forceinline__ double r_entry(const RoeScalars<ND> &rs, int c, int k
     return (c == 1 + t) ? 1.0 : 0.0;
 }
 
-template <int ND, int D>
-__device__ __forceinline__ double roe_eigensystem(const double (&ul)[ND], double Hl, double sl,
-                                                  const double (&ur)[ND], double Hr, double sr,
-                                                  double gm1, double (&Lm)[ND + 2][ND + 2],
-                                                  double (&Rm)[ND + 2][ND + 2],
-                                                  RoeScalars<ND> *rsp = nullptr)
-{
-    constexpr int nc = ND + 2;
-    RoeScalars<ND> rs;
-    const double c2 = roe_state<ND, D>(ul, Hl, sl, ur, Hr, sr, gm1, rs);
-#pragma unroll
-    for (int k = 0; k < nc; k++) {
-        double l[nc];
-        l_row<ND, D>(rs, k, l);
-#pragma unroll
-        for (int c = 0; c < nc; c++) {
-            Lm[k][c] = l[c];
-            Rm[c][k] = r_entry<ND, D>(rs, c, k);
-        }
-    }
-    if (rsp) *rsp = rs;
-    return c2;
-}
-
 }  // namespace teno
