@@ -262,18 +262,36 @@ __device__ __forceinline__ double fallback_value(const double (&v)[2 * H], int m
 #undef V
 }
 
+// What a reconstruction's tests share: the small stencils' separations and the
+// exponent of C_T.
+struct ReconTests {
+    double g0, g1, g2;
+    int nexp;
+};
+
+// Whether S_L passes its test against the small stencils (Sec. 3.3; a NaN passes).
+template <int H, int L>
+__device__ __forceinline__ bool recon_passes(const double (&v)[2 * H], const Consts &K,
+                                             const ReconTests &t)
+{
+    const double g = scale_sep(beta_large<H, L>(v), K.eps_beta);
+    const double chi = g / (((t.g0 + t.g1) + t.g2) + g);
+    return !(chi < TENO_TENPOW[t.nexp]);
+}
+
+__device__ __forceinline__ uint8_t ct_bits(int nexp) { return (uint8_t)(((nexp - 7) & 7) << 5); }
+
 // One reconstruction; flag: bits 0-1 selected large stencil (L-2) or 0 for the
 // small-stencil fallback, bits 2-4 deltas of S0..S2 (fallback), bits 5-7 C_T
-// exponent minus 7; S6 as bits 0-4 zero (large_code).
+// exponent minus 7; S6 as bits 0-4 zero (large_code).  In two parts: the tests'
+// inputs and the first group of the targeted ENO-like selection (Sec. 3.3), and
+// the rest of it.
 template <int H>
-__device__ __forceinline__ double teno_recon(const double (&v)[2 * H], const Consts &K,
-                                             uint8_t &flag)
+__device__ __forceinline__ bool recon_largest(const double (&v)[2 * H], const Consts &K,
+                                              ReconTests &t, double &out, uint8_t &flag)
 {
 #define V(m) v[(m) + H - 1]
-    const int nexp = ct_exponent<H>(v, K);
-    const double CT = TENO_TENPOW[nexp];
-    const uint8_t fct = (uint8_t)(((nexp - 7) & 7) << 5);
-
+    t.nexp = ct_exponent<H>(v, K);
     double a0 = V(-1) - V(1);
     double b0 = (V(-1) - 2.0 * V(0)) + V(1);
     double beta0 = 0.25 * (a0 * a0) + (13.0 / 12.0) * (b0 * b0);
@@ -283,41 +301,47 @@ __device__ __forceinline__ double teno_recon(const double (&v)[2 * H], const Con
     double a2 = (V(-2) - 4.0 * V(-1)) + 3.0 * V(0);
     double b2 = (V(-2) - 2.0 * V(-1)) + V(0);
     double beta2 = 0.25 * (a2 * a2) + (13.0 / 12.0) * (b2 * b2);
-    double g0 = scale_sep(beta0, K.eps_beta);
-    double g1 = scale_sep(beta1, K.eps_beta);
-    double g2 = scale_sep(beta2, K.eps_beta);
-    double g012 = (g0 + g1) + g2;
+    t.g0 = scale_sep(beta0, K.eps_beta);
+    t.g1 = scale_sep(beta1, K.eps_beta);
+    t.g2 = scale_sep(beta2, K.eps_beta);
+    if (!recon_passes<H, H>(v, K, t)) return false;
+    flag = (uint8_t)((H == 6 ? 0 : H - 2) | ct_bits(t.nexp));
+    out = flux_large<H, H>(v);
+    return true;
+#undef V
+}
 
-    // Targeted ENO-like selection (Sec. 3.3), largest group first.
+template <int H>
+__device__ __forceinline__ double recon_smaller(const double (&v)[2 * H], const Consts &K,
+                                                const ReconTests &t, uint8_t &flag)
+{
+    const uint8_t fct = ct_bits(t.nexp);
     if constexpr (H == 6) {
-        double g6 = scale_sep(beta_large<H, 6>(v), K.eps_beta);
-        double chi = g6 / (g012 + g6);
-        if (!(chi < CT)) { flag = fct; return flux_large<H, 6>(v); }
+        if (recon_passes<H, 5>(v, K, t)) { flag = (uint8_t)(3 | fct); return flux_large<H, 5>(v); }
     }
     if constexpr (H >= 5) {
-        double g5 = scale_sep(beta_large<H, 5>(v), K.eps_beta);
-        double chi = g5 / (g012 + g5);
-        if (!(chi < CT)) { flag = (uint8_t)(3 | fct); return flux_large<H, 5>(v); }
+        if (recon_passes<H, 4>(v, K, t)) { flag = (uint8_t)(2 | fct); return flux_large<H, 4>(v); }
     }
-    {
-        double g4 = scale_sep(beta_large<H, 4>(v), K.eps_beta);
-        double chi = g4 / (g012 + g4);
-        if (!(chi < CT)) { flag = (uint8_t)(2 | fct); return flux_large<H, 4>(v); }
-    }
-    {
-        double g3 = scale_sep(beta_large<H, 3>(v), K.eps_beta);
-        double chi = g3 / (g012 + g3);
-        if (!(chi < CT)) { flag = (uint8_t)(1 | fct); return flux_large<H, 3>(v); }
-    }
+    if (recon_passes<H, 3>(v, K, t)) { flag = (uint8_t)(1 | fct); return flux_large<H, 3>(v); }
 
     // Small-stencil fallback (Eq. renormalize, Eq. reconstuction), normalised
     // over S0, S1, S2.
-    double s = g012;
-    int d0 = !(g0 / s < CT), d1 = !(g1 / s < CT), d2 = !(g2 / s < CT);
+    const double CT = TENO_TENPOW[t.nexp];
+    const double s = (t.g0 + t.g1) + t.g2;
+    int d0 = !(t.g0 / s < CT), d1 = !(t.g1 / s < CT), d2 = !(t.g2 / s < CT);
     const int mask = d0 | (d1 << 1) | (d2 << 2);
     flag = (uint8_t)((mask << 2) | fct);
     return fallback_value<H>(v, mask);
-#undef V
+}
+
+template <int H>
+__device__ __forceinline__ double teno_recon(const double (&v)[2 * H], const Consts &K,
+                                             uint8_t &flag)
+{
+    ReconTests t;
+    double out;
+    if (recon_largest<H>(v, K, t, out, flag)) return out;
+    return recon_smaller<H>(v, K, t, flag);
 }
 
 // Coefficient of S_L's linear scheme at value index m of a 2H stencil, and

@@ -1046,57 +1046,123 @@ __device__ __forceinline__ double exact_warp(const double (&v)[2 * H], int row, 
 }
 
 // The listed reconstructions through the exact path: a warp for each while they
-// are few (at most kExactFew), a lane for each when they fill warps.
+// are few (at most kExactFew), a lane for each when they fill warps.  Bound by
+// the FP64 pipe (86 % busy).
 constexpr unsigned kExactFew = 152 * 16;
 
-template <int H, bool RECORD>
-__device__ __forceinline__ void exact_list(const DecideArgs &a, int which, unsigned block, unsigned blocks)
+// Entries of a long list that the largest stencil's test rejected, with what the
+// other tests need, until a warp of them is together: some 3 % reject in smooth
+// flow, spread over two thirds of the warps, whose lanes would all wait for the
+// smaller stencils' forms.
+struct ExactRest {
+    ReconTests t[64];
+    uint32_t q[64];
+};
+
+// Value (and, RECORD, decision byte) of entry q to its owner's place.
+template <bool RECORD>
+__device__ __forceinline__ void exact_out(const DecideArgs &a, uint32_t q, double val, uint8_t fl)
 {
-    constexpr int W = 2 * H;
     const SweepBuf &B = a.B;
-    const int nc = a.nc;
-    const int64_t per = 64 * nc, nq = B.nt * per, nf = B.nt * kTileFaces;
+    const uint32_t per = 64u * a.nc;
+    const int64_t nf = B.nt * kTileFaces;
+    const int slot = B.qslot[q];
+    const int64_t o = (slot >> 5) * nf + (int64_t)(q / per) * kTileFaces + (slot & 31);
+    if (!TENO_IN(a.st, o, 2 * a.nc * nf)) return;
+    B.R[o] = val;
+    if (RECORD) B.RD[o] = fl;
+}
+
+template <int H>
+__device__ __forceinline__ void exact_in(const SweepBuf &B, int64_t nq, uint32_t q, double (&v)[2 * H])
+{
+#pragma unroll
+    for (int kk = 0; kk < 2 * H; kk++) v[kk] = B.qv[kk * nq + q];
+}
+
+template <int H, bool RECORD>
+__device__ __forceinline__ void exact_list(const DecideArgs &a, int which, unsigned block,
+                                           unsigned blocks, ExactRest &rest)
+{
+    const SweepBuf &B = a.B;
+    const int64_t nq = B.nt * 64 * a.nc;
     const unsigned n = *a.nexact[which];
     if (n == 0) return;
     if (a.exact_count && block == 0 && threadIdx.x == 0)
         atomicAdd(a.exact_count, (unsigned long long)n);
-    const bool few = n <= kExactFew;
-    int row = -1;
-    double qc[W];
+    const int lane = threadIdx.x & 31;
+    const unsigned warp = block * (blockDim.x >> 5) + (threadIdx.x >> 5), warps = blocks * (blockDim.x >> 5);
+    if (n <= kExactFew) {
+        int row = -1;
+        double qc[2 * H];
 #pragma unroll
-    for (int c = 0; c < W; c++) qc[c] = 0.0;           // beyond the row's stencil
-    if (few) exact_row<H, H>(threadIdx.x & 31, row, qc);
-    const unsigned step = few ? blocks * (blockDim.x >> 5) : blocks * blockDim.x;
-    for (unsigned i = few ? block * (blockDim.x >> 5) + (threadIdx.x >> 5) : block * blockDim.x + threadIdx.x;
-         i < n; i += step) {
-        const uint32_t q = a.xlist[which][i];
-        if (!TENO_IN(a.st, q, nq)) continue;
-        double v[W];
-#pragma unroll
-        for (int kk = 0; kk < W; kk++) v[kk] = B.qv[kk * nq + q];
-        const int slot = B.qslot[q];
-        const int64_t o = (slot >> 5) * nf + (int64_t)(q / (uint32_t)per) * kTileFaces + (slot & 31);
-        if (!TENO_IN(a.st, o, 2 * nc * nf)) continue;
-        uint8_t fl;
-        const double val = few ? exact_warp<H>(v, row, qc, a.K, fl) : teno_recon<H>(v, a.K, fl);
-        if (!few || (threadIdx.x & 31) == 0) {
-            B.R[o] = val;
-            if (RECORD) B.RD[o] = fl;
+        for (int c = 0; c < 2 * H; c++) qc[c] = 0.0;   // beyond the row's stencil
+        exact_row<H, H>(lane, row, qc);
+        for (unsigned i = warp; i < n; i += warps) {
+            const uint32_t q = a.xlist[which][i];
+            if (!TENO_IN(a.st, q, nq)) continue;
+            double v[2 * H];
+            exact_in<H>(B, nq, q, v);
+            uint8_t fl;
+            const double val = exact_warp<H>(v, row, qc, a.K, fl);
+            if (lane == 0) exact_out<RECORD>(a, q, val, fl);
         }
+        return;
+    }
+    int held = 0;                                      // gathered (warp-uniform)
+    for (unsigned base = warp * 32; base < n; base += warps * 32) {
+        const bool last = base + warps * 32 >= n;
+        bool rejected = false;
+        uint32_t q = 0;
+        ReconTests t;
+        if (base + lane < n) {
+            q = a.xlist[which][base + lane];
+            if (TENO_IN(a.st, q, nq)) {
+                double v[2 * H], val;
+                uint8_t fl;
+                exact_in<H>(B, nq, q, v);
+                rejected = !recon_largest<H>(v, a.K, t, val, fl);
+                if (!rejected) exact_out<RECORD>(a, q, val, fl);
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, rejected);
+        if (rejected) {
+            const int at = held + __popc(m & ((1u << lane) - 1u));
+            rest.t[at] = t;
+            rest.q[at] = q;
+        }
+        held += __popc(m);
+        __syncwarp();
+        while (held >= 32 || (last && held > 0)) {
+            const int k = min(held, 32);
+            held -= k;
+            if (lane < k) {
+                const ReconTests tr = rest.t[held + lane];
+                const uint32_t qr = rest.q[held + lane];
+                double v[2 * H];
+                uint8_t fl;
+                exact_in<H>(B, nq, qr, v);
+                const double val = recon_smaller<H>(v, a.K, tr, fl);
+                exact_out<RECORD>(a, qr, val, fl);
+            }
+        }
+        __syncwarp();
     }
 }
 
 template <int H, bool RECORD, int MIX>
 __global__ void __launch_bounds__(128) exact_kernel(const DecideArgs a, int which)
 {
+    __shared__ ExactRest rest_[4];
+    ExactRest &rest = rest_[threadIdx.x >> 5];
     chain_next();
     chain_wait();
     if constexpr (MIX == 0) {
-        exact_list<H, RECORD>(a, which, blockIdx.x, gridDim.x);
+        exact_list<H, RECORD>(a, which, blockIdx.x, gridDim.x, rest);
     } else if (blockIdx.x & 1) {
-        exact_list<5, RECORD>(a, 1, blockIdx.x >> 1, gridDim.x >> 1);
+        exact_list<5, RECORD>(a, 1, blockIdx.x >> 1, gridDim.x >> 1, rest);
     } else {
-        exact_list<4, RECORD>(a, 0, blockIdx.x >> 1, gridDim.x >> 1);
+        exact_list<4, RECORD>(a, 0, blockIdx.x >> 1, gridDim.x >> 1, rest);
     }
 }
 
