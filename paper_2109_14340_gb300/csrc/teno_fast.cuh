@@ -353,6 +353,10 @@ __device__ __forceinline__ constexpr float sos_bound(int which)
 // C_r ((|a| + e)^2 + (|b| + e)^2) for the four pairs of neighbouring differences
 // (its epsilon only raises eta).
 //
+// Bit-identical finite values (states that no wave has reached) are accepted here
+// too, at the smooth exponent: a step of 4096 tubes with sharp initial states
+// takes 25.5 ms, 26.9 with those in the queue.
+//
 // The shifted values come from the bit patterns: every value, scaled by a
 // power of two to below 2, is cut exactly into h (24 bits) and l (the next
 // 23), and s_m = (h_m - h_0) + (l_m - l_0).  With M = max |s_m| and the error
@@ -447,8 +451,18 @@ __device__ __forceinline__ bool quick_large(const double (&v)[2 * H], const Fast
 #undef SS
     const float any = need_ct ? 0.0f : F.rho_acc[F.nexp_min];
     const float rho = smooth ? fmaxf(any, F.rho_acc[F.nexp_smooth]) : any;
-    flag = (uint8_t)(large_code(H) | (need_ct ? ((F.nexp_smooth - 7) & 7) << 5 : 0));
-    return range && M >= 9.5367431640625e-7f && xp <= rho * xs;
+    bool flat = false;
+    if (M == 0.0f && ev != 0x7FFu && F.flat_ok) {
+        unsigned differ = 0u;
+#pragma unroll
+        for (int j = 1; j < W; j++) {
+            differ |= (unsigned)(__double2hiint(v[j]) ^ __double2hiint(v[0]));
+            differ |= (unsigned)(__double2loint(v[j]) ^ __double2loint(v[0]));
+        }
+        flat = differ == 0u;
+    }
+    flag = (uint8_t)(large_code(H) | (need_ct || flat ? ((F.nexp_smooth - 7) & 7) << 5 : 0));
+    return flat || (range && M >= 9.5367431640625e-7f && xp <= rho * xs);
 }
 
 // A small indicator's FP64 input as the exact path forms it, converted to

@@ -16,6 +16,7 @@ if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
 import paper_2109_14340_gb300 as T
+import workloads
 
 
 def recon(scheme, v, fast, flags=False):
@@ -63,3 +64,29 @@ def test_quick_acceptance_matches_fp64(scheme):
         same = (a == b) | (torch.isnan(a) & torch.isnan(b))
         bad = (~same).nonzero().flatten()
         assert bad.numel() == 0, (bad.numel(), v[bad[0]].tolist(), a[bad[0]].item(), b[bad[0]].item())
+
+
+@pytest.mark.parametrize("over", [dict(), dict(ct_cr=2.0), dict(ct_alpha1=0.5, ct_alpha2=0.0)],
+                         ids=["paper", "cr-2", "ct-1"])
+@pytest.mark.parametrize("case", [
+    workloads.riemann_1d(517, scheme=8), workloads.riemann_1d(140000, scheme=12),
+    workloads.quadrants_2d(250, 231, scheme=10)], ids=["1d-517", "1d-140000", "2d"])
+def test_bit_identical_stencils(case, over):
+    """Sharp initial states: most stencils hold bit-identical values (velocities at
+    rest give zeros).  They are accepted by the first test only where its premise
+    holds; with C_r > 1, or C_T = 1 at m = 0, they must go the whole way.  Filter on
+    = filter off, bitwise, records included (NaN where a fallback keeps nothing)."""
+    p = T.teno_params_init(ndim=case["ndim"], n=case["n"], dx=case["dx"], scheme=case["scheme"],
+                           gamma=case["gamma"], bc_lo=case["bc_lo"], bc_hi=case["bc_hi"], **over)
+    s = T.Solver(p)
+    U = torch.from_numpy(case["U"]).cuda()
+    on, f_on = s.rhs(U, flags=True)
+    plain = s.rhs(U)
+    T.teno_set_decision_filter(0)
+    try:
+        off, f_off = s.rhs(U, flags=True)
+    finally:
+        T.teno_set_decision_filter(1)
+    assert torch.equal(f_on, f_off)
+    for r in (on, plain):
+        assert torch.equal(r.nan_to_num(7.0), off.nan_to_num(7.0))
