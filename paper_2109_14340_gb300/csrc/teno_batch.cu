@@ -653,7 +653,9 @@ int teno_batch_autotune(teno_batch *b, double *U_scratch, void *ws, size_t ws_by
     float best = 1e30f;
     int best_t = b->tile_idx, best_b = b->blocks_per_sm;
     const int bps_c[5] = {1, 2, 3, 4, 6};
-    for (int ti = 0; ti < 3; ti++) {
+    // the fused stages of a small batch have no such choice: every candidate would run
+    // the same launches
+    for (int ti = 0; ti < (b->small() ? 0 : 3); ti++) {
         for (int bi = 0; bi < 5; bi++) {
             int maxb = 0;
             const int TF = kTiles[ti];
