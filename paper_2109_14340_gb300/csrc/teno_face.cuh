@@ -10,15 +10,21 @@
 // lanes would diverge, over four kernels that pass values through memory
 // (about 1 kB per face at most, of a bandwidth that FP64 work leaves idle):
 //
-//   sweep   a warp per tile of 32 faces, a lane per face: staging, Roe state, projection, split fluxes.  Reconstructions
-//           that quick_large accepts for the largest stencil get their value;
-//           the others go to the tile's queue.
-//   decide  the queues of several tiles by one block: the whole filter for
-//           each entry, then the values, the large stencils' and the
-//           fallback's each on compact lanes.  What the filter leaves open
-//           goes to one list.
-//   exact   that list through the exact path, a lane per entry.
+//   sweep   a warp per tile of 32 faces, a lane per face: staging, Roe state,
+//           projection, split fluxes.  Reconstructions that quick_large accepts
+//           for the largest stencil get their value; the others go to the
+//           tile's queue.
+//   decide  the queues of several tiles by a warp: the whole filter for each
+//           entry, then the values, the large stencils' and the fallback's each
+//           on compact lanes.  What the filter leaves open goes to one list.
+//   exact   that list through the exact path, a lane or a warp per entry.
 //   finish  a lane per face: back-projection, limiter, the flux.
+//
+// 2 M faces of 128^3 TENO10 (smooth flow): sweep 2.61 ms, its FP64 unit 90 %
+// busy with 701 instructions per 32 faces; decide 0.18 to 0.26 ms, bound by the
+// instructions it issues (53 % of the slots; FP64 43 %); exact 0.02 to 0.04 ms;
+// finish 0.12 ms, FP64 86 % busy: 3.0 ms.  One kernel with its queue in shared
+// memory took 3.6 to 3.9 ms (FP64 80 to 84 % busy, 824 to 839 instructions).
 //
 // The buffers between them are sized for at most kChunkTiles tiles, so a larger
 // evaluation goes through them in chunks.  U and F are staged halved (exact: a
@@ -1080,19 +1086,25 @@ __device__ __forceinline__ void exact_in(const SweepBuf &B, int64_t nq, uint32_t
     for (int kk = 0; kk < 2 * H; kk++) v[kk] = B.qv[kk * nq + q];
 }
 
+// which: the list; kExactAll: every queued entry, where there is no filter to make
+// a list (the queues' lanes are nearly all filled then).
+constexpr int kExactAll = -1;
+
 template <int H, bool RECORD>
 __device__ __forceinline__ void exact_list(const DecideArgs &a, int which, unsigned block,
                                            unsigned blocks, ExactRest &rest)
 {
     const SweepBuf &B = a.B;
-    const int64_t nq = B.nt * 64 * a.nc;
-    const unsigned n = *a.nexact[which];
+    const uint32_t per = 64u * a.nc;
+    const int64_t nq = B.nt * per;
+    const bool all = which == kExactAll;
+    const unsigned n = all ? (unsigned)a.tiles * per : *a.nexact[which];
     if (n == 0) return;
-    if (a.exact_count && block == 0 && threadIdx.x == 0)
+    if (a.exact_count && !all && block == 0 && threadIdx.x == 0)
         atomicAdd(a.exact_count, (unsigned long long)n);
     const int lane = threadIdx.x & 31;
     const unsigned warp = block * (blockDim.x >> 5) + (threadIdx.x >> 5), warps = blocks * (blockDim.x >> 5);
-    if (n <= kExactFew) {
+    if (!all && n <= kExactFew) {
         int row = -1;
         double qc[2 * H];
 #pragma unroll
@@ -1115,8 +1127,19 @@ __device__ __forceinline__ void exact_list(const DecideArgs &a, int which, unsig
         bool rejected = false;
         uint32_t q = 0;
         ReconTests t;
-        if (base + lane < n) {
+        bool have = base + lane < n;
+        if (have && all) {
+            q = base + lane;
+            const uint32_t tile = q / per;
+            have = q - tile * per < (B.count[tile] & 0x7fffffffu);
+        } else if (have) {
             q = a.xlist[which][base + lane];
+        }
+        if (all && a.exact_count) {
+            const unsigned m = __ballot_sync(0xffffffffu, have);
+            if (lane == 0 && m) atomicAdd(a.exact_count, (unsigned long long)__popc(m));
+        }
+        if (have) {
             if (TENO_IN(a.st, q, nq)) {
                 double v[2 * H], val;
                 uint8_t fl;
@@ -1517,6 +1540,13 @@ __global__ void __launch_bounds__(64 * (ND + 2), ND == 1 ? 5 : (ND == 2 ? 3 : 2)
     small_tile<ND, H, MODE>(a.g, a.dir[d], a.FK, a.K, d, f0, x, y, z, a.exact_count, sm, a.fuse);
 }
 
+// Blocks of the exact kernel: 128 lanes for every possible entry, at most a wave.
+inline int64_t exact_blocks(const DecideArgs &a)
+{
+    const int64_t most = ((int64_t)a.tiles * a.nc + 1) / 2;
+    return most < 608 ? most : 608;
+}
+
 // The decide and exact kernels of one chunk (a's group and split are set here).
 // mixed: in a batch of both schemes, the one to take (MIX = 0).
 template <int H, bool RECORD, int MIX>
@@ -1534,9 +1564,8 @@ cudaError_t launch_decisions(DecideArgs &a, cudaStream_t s, int mixed = -1)
                                    (unsigned)((units + kDecideWarps - 1) / kDecideWarps),
                                    32 * kDecideWarps, 0, s, a, mixed);
     if (e != cudaSuccess) return e;
-    const int64_t most = ((int64_t)a.tiles * a.nc + 1) / 2;   // blocks of 128 lanes for every entry
     return launch_chained(a.tiles <= kChainTiles, exact_kernel<H, RECORD, MIX>,
-                          (unsigned)(sides * (most < 608 ? most : 608)), 128, 0, s, a, (int)(mixed > 0));
+                          (unsigned)(sides * exact_blocks(a)), 128, 0, s, a, (int)(mixed > 0));
 }
 
 template <int ND, int H, int MODE>
@@ -1580,7 +1609,11 @@ cudaError_t launch_chunk_mode(const SweepArgs &a, cudaStream_t s)
         d.st = a.g.st;
         d.FK = a.FK;
         d.K = a.K;
-        e = launch_decisions<H, MODE == kSweepRecord, 0>(d, s);
+        // no filter: the exact kernel takes the queues as they are (a pass of the decide
+        // kernel that only lists them costs 0.45 ms per 2 M faces)
+        e = d.fast ? launch_decisions<H, MODE == kSweepRecord, 0>(d, s)
+                   : launch_chained(a.tiles <= kChainTiles, exact_kernel<H, MODE == kSweepRecord, 0>,
+                                    (unsigned)exact_blocks(d), 128, 0, s, d, kExactAll);
         if (e != cudaSuccess) return e;
     }
     return launch_chained(a.tiles <= kChainTiles, finish_kernel<ND, MODE>, (unsigned)((a.tiles + 3) / 4), 128, 0,
