@@ -357,7 +357,7 @@ int teno_dt_from_speeds(const teno_params *p, const double *amax_device, int32_t
  * is captured).  The paper has no counterpart; this is an integration aid.
  *   Same arguments and result as teno_rhs, minus ws / ws_bytes.  Scratch is
  *   one file-scope device array of TENO_RHS_STATIC_SCRATCH_BYTES, and a second
- *   one of 32 MiB that the face sweeps work through in pieces (it limits no
+ *   one of 192 MiB that the face sweeps work through in pieces (it limits no
  *   grid), present on every GPU where the library's kernels are loaded until
  *   the process exits.
  *   Problems whose status header plus face-flux buffers (256 bytes + 8 *
@@ -421,8 +421,8 @@ int teno_profile_read(double *ms, int64_t *launches, int64_t *faces, int64_t *ex
 
 /* Bounds-checked build (libteno_gb300_debug.so, compiled with
  * -DTENO_DEBUG_BOUNDS; the same entry points): every global-memory index of
- * the face sweeps, the combine and the primitives kernel, and the sweeps'
- * shared-memory queue indices, are range-checked on the device; an index
+ * the face-flux kernels and their queue, the combine and the primitives
+ * kernel, is range-checked on the device; an index
  * outside its array is counted in the workspace's status block and the
  * access is skipped or redirected to an element inside the array (a load
  * gives 0), never faulting.  teno_debug_bounds synchronises the stream,

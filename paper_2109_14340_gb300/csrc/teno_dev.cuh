@@ -54,9 +54,9 @@ struct Status {
 };
 static_assert(sizeof(Status) == 256, "status block is 256 bytes");
 
-// Debug build (-DTENO_DEBUG_BOUNDS): every global-memory index of the face
-// sweeps, the combine and the primitives kernel, and the face sweeps'
-// shared-memory queue indices, are range-checked.  An index outside its
+// Debug build (-DTENO_DEBUG_BOUNDS): every global-memory index of the face-flux
+// kernels and their queue, the combine and the primitives kernel, is
+// range-checked.  An index outside its
 // array is counted in the status block (with the first offender's source
 // line, index and extent), and the access is skipped -- a load gives 0 --
 // instead of faulting (teno_debug_bounds reads the record).  In the
