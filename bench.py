@@ -116,38 +116,39 @@ def _acc(tot, add=0.0, mul=0.0, fma=0.0, div=0.0, sqrt=0.0, w=1.0):
 
 
 def face_fp64_instructions(nd, H, hist, exact_frac, tf=32):
-    """FP64 instructions the face-sweep kernel executes per face, by kind,
-    following its code: staged cells formed from the stored primitives
-    (flux, halving, speeds), Roe average and eigenvector rows, projection of
-    the halved staged values, one fma per split value, the 2H - 1 shifted
-    values the decision filter reads, each reconstruction's value formula
-    for its decided outcome (hist: fractions of fallback, S3 .. S_H) or the
-    whole method on the exact path (exact_frac), and the back-projection.
-    The filter's own single-precision and integer work is not FP64."""
+    """FP64 instructions the face-flux kernels execute per face, by kind,
+    following their code: staged cells formed from the stored primitives
+    (flux, speeds; halves on the exponent bits), Roe average and eigenvector
+    rows, projection of the halved staged values, one fma per split value,
+    each reconstruction's value formula for its decided outcome (hist:
+    fractions of fallback, S3 .. S_H) or the whole method on the exact path
+    (exact_frac), and the back-projection.  The filter's work is
+    single-precision and integer."""
     nc, W = nd + 2, 2 * H
     nrec = 2 * nc
     t = {"dadd": 0.0, "dmul": 0.0, "dfma": 0.0}
     staged = (tf + W - 1) / tf
-    _acc(t, add=5, mul=nd + 1 + 2 * nc, w=staged)                       # staged cells
+    _acc(t, add=5, mul=nd + 1, w=staged)                                # staged cells
     _acc(t, add=2, mul=2 * nd + 12, fma=2 * nd, div=2, sqrt=1)         # Roe state
-    _acc(t, add=5, mul=5 * nd + 2)                                     # eigenvector rows
+    _acc(t, add=5, mul=3 * nd - 2)                                     # eigenvector rows
     _acc(t, mul=3 * W * 2, fma=3 * W * 2 * (nc - 1))                   # acoustic, entropy
     _acc(t, add=(nd - 1) * W * 2, mul=(nd - 1) * W * 2)                # shear fields
     _acc(t, fma=nc * 2 * W)                                            # split values
-    _acc(t, add=nrec * (W - 1))                                        # shifted values
     for sel in range(5):                                               # decided values
         f = hist[sel] * nrec * (1.0 - exact_frac)
         if sel == 0:
-            _acc(t, add=6, mul=8, fma=2, div=3, w=f)
+            _acc(t, add=3, mul=8, fma=11, w=f)
+        elif sel == H - 2:
+            _acc(t, mul=1, fma=W - 1, w=f)
         else:
-            _acc(t, mul=1, fma=2 * (sel + 2) - 1, w=f)
-    _acc(t, add=nc + nd + 3, mul=nc + 1, fma=(nd - 1) + 2 * nc)        # back-projection
+            _acc(t, fma=W, w=f)
+    _acc(t, add=nc + nd, mul=nc - 1, fma=(nd - 1) + 2 * nc)            # back-projection
     exact = exact_frac * nrec * sum(hist[s] * recon_flops(H, s) for s in range(5))
     return t, exact
 
 
 def executed_fp64_per_face(hist, exact_frac, nd, H):
-    """FP64 flops the face kernel executes per face (add/mul 1, fma 2),
+    """FP64 flops the face-flux kernels execute per face (add/mul 1, fma 2),
     from face_fp64_instructions."""
     t, exact = face_fp64_instructions(nd, H, hist, exact_frac)
     return t["dadd"] + t["dmul"] + 2.0 * t["dfma"] + exact
@@ -155,14 +156,14 @@ def executed_fp64_per_face(hist, exact_frac, nd, H):
 
 def executed_fp64_instr_per_face(hist, exact_frac, nd, H):
     """FP64 instructions (thread level: DADD, DMUL, DFMA, each one slot of
-    the FP64 pipe) the face kernel executes per face; the rare exact-path
+    the FP64 pipe) the face-flux kernels execute per face; the rare exact-path
     reconstructions counted as if all their flops were fmas (a lower bound)."""
     t, exact = face_fp64_instructions(nd, H, hist, exact_frac)
     return t["dadd"] + t["dmul"] + t["dfma"] + 0.5 * exact
 
 
 def fp64_roofline(hist, exact_frac, nd, H, faces_per_launch, avg_launch_s, method_fpf):
-    """The face kernel against the FP64 pipe: executed FP64 instructions per
+    """The face-flux kernels against the FP64 pipe: executed FP64 instructions per
     second over the pipe's 2 lanes per SM per clock (the binding resource),
     with the same work in flops against the DFMA peak, and the plain
     method's op count over the same time."""
@@ -174,13 +175,13 @@ def fp64_roofline(hist, exact_frac, nd, H, faces_per_launch, avg_launch_s, metho
     ach_f = fpf * faces_per_launch / avg_launch_s / 1e12
     ach_m = method_fpf * faces_per_launch / avg_launch_s / 1e12
     return {
-        "bound": "alu", "kernel": "face_kernel (x/y/z face sweeps)",
+        "bound": "alu", "kernel": "sweep, decide, exact and finish kernels (all directions)",
         "achieved": ach_i, "peak": peak_i, "unit": "G FP64 instr/s", "frac": ach_i / peak_i,
         "peak_source": "derived: 152 SM x 2 FP64 lanes/clk x 2.07 GHz (DADD, DMUL and DFMA "
                        "each take one lane slot)",
-        "counted": "FP64 instructions executed per face, counted from the kernel's code with "
+        "counted": "FP64 instructions executed per face, counted from the kernels' code with "
                    "the live decision mix and exact-path fraction (div/sqrt expansions measured "
-                   "with ncu); ncu counts about 3 % more (sign and absolute-value operations)",
+                   "with ncu)",
         "fp64_instr_per_face": ipf,
         "flops": {"achieved": ach_f, "peak": peak_f, "unit": "TFLOP/s", "frac": ach_f / peak_f,
                   "fp64_flops_per_face": fpf,
@@ -462,7 +463,7 @@ def run_batched(args, dev, stream):
         H = scheme // 2
         hist = [0.0] * 5
         hist[H - 2] = 1.0
-        ti, _ = face_fp64_instructions(1, H, hist, 0.0, tf=tile)
+        ti, _ = face_fp64_instructions(1, H, hist, 0.0)
         nf = 3 * sum(c["n"][0] + 1 for c in cases if c["scheme"] == scheme)
         flops += nf * (ti["dadd"] + ti["dmul"] + 2.0 * ti["dfma"])
         instr += nf * (ti["dadd"] + ti["dmul"] + ti["dfma"])
@@ -480,14 +481,14 @@ def run_batched(args, dev, stream):
             "autotuned": {"tile_faces": tile, "warps_per_tile": tile // 32,
                           "blocks_per_sm": bps},
             "clocks": clk,
-            "roofline": {"bound": "alu", "kernel": "batch_face_kernel (3 per step) + small "
-                                                  "kernels, one CUDA graph",
+            "roofline": {"bound": "alu", "kernel": "a step's sweep, decide, exact, finish and "
+                                                  "combine kernels, one CUDA graph",
                          "achieved": achieved_i, "peak": peak_i, "unit": "G FP64 instr/s",
                          "frac": achieved_i / peak_i,
                          "flops": {"achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                                    "frac": achieved / peak},
-                         "counted": "FP64 instructions the three persistent face sweeps of a "
-                                    "step execute (largest-stencil value for every "
+                         "counted": "FP64 instructions the face fluxes of a step's three stages "
+                                    "execute (largest-stencil value for every "
                                     "reconstruction, primitives read from the stored rows), over "
                                     "the whole step's time: a lower bound"},
             "mode": "persistent (problem, tile) work list, step captured in a CUDA graph"}
@@ -953,7 +954,9 @@ def run_ours(args, rank, world, local_rank):
                  "avg_launch_ms": avg_launch_s * 1e3,
                  "face_kernel_share": face_ms / ms if ms > 0 else None,
                  "selection_mix": selection_mix(hist, scheme), "ct_exponent_mix": ct_hist})
-    launches_per_step = 3 + 3 * (2 + 3)       # CFL (2), primitives; per stage prepare, 3 sweeps, combine
+    # CFL (2), primitives; per stage prepare and combine, and the four face-flux
+    # kernels of every profiled group (sweep, decide, exact, finish)
+    launches_per_step = 3 + 3 * 2 + 4 * face_launches // args.steps
     hbm_peak, hbm_src = measured_hbm_peak()
     batched = None
     if not args.no_batched:
