@@ -180,7 +180,10 @@ inline void tile_shape(DirArgs &d, int64_t faces, int64_t pencils, int H)
 // against one: 1D 400 cells 58 against 34 us, 100 000 cells (3126 tiles) 163
 // against 154; 2D ten-point 128^2 (1088 tiles) 123 against 110, 256^2 (4200) 314
 // against 316; 2D twelve-point 96^2 (620) 124 against 107, 160^2 (1640) 151
-// against 183; 3D 20^3 (900) 131 against 138, 28^3 216 against 289.
+// against 183; 3D 20^3 (900) 131 against 138, 28^3 216 against 289.  Above the
+// line in 1D, three ten-point steps of a tube whose plateaus carry rounding
+// noise: 140 000 cells (4376 tiles) 2.13 against 2.15 ms, 200 000 2.75 against
+// 3.02, 300 000 3.74 against 4.45, 500 000 5.72 against 7.32.
 inline bool small_evaluation(int64_t tiles, int nd, int H)
 {
     return tiles <= (nd == 1 ? 4096 : (nd == 2 ? (H == 6 ? 1024 : 3072) : 512));
