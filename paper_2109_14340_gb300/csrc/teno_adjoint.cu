@@ -813,16 +813,11 @@ cudaError_t launch_adj_direction(AdjArgs &a, double *mu, cudaStream_t s)
 {
     constexpr size_t smem = sizeof(double) * (size_t)FaceSmem<ND, H>::TOTAL * kAdjWarps;
     constexpr size_t mixed = sizeof(double2) * (size_t)(ND + 2) * 2 * H * kMixedThreads;
-    static bool attr_done = false;
+    constexpr size_t table = sizeof(double) * 32 * 2 * H;                // coef_table
     cudaError_t e;
-    if (!attr_done) {
-        if ((e = cudaFuncSetAttribute(adj_face_kernel<ND, H, D>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(adj_mixed_kernel<ND, H, D>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mixed)) != cudaSuccess)
-            return e;
-        attr_done = true;
-    }
+    if ((e = allow_shared(adj_face_kernel<ND, H, D>, smem, table)) != cudaSuccess ||
+        (e = allow_shared(adj_mixed_kernel<ND, H, D>, mixed, table)) != cudaSuccess)
+        return e;
     const int64_t fast = D == 0 ? a.g.n[1] : a.g.n[0];
     tile_shape(a.d, a.g.n[D] + 1, fast, H);
     a.tiles = a.d.line_tiles * a.d.groups * (a.g.ncell / a.g.n[D] / fast);

@@ -40,6 +40,17 @@ inline cudaError_t launch_chained(bool on, void (*kernel)(P...), dim3 grid, dim3
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// A launch with more than 48 KB of shared memory (dynamic and the kernel's own)
+// has to ask for it.  The permission belongs to the device that is current
+// (another GPU of the process starts without it), so it is not remembered: each
+// such launch asks, beside kernels of 20 us and more.
+template <class... P>
+inline cudaError_t allow_shared(void (*kernel)(P...), size_t dynamic, size_t own)
+{
+    if (dynamic + own <= (size_t)48 << 10) return cudaSuccess;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic);
+}
+
 // Workspace header (first 256 bytes of every workspace).
 struct Status {
     unsigned long long nonphys;    // non-physical cells + faces (teno_status)

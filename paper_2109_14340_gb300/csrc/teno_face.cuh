@@ -1247,6 +1247,7 @@ struct SmallSmem {
     static constexpr int PRJ = SPD + 4 * 32;           // [2 nc][W][32] halved w and g
     static constexpr int VAL = PRJ + NW * W * 32;      // [2 nc][32] values
     static constexpr int BYTES = 8 * (VAL + NW * 32);
+    static constexpr int ARG = 4 * 32 * 2;             // maximising cells, small_tile's own array
     // the limiter's rows [4 nc + 1][32] take the projections' room once those were read
     static_assert(4 * nc + 1 <= NW * W, "limiter rows fit in the projections' room");
 };
@@ -1358,7 +1359,7 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
     using SS = SmallSmem<ND, H>;
     constexpr int nc = ND + 2, last = nc - 1, W = 2 * H, NS = SL::NS, NT = 32 * SS::NW;
     const bool fused = ND == 1 && fuse.mode >= 0;
-    __shared__ uint16_t arg[4 * 32];
+    __shared__ uint16_t arg[SS::ARG / 2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = warp >> 1, s = warp & 1;
     const int tps = ND == 1 ? 0 : da.tps;
     int p, fo, b0, bs;
@@ -1575,23 +1576,12 @@ template <int ND, int H, int MODE>
 cudaError_t launch_chunk_mode(const SweepArgs &a, cudaStream_t s)
 {
     constexpr size_t smem = sizeof(double) * (size_t)FaceSmem<ND, H>::TOTAL * kSweepWarps;
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(sweep_kernel<ND, H, MODE>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static_assert(smem <= (size_t)48 << 10, "launched without allow_shared");
     if constexpr (MODE != kSweepFrozen) {
         if (a.small) {
             constexpr size_t bytes = SmallSmem<ND, H>::BYTES;
-            static bool small_done = false;
-            if (!small_done) {
-                cudaError_t e = cudaFuncSetAttribute(small_kernel<ND, H, MODE>,
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-                if (e != cudaSuccess) return e;
-                small_done = true;
-            }
+            const cudaError_t e = allow_shared(small_kernel<ND, H, MODE>, bytes, SmallSmem<ND, H>::ARG);
+            if (e != cudaSuccess) return e;
             return launch_chained(a.tiles <= kChainTiles, small_kernel<ND, H, MODE>, (unsigned)a.tiles,
                                   64 * (ND + 2), bytes, s, a);
         }
