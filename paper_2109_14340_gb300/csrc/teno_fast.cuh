@@ -345,7 +345,8 @@ __device__ __forceinline__ constexpr float sos_bound(int which)
 // whatever the exponent (chi_p >= C_T holds if sum_k (x_p / x_k)^7 <=
 // 3 (x_p / min_k x_k)^7 <= thr[nexp_min]), or at the smooth exponent where
 // eta >= C_r (m = 0) is certain; only the latter where the exponent is recorded
-// (need_ct).  flag: the decision byte.  Most reconstructions of a resolved flow
+// (need_ct).  flag: the decision byte, its C_T bits zero where S_p is accepted at
+// every exponent.  Most reconstructions of a resolved flow
 // end here, so it uses no FP64 operation at
 // all and few others; whatever it leaves open goes to fast_decide.
 //
@@ -461,7 +462,8 @@ __device__ __forceinline__ bool quick_large(const double (&v)[2 * H], const Fast
         }
         flat = differ == 0u;
     }
-    flag = (uint8_t)(large_code(H) | (need_ct || flat ? ((F.nexp_smooth - 7) & 7) << 5 : 0));
+    // the exponent's bits wherever it decided, recorded for its own sake or not
+    flag = (uint8_t)(large_code(H) | (flat || xp > any * xs ? ((F.nexp_smooth - 7) & 7) << 5 : 0));
     return flat || (range && M >= 9.5367431640625e-7f && xp <= rho * xs);
 }
 
