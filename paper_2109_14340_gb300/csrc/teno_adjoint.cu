@@ -498,12 +498,20 @@ __global__ void __launch_bounds__(32 * kAdjWarps, 4) adj_face_kernel(const AdjAr
                 if (j == 0 || speed_gt(ep, s.ap)) { s.ap = ep; s.jp = j; }
                 if (j == 0 || speed_gt(er, s.ar)) { s.ar = er; s.jr = j; }
             }
-            // c = (|u| + c) - |u|, for the sign of u -+ c only
+            // c = (|u| + c) - |u|, for the sign of u -+ c only; where that lies within
+            // the rounding of |u| + c, the stored c
+            auto sound = [&](int j, double v, double lr, double lambda) {
+                if (lambda > 1.0e-15 * lr) return lr - fabs(v);
+                int rule;
+                const int64_t g = map_index(f - H + j, a.g.n[D], H, a.d.bc_lo, a.d.bc_hi, rule);
+                const int64_t id = (D == 0 ? g : x) + a.g.n[0] * ((D == 1 ? g : y) + a.g.n[1] * (D == 2 ? g : z));
+                return a.g.P[PrimRows<ND>::C * a.g.ncell + id];
+            };
             const int im = b0 + s.jm * bs, ip = b0 + s.jp * bs;
             s.vm = TMP(SL::QV + D, im);
-            s.cm = TMP(SL::QLR, im) - fabs(s.vm);
+            s.cm = sound(s.jm, s.vm, TMP(SL::QLR, im), s.am);
             s.vp = TMP(SL::QV + D, ip);
-            s.cp = TMP(SL::QLR, ip) - fabs(s.vp);
+            s.cp = sound(s.jp, s.vp, TMP(SL::QLR, ip), s.ap);
             s.v0 = TMP(SL::QV + D, b0 + s.j0 * bs);
             s.vr = TMP(SL::QV + D, b0 + s.jr * bs);
             double Fb[nc];
