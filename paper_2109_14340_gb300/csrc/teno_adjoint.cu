@@ -990,6 +990,7 @@ int rhs_vjp_impl(const teno_params *p, const double *U, const double *lam, const
         memset(&a, 0, sizeof(a));
         a.g.U = U;
         a.g.P = P;
+        a.g.st = (Status *)(ws + L.fwd);       // the checked build's range checks
         for (int k = 0; k < 3; k++) a.g.n[k] = p->n[k];
         a.g.ncell = cells_of(p);
         a.d.nfaces = faces_of(p, d);

@@ -474,7 +474,8 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
     int p, fo;
     tile_lane<D>(tps, lane, p, fo);
     const int64_t f = f0 + fo;
-    const bool active = f <= nD - da.skip_last && p < npen;
+    const int64_t nf = B.nt * kTileFaces, cf = tile * kTileFaces + lane;   // in the buffers
+    const bool active = f <= nD - da.skip_last && p < npen && TENO_IN(a.st, cf, nf);
     // the lane's first cell, the step to the next, and cells i and i+1
     const int b0 = D == 0 ? p * nsf + fo : lane, bs = D == 0 ? 1 : tp;
     const int bl = b0 + (H - 1) * bs, br = bl + bs;
@@ -482,7 +483,6 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
     RoeScalars<ND> rs;                 // eigenvector rows / columns are built from these
     double am = 0.0, a0 = 0.0, ap = 0.0, ar = 0.0;
     int64_t flin = 0;
-    const int64_t nf = B.nt * kTileFaces, cf = tile * kTileFaces + lane;   // in the buffers
     if (active) {
         // Roe average and eigenvectors (Sec. 5).
         double ul[ND], ur[ND];
@@ -607,7 +607,7 @@ __device__ __forceinline__ void sweep_tile(const GridArgs &a, const DirArgs &da,
             for (int kk = 0; kk < W; kk++) v[kk] = vm[kk];
         }
     }
-    if (MODE != kSweepFrozen && lane == 0) B.count[tile] = (uint32_t)cnt | a.tag;
+    if (MODE != kSweepFrozen && lane == 0 && TENO_IN(a.st, tile, B.nt)) B.count[tile] = (uint32_t)cnt | a.tag;
     __syncwarp();
 #undef TMP
 }
@@ -715,7 +715,7 @@ __device__ __forceinline__ void finish_face(const DirArgs &da, int limiter, cons
 {
     constexpr int nc = ND + 2;
     const int64_t nf = B.nt * kTileFaces;
-    if (!TENO_IN(st, flin, da.nfaces)) return;
+    if (!TENO_IN(st, flin, da.nfaces) || !TENO_IN(st, cf, nf)) return;
     double Fo[nc];
     face_flux<ND, D, MODE>(da, limiter, limiter ? *da.lam : 0.0, K, B, cf, flin, Fo);
     if constexpr (MODE == kSweepRecord && BYTES) {

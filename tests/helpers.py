@@ -43,3 +43,28 @@ def advance_oracle(p, U, t_end, cfl=0.4, threads=1, stage_hook=None, max_steps=1
         t += dt
         steps += 1
     return U, steps
+
+
+def tiles_of(case):
+    """Tiles of 32 faces an evaluation of the case's grid has at most, over all
+    directions (the launch rules count them): a tile is 2^k pencils side by side
+    of 32 / 2^k faces each, k the cheapest of 0, 1, 2 in lanes without a face and
+    cells staged; the last face of a periodic axis may be left out."""
+    n, H, total = list(case["n"]) + [1] * (3 - len(case["n"])), case["scheme"] // 2, 0
+    for d in range(case["ndim"]):
+        pencils = n[1] if d == 0 else n[0]
+        rest = n[0] * n[1] * n[2] // n[d] // pencils
+        most = 0
+        for skip in (0, 1):
+            best = None
+            for k in range(3):
+                tp, tf = 1 << k, 32 >> k
+                tiles = -(-(n[d] + 1 - skip) // tf) * -(-pencils // tp)
+                cost = tiles * (690.0 + 12.0 * -(-tp * (tf + 2 * H - 1) // 32))
+                if best is None or cost < best[0]:
+                    best = (cost, tiles)
+                if pencils == 1:
+                    break
+            most = max(most, best[1] * rest)
+        total += most
+    return total
