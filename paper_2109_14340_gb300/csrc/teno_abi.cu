@@ -601,7 +601,6 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
         D.skip_last = (p->bc_lo[d] == TENO_BC_PERIODIC && !fl && !fz) ? 1 : 0;
         tiles[d] = shape_tiles(p, d, D.skip_last, D);
         if (fused) {                  // every face, tiles overlapping by one
-            D.skip_last = 0;
             D.own = kTileFaces - 1;
             tiles[d] = D.line_tiles = (p->n[d] + D.own - 1) / D.own;
         }

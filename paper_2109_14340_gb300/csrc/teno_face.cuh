@@ -58,7 +58,8 @@ struct DirArgs {
     int64_t nfaces;
     int bc_lo, bc_hi;      // boundary rules at the two ends of the axis
     int skip_last;         // 1: face n of each line is not computed (periodic axis, no
-                           // decision record: its flux is face 0's, bitwise)
+                           // decision record: its flux is face 0's, bitwise); the fused 1D
+                           // stage computes it, but counts nothing there
     // A tile is 2^tps pencils (side by side in x, in y for the x sweep) by 32 >> tps
     // faces; tiles per line of faces, and groups of 2^tps pencils along that axis.
     int tps;
@@ -1378,9 +1379,12 @@ __device__ __forceinline__ void small_tile(const GridArgs &a, const DirArgs &da,
         npen = a.n[0] - x;
         flin = d == 1 ? face_index<1>(a.n, f0 + fo, x + p, y, z) : face_index<2>(a.n, f0 + fo, x + p, y, z);
     }
-    const bool active = f0 + fo <= (d == 0 ? a.n[0] : (d == 1 ? a.n[1] : a.n[2])) - da.skip_last && p < npen;
+    const int64_t last_face = (d == 0 ? a.n[0] : (d == 1 ? a.n[1] : a.n[2])) - da.skip_last;
+    // the fused update of the last cell takes face n also where skip_last leaves it out
+    const bool active = f0 + fo <= (fused ? a.n[0] : last_face) && p < npen;
     if (active && !TENO_IN(a.st, flin, da.nfaces)) flin = 0;     // debug build: counted, redirected
-    const bool own = fo < da.own || f0 + fo == a.n[0];           // (all, unless tiles overlap)
+    // counted here: all, unless tiles overlap or face n is the periodic image of face 0
+    const bool own = f0 + fo <= last_face && (fo < da.own || f0 + fo == a.n[0]);
     // the fused update's inputs, on their way while the fluxes are computed
     double Uk[nc], Un[nc], dt = 0.0;
     const int64_t ic = f0 + lane;                                 // the lane's cell
