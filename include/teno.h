@@ -131,7 +131,8 @@ void teno_params_init(teno_params *p);
 /* Workspace bytes needed by every call below for these parameters: status
  * header, face fluxes, one stage state, the primitive rows, and the buffers of
  * the face sweeps' queue (0.5 to 1.4 KB per face, up to 2.1 million faces at a
- * time: 1.1 to 2.8 GB for every larger grid).
+ * time: 1.1 to 2.8 GB for every larger grid; grids of few tiles, which take one
+ * launch, have no queue: 0.1 to 0.3 KB per face).
  * Returns TENO_EINVAL for invalid parameters (then *bytes is untouched). */
 int teno_workspace_bytes(const teno_params *p, size_t *bytes);
 

@@ -306,6 +306,7 @@ struct SweepMem {
     char *mem;
     unsigned *counters;
     int64_t nt, nchunks;
+    bool queue;
     size_t bytes;
 };
 
@@ -319,7 +320,8 @@ static SweepMem sweep_mem(const teno_params *p, char *mem, int64_t most)
     const size_t c = sweep_align(sizeof(unsigned) * (size_t)m.nchunks);
     m.counters = (unsigned *)mem;
     m.mem = mem + c;
-    m.bytes = c + sweep_buf_layout(b, m.mem, m.nt, p->ndim, p->scheme, p->limiter != 0);
+    m.queue = !small_evaluation(all, p->ndim, p->scheme / 2);
+    m.bytes = c + sweep_buf_layout(b, m.mem, m.nt, p->ndim, p->scheme, p->limiter != 0, m.queue);
     return m;
 }
 
@@ -582,7 +584,7 @@ static int stage(const teno_params *p, const double *Uk, const double *Un, doubl
     a.exact_count = g_prof.on ? g_prof.exact : nullptr;
     a.FK = fastk_of(p);
     a.K = K;
-    sweep_buf_layout(a.buf, M.mem, M.nt, nd, p->scheme, p->limiter != 0);
+    sweep_buf_layout(a.buf, M.mem, M.nt, nd, p->scheme, p->limiter != 0, M.queue);
     int64_t tiles[3] = {0, 0, 0};
     for (int d = 0; d < nd; d++) {
         DirArgs &D = a.dir[d];

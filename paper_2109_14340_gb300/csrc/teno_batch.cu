@@ -393,7 +393,7 @@ int enqueue_step(teno_batch *b, double *U, double cfl, char *ws, int tile_idx, i
     double *Us = (double *)(ws + b->off_Us);
     double *P = (double *)(ws + b->off_P);
     SweepBuf B;
-    sweep_buf_layout(B, ws + b->off_sweep, b->chunk_tiles, 1, 10, b->has_limiter);
+    if (!b->small()) sweep_buf_layout(B, ws + b->off_sweep, b->chunk_tiles, 1, 10, b->has_limiter, true);
     uint32_t *xlist10 = (uint32_t *)(ws + b->off_xlist10);
     const int ncitems = b->cprefix[np];
     const int grid_c = std::max(1, std::min(ncitems, b->num_sms * 8));
@@ -571,9 +571,12 @@ int teno_batch_create(const teno_params *common, const teno_batch_problem *probs
     off += a256(sizeof(double) * b->p_len);
     SweepBuf B;
     b->off_sweep = off;
-    off += sweep_buf_layout(B, nullptr, b->chunk_tiles, 1, 10, b->has_limiter);
     b->off_xlist10 = off;
-    off += a256(sizeof(uint32_t) * 64 * 3 * (size_t)b->chunk_tiles);
+    if (!b->small()) {                           // the fused stages use neither
+        off += sweep_buf_layout(B, nullptr, b->chunk_tiles, 1, 10, b->has_limiter, true);
+        b->off_xlist10 = off;
+        off += a256(sizeof(uint32_t) * 64 * 3 * (size_t)b->chunk_tiles);
+    }
     b->off_single = off;
     off += a256(single);
     b->total = off;

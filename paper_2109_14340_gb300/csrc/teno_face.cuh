@@ -102,21 +102,24 @@ struct SweepBuf {
 inline size_t sweep_align(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Lays the buffers for nt tiles out from p (null: only measures); W values per
-// entry.  Returns the bytes used.
-inline size_t sweep_buf_layout(SweepBuf &b, char *p, int64_t nt, int nd, int W, bool limiter)
+// entry.  queue = false: only what a frozen replay passes on (R, RO, RL), for grids
+// whose other evaluations take the single launch (2D 128^2 ten-point: 4 MB in place
+// of 28).  Returns the bytes used.
+inline size_t sweep_buf_layout(SweepBuf &b, char *p, int64_t nt, int nd, int W, bool limiter,
+                               bool queue)
 {
     const int nc = nd + 2;
-    const size_t q = (size_t)nt * 64 * nc, f = (size_t)nt * kTileFaces;
+    const size_t q = queue ? (size_t)nt * 64 * nc : 0, f = (size_t)nt * kTileFaces;
     size_t off = 0;
     auto take = [&](size_t bytes) { char *r = p + off; off += sweep_align(bytes); return r; };
     b.nt = nt;
     b.qv = (double *)take(sizeof(double) * W * q);
     b.xlist = (uint32_t *)take(sizeof(uint32_t) * q);
     b.qslot = (uint16_t *)take(sizeof(uint16_t) * q);
-    b.count = (uint32_t *)take(sizeof(uint32_t) * nt);
+    b.count = (uint32_t *)take(queue ? sizeof(uint32_t) * nt : 0);
     b.R = (double *)take(sizeof(double) * 2 * nc * f);
     b.RO = (double *)take(sizeof(double) * (nd + 4) * f);
-    b.RD = (uint8_t *)take(2 * nc * f);
+    b.RD = (uint8_t *)take(queue ? 2 * nc * f : 0);
     b.RL = limiter ? (double *)take(sizeof(double) * (4 * nc + 1) * f) : nullptr;
     return off;
 }
