@@ -1,6 +1,10 @@
 // C ABI of the TENO-AA library (declared in include/teno.h): parameter
-// validation, workspace layout, and the per-stage launch sequence
-//   [wave maxima] -> prepare -> face sweep x [-> y [-> z]] -> combine.
+// validation, workspace layout, and a stage's launches, all directions' tiles in
+// one list:
+//   many tiles   [wave maxima] -> prepare -> (sweep -> decide -> exact -> finish)
+//                per chunk of tiles -> combine
+//   few tiles    [wave maxima -> prepare] -> small_kernel -> combine
+//   few, in 1D   small_kernel alone, where it may write another array than it reads
 #include <cmath>
 #include <cstdio>
 #include <cstddef>
@@ -440,8 +444,6 @@ static int grid_for(int64_t n, int block)
     do {                                              \
         if ((x) != cudaSuccess) return TENO_ECUDA;    \
     } while (0)
-
-static double3 inv_dx_of(const teno_params *p);
 
 static bool chained(const teno_params *p) { return all_tiles(p) <= kChainTiles; }
 

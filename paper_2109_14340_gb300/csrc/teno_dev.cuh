@@ -109,7 +109,6 @@ static __constant__ double TENO_LIN5[10] = {
     -0.221228429084247, 0.6657332621611695, 0.6557332621611695,
     -0.2145617624175796, 0.07053731329146805, -0.01631901203296621,
     0.001832421220128962};
-// Optimal weights of the small stencils S0, S1, S2 (Sec. 4.1).
 // C_T = 10^-[beta] (Eq. CT_definition), [beta] clamped to 0..22.
 static __constant__ double TENO_TENPOW[23] = {
     1e0, 1e-1, 1e-2, 1e-3, 1e-4, 1e-5, 1e-6, 1e-7, 1e-8, 1e-9, 1e-10, 1e-11,

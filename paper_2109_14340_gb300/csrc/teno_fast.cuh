@@ -12,11 +12,13 @@
 // so every decision equals the FP64 evaluation of the same formulas, and the
 // value is then computed in FP64 with the exact path's own arithmetic.
 //
-// FP64 part kept: the shifted values s_m = v_m - v_0, computed with exactly
-// the operations of the exact path.  FP32 parts: the three small indicators,
-// the large-stencil indicators, the scale separation and normalisation (all
-// the divisions), and the first-order undivided-difference measure eta -> m
-// -> g -> [beta].  The printed quadratic forms of the large indicators
+// The shifted values s_m = v_m - v_0 come from the bit patterns, as pairs of
+// FP32 numbers (24 and 23 bits of each value) or, on plateaus with rounding noise,
+// as integers (quick_large, front_bits); what fits neither form takes FP64
+// subtractions (front_fp64).  FP32 parts: the three small indicators, the
+// large-stencil indicators, the scale separation and normalisation (all the
+// divisions), and the first-order undivided-difference measure eta -> m -> g ->
+// [beta].  The printed quadratic forms of the large indicators
 // cancel about six orders of magnitude on smooth data, so FP32 evaluates
 // instead their exact rational L D L^T factorisations, beta = sum_i D_i y_i^2
 // (sums of non-negative terms); the bound on the error includes the rounding
